@@ -6,8 +6,9 @@ widths, every storage type, and the three ways of issuing a call (directly, prep
 CUDA graph).  Shapes come from ``paper_2509_07506_b200.workloads``, the test suite and ``bench.py``.
 
 ``listed()`` gives the named cases, ``draw(rng)`` another one of the same ranges; ``prepare`` builds the
-tensors a caller has in hand, ``run`` issues the calls, ``work`` states the unavoidable bytes and
-operations, ``tolerance`` how far another correct implementation may be off.
+tensors a caller has in hand, ``run`` issues the calls, ``exact`` gives their results in 64 bits, ``work``
+states the unavoidable bytes and operations, ``tolerance`` how far another correct implementation may
+be off.
 """
 from __future__ import annotations
 
@@ -246,6 +247,58 @@ def run(st):
     if op == "chain":
         return [st["x"], st["r"], st["out"], st["vo"], st["so"]]
     return [st["xs"], st["r"], st["out"], st["vo"], st["so"]]
+
+
+# ---- the same pass in 64 bits -----------------------------------------------------------------------
+
+def _exact_norm(x, r, w):
+    """(normalised rows, unrounded residual) of the add and RMSNorm; all arithmetic in 64 bits."""
+    s = x.double() + r.double()
+    return s * torch.rsqrt((s * s).mean(dim=1, keepdim=True) + EPS) * w.double(), s
+
+
+def _exact_silu(inp):
+    a, b = inp.double().chunk(2, dim=1)
+    return a * torch.sigmoid(a) * b
+
+
+def _exact_merge(va, sa, vb, sb):
+    sa, sb = sa.double(), sb.double()
+    m = torch.maximum(sa, sb)
+    m = m.masked_fill(m == float("-inf"), 0.0)
+    ea, eb = torch.exp(sa - m), torch.exp(sb - m)
+    total = ea + eb
+    share = torch.where(total > 0, 1.0 / total, total)   # two empty states merge to an empty one
+    v = (ea * share).unsqueeze(2) * va.double() + (eb * share).unsqueeze(2) * vb.double()
+    return v, m + torch.log(total)
+
+
+def exact(case, seed):
+    """What ``run`` returns for these inputs, in 64 bits.  The residual stream of the graph case is kept in
+    its storage type between the layers, as the caller's buffer keeps it."""
+    st = prepare(case, seed)
+    op = case["op"]
+    if op == "rmsnorm":
+        return list(_exact_norm(st["x"], st["r"], st["w"]))
+    if op == "silu":
+        return [_exact_silu(st["inp"])]
+    if op == "merge":
+        return list(_exact_merge(st["va"], st["sa"], st["vb"], st["sb"]))
+    if op == "allreduce":
+        total = st["parts"][0].double()
+        for p in st["parts"][1:]:
+            total = total + p.double()
+        y, r = _exact_norm(total, st["r"], st["w"])
+        return [[y] * len(st["ys"]), [r] * len(st["rs"])]
+    silu, (vo, so) = _exact_silu(st["inp"]), _exact_merge(st["va"], st["sa"], st["vb"], st["sb"])
+    if op == "chain":
+        return [*_exact_norm(st["x"], st["r"], st["w"]), silu, vo, so]
+    ys, r = [], st["r"]
+    for x, w in zip(st["xs"], st["ws"]):
+        y, s = _exact_norm(x, r, w)
+        ys.append(y)
+        r = s.to(st["r"].dtype)
+    return [torch.stack(ys), s, silu, vo, so]
 
 
 # ---- what a pass cannot do without ------------------------------------------------------------------
