@@ -112,4 +112,101 @@ silu_and_mul_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gat
     }
 }
 
+// SiLU(a) * b on whole packs.
+template <int DT, int UV> __device__ __forceinline__ Pack<UV> silu_mul_pack(const Pack<UV> &a, const Pack<UV> &b) {
+    constexpr int VEC = UV / Storage<DT>::UNITS;
+    float fa[VEC], fb[VEC], fo[VEC];
+    widen<DT, VEC>(a, fa);
+    widen<DT, VEC>(b, fb);
+#pragma unroll
+    for (int i = 0; i < VEC; i += 2) {
+        const float2 o = silu_mul2(make_float2(fa[i], fa[i + 1]), make_float2(fb[i], fb[i + 1]));
+        fo[i] = o.x;
+        fo[i + 1] = o.y;
+    }
+    return narrow<DT, VEC>(fo);
+}
+
+// Rows that start at any element: the widths and pitches whose common divisor leaves less than a 16-byte
+// access (odd widths above all, where the flat kernel moves one element per load).
+//
+// The output row is cut into 16-byte granules that are aligned in the OUTPUT; a thread owns one.  Its 8
+// units of gate (and of up) straddle two aligned granules of that input, at an offset that is the same
+// for the whole row: both are loaded with 16-byte accesses (the second one is the neighbour thread's first,
+// an L1 hit) and the 8 units are taken out of them with ASTRA_FOR_SHIFT, uniformly for the block, which
+// covers one piece of one row.
+//
+// What bounds it: HBM, then issue slots (about 165 warp instructions per 32 granules against 113 of the
+// aligned kernel; 73 % of the slots at [8192, 4099]).  Measured L2-cold, fp16, against the narrow flat
+// kernels: 28.5 -> 14.1 us at [1000, 14337] (12.5 us at 6.9 TB/s), 64.0 -> 33.7 us at [8192, 4099], 39.9 -> 33.7 us at
+// [8192, 4098], 5.69 -> 4.5 us at [300, 11010]; fp32 16.0 -> 13.1 us at [1000, 7001].  Also tried: flat
+// indexing over all rows' granules (15.3 and 33.8 us: the shifts are then per thread and need selects),
+// the neighbour's granule by shuffles (18.6 and 43.9 us), two granules per thread (16.5 us), 32-byte
+// granules (16.0 and 37.7 us), blocks of 256 and 448 threads instead of about 192 (14.7 and 15.9 us).
+//
+// Accesses stay inside the tensors: a granule of a row other than the launch's first and last may reach
+// up to 14 units into the row before it or 15 into the one after, which exist (the launch code asks for
+// rows of at least 16 units, and that the output shares no address range with the inputs, so that
+// nothing that is written is read); the first and last row load the few granules that would pass their
+// ends element by element, and so are the ends of every output row stored.
+constexpr int kSiluRaggedMaxThreads = 256;
+struct RaggedGranule {
+    int at;                // first unit of the output granule, in the row (negative before its start)
+    int shift_a, shift_b;  // of its units in the aligned granules of gate and up
+    bool whole;            // the aligned granules lie inside the tensors
+};
+__host__ __device__ __forceinline__ RaggedGranule ragged_granule(const uint16_t *out_row, const uint16_t *gate_row,
+                                                                 const uint16_t *up_row, int granule, int D, bool end_row) {
+    constexpr int UV = 8;
+    const int lead = misalignment<UV>(out_row);
+    RaggedGranule g;
+    g.at = granule * UV - lead;
+    g.shift_a = (misalignment<UV>(gate_row) - lead) & (UV - 1);
+    g.shift_b = (misalignment<UV>(up_row) - lead) & (UV - 1);
+    g.whole = !(end_row && (g.at < UV || g.at + 2 * UV > D));
+    return g;
+}
+
+template <int DT, int ALIGN>
+__global__ void __launch_bounds__(kSiluRaggedMaxThreads, 8)
+silu_and_mul_ragged_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gate,
+                           const uint16_t *__restrict__ up, FastDiv pieces, uint32_t last_row, int D,
+                           int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch) {
+    constexpr int UV = 8, UNITS = Storage<DT>::UNITS;
+    const uint32_t row = pieces.div(blockIdx.x);
+    const int first = static_cast<int>((blockIdx.x - row * pieces.d) * blockDim.x) * UV;
+    const uint16_t *a = gate + static_cast<int64_t>(row) * gate_pitch;
+    const uint16_t *b = up + static_cast<int64_t>(row) * up_pitch;
+    uint16_t *o = out + static_cast<int64_t>(row) * out_pitch;
+    if (threadIdx.x == 0) {
+        const int64_t n = min(static_cast<int>(blockDim.x) * UV, D - first);
+        if (n > 0) {
+            prefetch_l2_range(a + first, n * 2);
+            prefetch_l2_range(b + first, n * 2);
+        }
+    }
+    const RaggedGranule g = ragged_granule(o, a, b, first / UV + static_cast<int>(threadIdx.x), D,
+                                           row == 0 || row == last_row);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (g.at >= D) return;
+    Pack<UV> va, vb;
+    if (g.whole) {
+        // cached loads: the second granule is some other thread's first
+        const uint16_t *pa = a + (g.at - g.shift_a), *pb = b + (g.at - g.shift_b);
+        const Pack<UV> a0 = load<UV, Ld::Keep>(pa), b0 = load<UV, Ld::Keep>(pb);
+        Pack<UV> a1, b1;
+        if (g.shift_a) a1 = load<UV, Ld::Keep>(pa + UV);
+        if (g.shift_b) b1 = load<UV, Ld::Keep>(pb + UV);
+        ASTRA_FOR_SHIFT(g.shift_a, ALIGN, va = (realign<SHIFT, UV>(a0, a1)))
+        ASTRA_FOR_SHIFT(g.shift_b, ALIGN, vb = (realign<SHIFT, UV>(b0, b1)))
+    } else {
+        va = load_edge<UNITS, UV, Ld::StreamReadOnly>(a, g.at, D);
+        vb = load_edge<UNITS, UV, Ld::StreamReadOnly>(b, g.at, D);
+    }
+    const Pack<UV> v = silu_mul_pack<DT, UV>(va, vb);
+    if (g.at >= 0 && g.at + UV <= D) store<UV, St::Stream>(o + g.at, v);
+    else store_edge<UNITS, UV, St::Stream>(o, g.at, D, v);
+}
+
 }  // namespace astra

@@ -71,11 +71,11 @@ enum class St { Stream, Default };
 
 template <int VEC> struct Pack {
     static_assert(VEC == 2 || VEC == 4 || VEC == 8 || VEC == 16, "unsupported vector width");
-    static constexpr int WORDS = VEC / 2;
+    static constexpr int WORDS = VEC / 2, UNITS_PER_PACK = VEC;
     uint32_t w[WORDS];
 };
 template <> struct Pack<1> {
-    static constexpr int WORDS = 1;
+    static constexpr int WORDS = 1, UNITS_PER_PACK = 1;
     uint32_t w[1];  // low 16 bits hold the element
 };
 
@@ -195,6 +195,85 @@ __device__ __forceinline__ Pack<VEC * Storage<DT>::UNITS> narrow(const float (&f
         for (int i = 0; i < VEC / 2; ++i) v.w[i] = Storage<DT>::narrow2(f[2 * i], f[2 * i + 1]);
     }
     return v;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Rows that start at any element (odd widths, odd pitches): a row is cut into granules of UV units that
+// are aligned to 2*UV bytes, so that all but its first and last one are ordinary vector accesses.
+// ---------------------------------------------------------------------------------------------
+// Units by which p lies beyond the last address that is aligned to UV units.
+template <int UV> __host__ __device__ __forceinline__ int misalignment(const uint16_t *p) {
+    return static_cast<int>((reinterpret_cast<uint64_t>(p) >> 1) & (UV - 1));
+}
+
+// Units [SHIFT, SHIFT + UV) of the 2*UV units lo, hi.  The shift is a constant: an odd one costs one
+// funnel shift per word, an even one nothing.  (Selecting among run-time shifts costs 11 selects more per
+// 16-byte granule; the callers' shift is the same for a whole block, so they branch over its values once.)
+template <int SHIFT, int UV> __device__ __forceinline__ Pack<UV> realign(const Pack<UV> &lo, const Pack<UV> &hi) {
+    constexpr int N = UV / 2;
+    uint32_t w[2 * N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        w[i] = lo.w[i];
+        w[N + i] = hi.w[i];
+    }
+    Pack<UV> v;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        if constexpr (SHIFT % 2 != 0) v.w[i] = __funnelshift_r(w[i + SHIFT / 2], w[i + SHIFT / 2 + 1], 16);
+        else v.w[i] = w[i + SHIFT / 2];
+    }
+    return v;
+}
+
+// Runs CALL with the compile-time constant SHIFT set to `shift` (0 <= shift < UV, UV of 8 or 16 in scope,
+// shift a multiple of STEP).
+#define ASTRA_SHIFT_CASE(K, STEP, CALL)                    \
+    case K:                                               \
+        if constexpr (K < UV && K % (STEP) == 0) {        \
+            constexpr int SHIFT = K;                      \
+            CALL;                                         \
+        }                                                 \
+        break;
+#define ASTRA_FOR_SHIFT(shift, STEP, CALL)                                                                        \
+    switch (shift) {                                                                                              \
+        ASTRA_SHIFT_CASE(0, STEP, CALL) ASTRA_SHIFT_CASE(1, STEP, CALL) ASTRA_SHIFT_CASE(2, STEP, CALL)            \
+        ASTRA_SHIFT_CASE(3, STEP, CALL) ASTRA_SHIFT_CASE(4, STEP, CALL) ASTRA_SHIFT_CASE(5, STEP, CALL)            \
+        ASTRA_SHIFT_CASE(6, STEP, CALL) ASTRA_SHIFT_CASE(7, STEP, CALL) ASTRA_SHIFT_CASE(8, STEP, CALL)            \
+        ASTRA_SHIFT_CASE(9, STEP, CALL) ASTRA_SHIFT_CASE(10, STEP, CALL) ASTRA_SHIFT_CASE(11, STEP, CALL)          \
+        ASTRA_SHIFT_CASE(12, STEP, CALL) ASTRA_SHIFT_CASE(13, STEP, CALL) ASTRA_SHIFT_CASE(14, STEP, CALL)         \
+        ASTRA_SHIFT_CASE(15, STEP, CALL)                                                                          \
+        default: break;                                                                                           \
+    }
+
+// The UV units of a row at offset `at` (in units; the row has `width` of them and starts at `row`), unit
+// by unit and only those that exist; zeros elsewhere.
+template <int UNITS, int UV, Ld HINT>
+__device__ __forceinline__ Pack<UV> load_edge(const uint16_t *row, int at, int width) {
+    Pack<UV> v;
+#pragma unroll
+    for (int i = 0; i < UV / 2; ++i) v.w[i] = 0;
+#pragma unroll
+    for (int k = 0; k < UV; k += UNITS) {
+        if (at + k >= 0 && at + k < width) {
+            const Pack<UNITS> e = load<UNITS, HINT>(row + at + k);
+            if constexpr (UNITS == 2) v.w[k / 2] = e.w[0];
+            else v.w[k / 2] |= (k & 1) ? e.w[0] << 16 : (e.w[0] & 0xffffu);
+        }
+    }
+    return v;
+}
+
+template <int UNITS, int UV, St HINT>
+__device__ __forceinline__ void store_edge(uint16_t *row, int at, int width, const Pack<UV> &v) {
+#pragma unroll
+    for (int k = 0; k < UV; k += UNITS) {
+        if (at + k >= 0 && at + k < width) {
+            Pack<UNITS> e;
+            e.w[0] = UNITS == 2 ? v.w[k / 2] : ((k & 1) ? v.w[k / 2] >> 16 : v.w[k / 2]);
+            store<UNITS, HINT>(row + at + k, e);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -1,0 +1,67 @@
+"""Index arithmetic of the kernels for rows that start at any element, run on the host: the geometry
+functions of the kernel headers are compiled into a small program that walks every alignment of every
+operand, widths around multiples of the vector size, and all threads, and checks that each unit of a row
+belongs to exactly one thread, that every access lies inside its tensor and is aligned to its size."""
+import subprocess
+
+
+from paper_2509_07506_b200 import build as astra_build
+
+PROGRAM = r"""
+#include <cstdio>
+#include <vector>
+#include "silu_and_mul.cuh"
+using namespace astra;
+
+static long failures = 0;
+static void expect(bool ok, const char *what, long a, long b, long c, long d) {
+    if (!ok && failures++ < 5) printf("%s: %ld %ld %ld %ld\n", what, a, b, c, d);
+}
+static const uint16_t *at_unit(long u) { return reinterpret_cast<const uint16_t *>(4096 + 2 * u); }
+
+// All granules of a [rows, D] call with pitched operands; every tensor is [0, span) units from its base.
+template <int UNITS> static void silu_rows(long o0, long a0, long b0, int rows, int D, long po, long pa, long pb) {
+    const long sa = (rows - 1) * pa + D, sb = (rows - 1) * pb + D;
+    for (int r = 0; r < rows; ++r) {
+        std::vector<int> owner(D, 0);
+        const uint16_t *o = at_unit(o0 + r * po), *a = at_unit(a0 + r * pa), *b = at_unit(b0 + r * pb);
+        for (int n = 0; n < (D + 14) / 8; ++n) {
+            const RaggedGranule g = ragged_granule(o, a, b, n, D, r == 0 || r == rows - 1);
+            if (g.at >= D) continue;
+            expect((o0 + r * po + g.at) % 8 == 0, "granule", r, D, g.at, 0);
+            expect(g.shift_a % UNITS == 0 && g.shift_b % UNITS == 0 && g.at % UNITS == 0, "units", r, D, g.at, 0);
+            if (g.whole) {
+                const long la = r * pa + g.at - g.shift_a, lb = r * pb + g.at - g.shift_b;
+                expect((a0 + la) % 8 == 0 && (b0 + lb) % 8 == 0, "aligned loads", r, D, g.at, 0);
+                expect(la >= 0 && la + (g.shift_a ? 16 : 8) <= sa, "gate granules", r, D, g.at, la);
+                expect(lb >= 0 && lb + (g.shift_b ? 16 : 8) <= sb, "up granules", r, D, g.at, lb);
+            }
+            for (int k = 0; k < 8; ++k) if (g.at + k >= 0 && g.at + k < D) ++owner[g.at + k];
+        }
+        for (int u = 0; u < D; ++u) expect(owner[u] == 1, "covered once", r, D, u, owner[u]);
+    }
+}
+
+int main() {
+    for (int D : {512, 513, 514, 519, 520, 527})
+        for (int rows : {1, 2, 3, 5})
+            for (long o = 0; o < 8; ++o)
+                for (long a = 0; a < 8; ++a) {
+                    silu_rows<1>(o, a, a + D, rows, D, D, 2 * D, 2 * D);        // the packed form
+                    silu_rows<1>(o, a, (5 * a + 3) % 8, rows, D, D + 3, D, D + 1);
+                    if (D % 2 == 0 && o % 2 == 0 && a % 2 == 0) silu_rows<2>(o, a, a + D, rows, D, D, 2 * D, 2 * D);
+                }
+    printf("%ld failures\n", failures);
+    return failures != 0;
+}
+"""
+
+
+def test_every_unit_of_a_ragged_row_has_one_owner_and_stays_inside(tmp_path):
+    src = tmp_path / "ragged.cu"
+    src.write_text(PROGRAM)
+    exe = tmp_path / "ragged"
+    subprocess.check_call([astra_build._nvcc(), "-std=c++17", "-O1", "-gencode", "arch=compute_100a,code=sm_100a",
+                           "-I", astra_build.INCLUDE, "-I", astra_build.CSRC, "-o", str(exe), str(src)])
+    done = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stdout
