@@ -402,6 +402,60 @@ bool launch_rmsnorm_wide(const RmsnormOperands &op, const uint16_t *w, int64_t T
     return true;
 }
 
+// Rows that start at any element, as long as x, residual and both outputs start at the same place within
+// 32 bytes (dense tensors always do).
+#ifndef ASTRA_RMSNORM_RAGGED_MIN_UNITS
+#define ASTRA_RMSNORM_RAGGED_MIN_UNITS 1024
+#endif
+constexpr int64_t kRmsnormRaggedMinUnits = ASTRA_RMSNORM_RAGGED_MIN_UNITS;  // at least 64 threads with one vector each
+
+template <int DT, int VPT, bool EARLY_W>
+cudaError_t launch_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T, int H, int threads, float eps,
+                                  cudaStream_t stream) {
+    const float inv_H = 1.0f / static_cast<float>(H);
+    for (int64_t t0 = 0; t0 < T; t0 += kMaxGridX) {
+        const unsigned rows = static_cast<unsigned>(T - t0 < kMaxGridX ? T - t0 : kMaxGridX);
+        RmsnormOperands o = op;
+        o.x += t0 * op.x_pitch;
+        o.r += t0 * op.r_pitch;
+        o.y += t0 * op.y_pitch;
+        o.r_out += t0 * op.r_out_pitch;
+        const cudaError_t err = launch(fused_add_rmsnorm_ragged_kernel<DT, VPT, EARLY_W>, rows, threads, stream, o, w, H,
+                                       eps, inv_H);
+        if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
+}
+
+// False where the ragged kernel does not apply.  One vector per thread up to 320 threads, then two (up to
+// 512 threads), then, for binary32 rows only (half the sums per unit), four: 21.3 us with one and 21.6 with two
+// at [4096, 4099], 45.1 and 41.4 us at [4096, 8188], 39.2 and 28.8 us at [2048, 11007].  Two also where that
+// makes one wave of what would be a little more (5 blocks of 256 threads per SM at 48 registers against 8
+// of 128 at 64: 6.8 -> 6.6 us at [1024, 4101]).  A few wide rows of 8-byte vectors are left to the clusters,
+// which spread each over several SMs (3.1 against 4.9 us at fp32 [16, 16382], 4.9 and 5.1 at 64 rows, 9.5 and
+// 6.5 at 128).
+constexpr int64_t kRmsnormRaggedWideRows = 64;
+template <int DT>
+bool try_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T, int H, int vec, float eps,
+                        cudaStream_t stream, cudaError_t *err) {
+    const int64_t Hu = static_cast<int64_t>(H) * Storage<DT>::UNITS;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(op.x);
+    const bool together = (op.x_pitch - op.r_pitch) % 16 == 0 && (op.x_pitch - op.y_pitch) % 16 == 0 &&
+                          (op.x_pitch - op.r_out_pitch) % 16 == 0 && (reinterpret_cast<uintptr_t>(op.r) - at) % 32 == 0 &&
+                          (reinterpret_cast<uintptr_t>(op.y) - at) % 32 == 0 &&
+                          (reinterpret_cast<uintptr_t>(op.r_out) - at) % 32 == 0;
+    if (!together || Hu < kRmsnormRaggedMinUnits) return false;
+    const int64_t nvec = Hu / 16;
+    auto threads_for = [&](int v) { const int64_t t = (nvec + v - 1) / v; return static_cast<int>((t + 31) / 32 * 32); };
+    const int64_t wave1 = 148 * (65536 / (48 * threads_for(1))), wave2 = 148 * (65536 / (64 * threads_for(2)));
+    if (nvec <= 320 && !(T > wave1 && T <= wave2)) *err = launch_rmsnorm_ragged<DT, 1, true>(op, w, T, H, threads_for(1), eps, stream);
+    else if (nvec <= 2 * kRmsnormRaggedMaxThreads) *err = launch_rmsnorm_ragged<DT, 2, false>(op, w, T, H, threads_for(2), eps, stream);
+    else if (DT == ASTRA_FP32 && nvec <= 4 * kRmsnormRaggedMaxThreads && !(vec == 4 && T <= kRmsnormRaggedWideRows)) {
+        if constexpr (DT == ASTRA_FP32) *err = launch_rmsnorm_ragged<DT, 4, false>(op, w, T, H, threads_for(4), eps, stream);
+    } else return false;
+    return true;
+}
+
 template <int DT>
 cudaError_t dispatch_rmsnorm(const RmsnormOperands &op, const uint16_t *w, int64_t T, int H, float eps,
                       cudaStream_t stream) {
@@ -412,6 +466,10 @@ cudaError_t dispatch_rmsnorm(const RmsnormOperands &op, const uint16_t *w, int64
         cudaError_t err = cudaSuccess;
         if (launch_rmsnorm_wide<DT>(op, w, T, H, eps, stream, &err)) return err;
         vec = 8;  // everything that is 32-byte aligned is 16-byte aligned
+    }
+    if (vec < 8) {
+        cudaError_t err = cudaSuccess;
+        if (try_rmsnorm_ragged<DT>(op, w, T, H, vec, eps, stream, &err)) return err;
     }
     switch (vec) {
         case 8: return launch_rmsnorm<DT, 8>(op, w, T, H, eps, stream);

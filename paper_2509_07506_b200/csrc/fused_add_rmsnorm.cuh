@@ -12,6 +12,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "vec.cuh"
 
 namespace astra {
@@ -173,6 +175,150 @@ fused_add_rmsnorm_reg_kernel(RmsnormOperands op, const uint16_t *__restrict__ we
             store<UV, STH>(yr + v * UV, narrow<DT, VEC>(fy));
         }
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Rows that start at any element (odd widths): x, residual and the outputs start at the same place within
+// a 32-byte granule, row by row, so the granules that lie inside the row (its body) are 32-byte accesses
+// of all four; the few units before and after them (the edge, at most 61) are one element per lane of the
+// first two warps.  Only the weight, which starts the same way for every row, lies at an offset to them:
+// its two granules per body vector are loaded whole and shifted, by an amount that is the row's.
+// ---------------------------------------------------------------------------------------------
+struct RaggedRow {
+    int first, nvec;  // the body: vectors [first, first + 16 * nvec)
+    int shift;        // of the weight against the body
+    int edge;         // this thread's edge unit, or -1
+};
+
+// The share of thread `thread` of a row of `units` units at `row`.  Body vectors whose weight granules would pass the weight's ends are left
+// to the edge: at most 31 units before the body and 30 after it.
+template <int UNITS>
+__host__ __device__ __forceinline__ RaggedRow ragged_row(const uint16_t *row, const uint16_t *weight, int units, int thread) {
+    constexpr int UV = 16;
+    RaggedRow g;
+    g.first = (UV - misalignment<UV>(row)) & (UV - 1);
+    g.shift = (misalignment<UV>(weight) + g.first) & (UV - 1);
+    if (g.shift > g.first) g.first += UV;
+    const int room = units - g.first - (g.shift ? UV - g.shift : 0);
+    g.nvec = room > 0 ? room / UV : 0;
+    int e = thread * UNITS;
+    if (e >= g.first) e += g.nvec * UV;
+    g.edge = e < units ? e : -1;
+    return g;
+}
+
+// The rest of a ragged row once its sums s (and the edge's es) are formed: reduction, weight, y.  EARLY_W
+// fetches the weight before the reduction (one vector per thread: no register more than the row's sums
+// needed).  STORE(unit offset, pack) writes y.
+template <int SHIFT, int DT, int VPT, bool EARLY_W, typename STORE>
+__device__ __forceinline__ void ragged_finish(const RaggedRow &g, const uint16_t *weight, float acc, float eps, float inv_H,
+                                              float *slots, float (&s)[VPT][16 / Storage<DT>::UNITS], float (&es)[1],
+                                              const Pack<Storage<DT>::UNITS> &ew, STORE store_y) {
+    constexpr int UV = 16, VEC = UV / Storage<DT>::UNITS;
+    Pack<UV> w0[VPT], w1[VPT];
+    auto fetch_weight = [&] {
+#pragma unroll
+        for (int i = 0; i < VPT; ++i) {
+            const int v = threadIdx.x + i * blockDim.x;
+            if (v < g.nvec) {
+                const uint16_t *w = weight + (g.first + v * UV - SHIFT);
+                w0[i] = load<UV, Ld::Keep>(w);
+                if constexpr (SHIFT != 0) w1[i] = load<UV, Ld::Keep>(w + UV);
+            }
+        }
+    };
+    if constexpr (EARLY_W) fetch_weight();
+    const float total = block_sum(acc, slots);
+    const float rstd = rsqrtf(fmaf(total, inv_H, eps));
+    if constexpr (!EARLY_W) fetch_weight();
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int v = threadIdx.x + i * blockDim.x;
+        if (v < g.nvec) {
+            float fw[VEC], fy[VEC];
+            widen<DT, VEC>(realign<SHIFT, UV>(w0[i], w1[i]), fw);
+            scale(s[i], rstd, fw, fy);
+            store_y(g.first + v * UV, narrow<DT, VEC>(fy));
+        }
+    }
+    if (g.edge >= 0) {
+        float fw[1], fy[1];
+        widen<DT, 1>(ew, fw);
+        scale(es, rstd, fw, fy);
+        store_y(g.edge, narrow<DT, 1>(fy));
+    }
+}
+
+// HBM-bound like the aligned kernel, of which it moves the same bytes in the same widths; what it pays for
+// the row's place is the second weight granule, a funnel shift per word of weight and two warps' edge.
+// Launched with at least 64 threads (the edge), VPT vectors per thread covering units / 16 of them.
+// Measured L2-cold, fp16, against the kernels for 2-, 4- and 8-byte vectors: 41.8 -> 21.3 us at [4096, 4099]
+// (19.5 us at 6.9 TB/s), 99.4 -> 28.8 us at [2048, 11007], 142 -> 41.0 us at [2048, 16383], 12.3 -> 6.9 us at
+// [1024, 4101], 2.9 -> 2.0 us at [16, 4099], 25.0 -> 21.3 us at [4096, 4098], 79.7 -> 78.8 us at [16384, 4100];
+// fp32 56.9 -> 40.9 us at [2048, 8191], 81 -> 43 us at [1024, 16383].  Also tried: 16-byte granules (21.7 and
+// 29.2 us at [4096, 4099] and [2048, 11007]), run-time shifts by selects (22.6 and 40.4 us), the edge as
+// partial vectors in the main loop (29.8 and 54.6 us: its branches serialise the loads).
+// Two vectors per thread hold the sums of 16384 units in two blocks of 512 threads per SM at 64 registers.
+constexpr int kRmsnormRaggedMaxThreads = 512;
+template <int DT, int VPT, bool EARLY_W>
+__global__ void __launch_bounds__(kRmsnormRaggedMaxThreads, VPT <= 2 ? 2 : 1)
+fused_add_rmsnorm_ragged_kernel(RmsnormOperands op, const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
+    constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
+    __shared__ float slots[kMaxWarps];
+    const int units = H * UNITS;
+    const int64_t row = blockIdx.x;
+    const uint16_t *xr = op.x + row * op.x_pitch;
+    const uint16_t *rr = op.r + row * op.r_pitch;
+    uint16_t *yr = op.y + row * op.y_pitch;
+    uint16_t *ror = op.r_out + row * op.r_out_pitch;
+    if (threadIdx.x == 0) {
+        prefetch_l2_range(xr, static_cast<int64_t>(units) * 2);
+        prefetch_l2_range(rr, static_cast<int64_t>(units) * 2);
+    }
+    const RaggedRow g = ragged_row<UNITS>(xr, weight, units, static_cast<int>(threadIdx.x));
+    grid_dependency_wait();
+    grid_launch_dependents();
+
+    Pack<UV> px[VPT], pr[VPT];
+    Pack<UNITS> ex, er, ew;
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int v = threadIdx.x + i * blockDim.x;
+        if (v < g.nvec) {
+            px[i] = load<UV, Ld::Stream>(xr + (g.first + v * UV));
+            pr[i] = load<UV, Ld::Stream>(rr + (g.first + v * UV));
+        }
+    }
+    if (g.edge >= 0) {
+        ex = load<UNITS, Ld::Stream>(xr + g.edge);
+        er = load<UNITS, Ld::Stream>(rr + g.edge);
+        ew = load<UNITS, Ld::Keep>(weight + g.edge);
+    }
+    float s[VPT][VEC], es[1];
+    float acc = 0.f;
+    float2 acc2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int v = threadIdx.x + i * blockDim.x;
+        if (v < g.nvec) {
+            float fx[VEC], fr[VEC];
+            widen<DT, VEC>(px[i], fx);
+            widen<DT, VEC>(pr[i], fr);
+            add_and_square(fx, fr, s[i], acc, acc2);
+            store<UV, St::Stream>(ror + (g.first + v * UV), narrow<DT, VEC>(s[i]));
+        }
+    }
+    if (g.edge >= 0) {
+        float fx[1], fr[1];
+        widen<DT, 1>(ex, fx);
+        widen<DT, 1>(er, fr);
+        add_and_square(fx, fr, es, acc, acc2);
+        store<UNITS, St::Stream>(ror + g.edge, narrow<DT, 1>(es));
+    }
+    auto store_y = [&](int at, const auto &v) { store<std::decay_t<decltype(v)>::UNITS_PER_PACK, St::Stream>(yr + at, v); };
+    ASTRA_FOR_SHIFT(g.shift, UNITS,
+                    (ragged_finish<SHIFT, DT, VPT, EARLY_W>(g, weight, acc + (acc2.x + acc2.y), eps, inv_H, slots, s, es, ew,
+                                                            store_y)))
 }
 
 // Rows too wide for one block's registers: a thread-block cluster owns the row.  Each block keeps

@@ -1,6 +1,7 @@
 """Rows that start at any element: the kernels for odd widths and pitches against the oracle, at the edges
 of their ranges, every storage type, operand offsets of every alignment class, pitches that move the
 operands against one another."""
+import numpy as np
 import pytest
 import torch
 
@@ -8,7 +9,7 @@ import oracle
 import paper_2509_07506_b200 as astra
 from paper_2509_07506_b200 import workloads as wl
 from parity import check_values
-from test_gpu_parity import f64, run_silu
+from test_gpu_parity import f64, run_rmsnorm, run_silu
 from test_gpu_strided import pitched, untouched
 
 pytestmark = pytest.mark.gpu
@@ -36,3 +37,26 @@ def test_silu_ragged_pitches(D, pitches):
     check_values(f64(ov.cpu()), oracle.silu_and_mul(wl.bits(inp.input), BF16), BF16, what="silu ragged pitches")
     for buf in (gb, ub, ob):
         assert untouched(buf, 0, D)
+
+
+@pytest.mark.parametrize("dtype", [BF16, FP16, FP32])
+@pytest.mark.parametrize("offset", [0, 1, 6, 15])
+@pytest.mark.parametrize("T,H", [(1, 1025), (3, 1039), (17, 2051), (5, 5121), (4, 5135), (300, 4099), (6, 5137), (3, 8191),
+                                 (7, 11007), (5, 16383), (3, 16401), (1030, 2050)])
+def test_rmsnorm_ragged_rows(T, H, offset, dtype):
+    run_rmsnorm(wl.rmsnorm_inputs(T, H, dtype, eps=1e-5, seed=H + offset), offset=offset)
+
+
+@pytest.mark.parametrize("pads", [(0, 0, 0, 0), (16, 128, 0, 32), (16, 8, 0, 0)])
+def test_rmsnorm_ragged_pitches(pads):
+    """Pitches that keep the four tensors together modulo 32 bytes, and (last) pitches that do not."""
+    T, H = 19, 4099
+    inp = wl.rmsnorm_inputs(T, H, FP16, eps=1e-5, seed=sum(pads))
+    (xb, xv), (rb, rv) = pitched(inp.x, H + pads[0], 0), pitched(inp.residual, H + pads[1], 0)
+    (yb, yv), (ob, ov) = (pitched(torch.zeros_like(inp.x), H + p, 0) for p in pads[2:])
+    astra.astra_fused_add_rmsnorm_ex(yv, ov, xv, rv, inp.weight.cuda(), inp.eps)
+    oy, orr = oracle.fused_add_rmsnorm(wl.bits(inp.x), wl.bits(inp.residual), wl.bits(inp.weight), inp.eps, FP16)
+    assert np.array_equal(wl.bits(ov.cpu().contiguous()), orr)
+    check_values(f64(yv.cpu()), oy, FP16, what="rmsnorm ragged pitches")
+    for buf in (xb, rb, yb, ob):
+        assert untouched(buf, 0, H)

@@ -10,6 +10,7 @@ from paper_2509_07506_b200 import build as astra_build
 PROGRAM = r"""
 #include <cstdio>
 #include <vector>
+#include "fused_add_rmsnorm.cuh"
 #include "silu_and_mul.cuh"
 using namespace astra;
 
@@ -18,6 +19,28 @@ static void expect(bool ok, const char *what, long a, long b, long c, long d) {
     if (!ok && failures++ < 5) printf("%s: %ld %ld %ld %ld\n", what, a, b, c, d);
 }
 static const uint16_t *at_unit(long u) { return reinterpret_cast<const uint16_t *>(4096 + 2 * u); }
+
+// Body and edge of one row, over all threads of a block of `threads` with `vpt` vectors each.
+template <int UNITS> static void norm_row(long row, long weight, int units, int vpt, int threads) {
+    std::vector<int> owner(units, 0);
+    for (int t = 0; t < threads; ++t) {
+        const RaggedRow g = ragged_row<UNITS>(at_unit(row), at_unit(weight), units, t);
+        for (int i = 0; i < vpt; ++i) {
+            const int v = t + i * threads;
+            if (v >= g.nvec) continue;
+            const int at = g.first + v * 16;
+            expect((row + at) % 16 == 0 && (weight + at - g.shift) % 16 == 0, "alignment", row, weight, units, at);
+            expect(at >= 0 && at + 16 <= units, "body", row, weight, units, at);
+            expect(at - g.shift >= 0 && at - g.shift + (g.shift ? 32 : 16) <= units, "weight", row, weight, units, at);
+            for (int k = 0; k < 16; ++k) ++owner[at + k];
+        }
+        if (g.edge >= 0) {
+            expect(g.edge + UNITS <= units, "edge", row, weight, units, g.edge);
+            for (int k = 0; k < UNITS; ++k) ++owner[g.edge + k];
+        }
+    }
+    for (int u = 0; u < units; ++u) expect(owner[u] == 1, "covered once", row, weight, units, u);
+}
 
 // All granules of a [rows, D] call with pitched operands; every tensor is [0, span) units from its base.
 template <int UNITS> static void silu_rows(long o0, long a0, long b0, int rows, int D, long po, long pa, long pb) {
@@ -43,6 +66,14 @@ template <int UNITS> static void silu_rows(long o0, long a0, long b0, int rows, 
 }
 
 int main() {
+    for (int units : {1024, 1025, 1039, 1040, 1041, 1055, 1056, 2051, 5120, 5135, 5136})
+        for (long row = 0; row < 16; ++row)
+            for (long weight = 0; weight < 16; ++weight) {
+                const int one = (units / 16 + 31) / 32 * 32, two = ((units / 16 + 1) / 2 + 31) / 32 * 32;
+                norm_row<1>(row, weight, units, 1, one);
+                norm_row<1>(row, weight, units, 2, two < 64 ? 64 : two);
+                if (units % 2 == 0 && row % 2 == 0 && weight % 2 == 0) norm_row<2>(row, weight, units, 1, one);
+            }
     for (int D : {512, 513, 514, 519, 520, 527})
         for (int rows : {1, 2, 3, 5})
             for (long o = 0; o < 8; ++o)
