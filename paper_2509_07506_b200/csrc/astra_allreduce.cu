@@ -14,6 +14,9 @@ using namespace astra::host;
 
 inline int round_up_to(int v, int m) { return (v + m - 1) / m * m; }
 
+constexpr int kStreamGroup = 2;  // partial loads in flight: long streams,
+constexpr int kDeepGroup = 8;    // and few rows
+
 // Register-resident rows hold at most 32 16-bit units per thread in vectors of 8, 16 or 32 bytes.
 // UVEC is the vector width in units, VPT the vectors per thread.
 // `dense` selects the instantiation whose registers are capped so that five 256-thread blocks fit an
@@ -44,8 +47,6 @@ cudaError_t launch_reg(const AllreduceOperands &op, const uint16_t *w, unsigned 
 //    partial loads in flight and 8 units per thread (512-thread blocks), so that all partials of a
 //    row arrive in one round trip: 2.5 against 3.9 us at [16, 4096] with 8 partials (with one or two
 //    partials the queue stays at two, the per-thread share is still 8 units: 1.8 against 2.0 us).
-constexpr int kStreamGroup = 2;
-constexpr int kLatencyGroup = 8;
 #ifndef ASTRA_ALLREDUCE_LATENCY_ROWS
 #define ASTRA_ALLREDUCE_LATENCY_ROWS (2 * 148)
 #endif
@@ -71,8 +72,17 @@ inline int pick_vpt(int nvec, int start_units, int *threads_out) {
     return vpt;
 }
 
+// The ragged kernel (rows that start anywhere): 32-byte vectors, one or two per thread.
+template <int DT, int UVEC, int VPT, int GROUP>
+cudaError_t launch_ragged(const AllreduceOperands &op, const uint16_t *w, unsigned rows, int threads, int H, float eps,
+                          float inv_H, cudaStream_t stream) {
+    if constexpr (UVEC == 16 && VPT <= 2 && !(GROUP == kDeepGroup && VPT > 1))
+        return launch(fused_allreduce_add_rmsnorm_ragged_kernel<DT, VPT, GROUP>, rows, threads, stream, op, w, H, eps, inv_H);
+    return cudaErrorInvalidValue;
+}
+
 // Launches over all rows (split where the grid limit requires).  vpt = 0 selects the two-sweep kernel.
-template <int DT, int UVEC, int GROUP>
+template <int DT, int UVEC, int GROUP, bool RAGGED = false>
 cudaError_t launch_rows(AllreduceOperands op, const uint16_t *w, int64_t T, int H, float eps, int vpt,
                         int threads, cudaStream_t stream) {
   if constexpr (UVEC >= Storage<DT>::UNITS) {
@@ -94,6 +104,12 @@ cudaError_t launch_rows(AllreduceOperands op, const uint16_t *w, int64_t T, int 
         }
         o.r += t0 * row_units;
         cudaError_t err;
+        if constexpr (RAGGED) {
+            err = vpt == 1 ? launch_ragged<DT, UVEC, 1, GROUP>(o, w, rows, threads, H, eps, inv_H, stream)
+                           : launch_ragged<DT, UVEC, 2, GROUP>(o, w, rows, threads, H, eps, inv_H, stream);
+            if (err != cudaSuccess) return err;
+            continue;
+        }
         switch (vpt) {
             case 0: err = launch(fused_allreduce_add_rmsnorm_twopass_kernel<DT, VEC, GROUP>, rows, sweep_threads,
                                  stream, o, w, H, eps, inv_H); break;
@@ -115,8 +131,8 @@ cudaError_t choose_shape(const AllreduceOperands &op, const uint16_t *w, int64_t
     const int nvec = H / (UVEC / Storage<DT>::UNITS);
     int threads = 0;
     if (T <= kLatencyRows && op.n_parts > kStreamGroup) {
-        const int vpt = pick_vpt<UVEC, kLatencyGroup>(nvec, 8, &threads);
-        if (vpt > 0) return launch_rows<DT, UVEC, kLatencyGroup>(op, w, T, H, eps, vpt, threads, stream);
+        const int vpt = pick_vpt<UVEC, kDeepGroup>(nvec, 8, &threads);
+        if (vpt > 0) return launch_rows<DT, UVEC, kDeepGroup>(op, w, T, H, eps, vpt, threads, stream);
     }
     const int start_units = T <= kLatencyRows ? 8 : 16;
     const int vpt = pick_vpt<UVEC, kStreamGroup>(nvec, start_units, &threads);  // 0: the row does not fit the registers
@@ -150,30 +166,34 @@ struct WideShape {
 constexpr int64_t kDeepQueueRows = ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS;
 constexpr WideShape kWideShapes[] = {
     {1, 4, 72, 512, 128}, {2, 4, 128, 256, 64}, {1, 2, 56, 1024, 128}, {2, 2, 96, 512, 64}};
+// The same shapes of the ragged kernel, with its registers (the last one takes fewer for binary32).
+template <int DT> constexpr WideShape kRaggedShapes[] = {
+    {1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, DT == ASTRA_FP32 ? 96 : 120, 512, 64}};
 constexpr int64_t kWideBytesInFlight = 90 * 1024;
 
-template <int DT>
+template <int DT, bool RAGGED>
 bool launch_wide(const AllreduceOperands &op, const uint16_t *w, int64_t T, int H, float eps, cudaStream_t stream,
                  cudaError_t *err) {
     constexpr int UVEC = 16;
-    const int nvec = H / (UVEC / Storage<DT>::UNITS);
+    const int nvec = H / (UVEC / Storage<DT>::UNITS);  // whole vectors (a ragged row has no more inside it)
     // Few rows and more than four partials: all of a row's partials in one round trip (eight loads in
     // flight, one vector per thread); with so few blocks the registers that costs do not matter.
     // Device time from a graph, 8 partials, against the streaming shapes: 3.19 -> 2.70 us at [16, 4096],
     // 4.17 -> 3.41 us at [16, 8192], 4.12 -> 3.85 us at [128, 4096]; slower from 192 rows on (7.93 -> 8.89 us
     // at [192, 8192]).  With up to four partials the streaming shapes are the fastest at every row
     // count (1.65 / 1.98 us at [16, 4096] with 2 / 4 partials, where the 16-byte shapes took 2.08 / 2.40).
-    if (T <= kDeepQueueRows && op.n_parts > 4) {
+    // (The ragged kernel's four-in-flight shape fetches its edge last, so there four partials count as many.)
+    if (T <= kDeepQueueRows && op.n_parts > (RAGGED ? 3 : 4)) {
         const int threads = round_up_to(nvec, 32);
-        if (threads >= 128 && threads <= allreduce_reg_max_threads(16, kLatencyGroup)) {
-            *err = launch_rows<DT, UVEC, kLatencyGroup>(op, w, T, H, eps, 1, threads, stream);
+        if (threads >= (RAGGED ? 64 : 128) && threads <= allreduce_reg_max_threads(16, kDeepGroup)) {
+            *err = launch_rows<DT, UVEC, kDeepGroup, RAGGED>(op, w, T, H, eps, 1, threads, stream);
             return true;
         }
     }
     int best = -1, best_threads = 0;
     int64_t best_bytes = 0;
     for (int c = 0; c < 4; ++c) {
-        const WideShape &sh = kWideShapes[c];
+        const WideShape &sh = RAGGED ? kRaggedShapes<DT>[c] : kWideShapes[c];
         if (sh.group > kStreamGroup && op.n_parts < sh.group) continue;
         const int threads = round_up_to((nvec + sh.vpt - 1) / sh.vpt, 32);
         if (threads > sh.max_threads || threads < sh.min_threads) continue;
@@ -188,11 +208,21 @@ bool launch_wide(const AllreduceOperands &op, const uint16_t *w, int64_t T, int 
         if (bytes >= kWideBytesInFlight) break;  // the first shape that reaches it is also the largest so far
     }
     if (best < 0) return false;
-    const WideShape &sh = kWideShapes[best];
+    const WideShape &sh = RAGGED ? kRaggedShapes<DT>[best] : kWideShapes[best];
     if (sh.group == 4)
-        *err = launch_rows<DT, UVEC, 4>(op, w, T, H, eps, sh.vpt, best_threads, stream);
+        *err = launch_rows<DT, UVEC, 4, RAGGED>(op, w, T, H, eps, sh.vpt, best_threads, stream);
     else
-        *err = launch_rows<DT, UVEC, kStreamGroup>(op, w, T, H, eps, sh.vpt, best_threads, stream);
+        *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED>(op, w, T, H, eps, sh.vpt, best_threads, stream);
+    return true;
+}
+
+// Do all row-addressed operands start at the same place within 32 bytes?
+inline bool rows_together(const AllreduceOperands &op) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(op.r);
+    auto same = [&](const void *p) { return (reinterpret_cast<uintptr_t>(p) - at) % 32 == 0; };
+    for (int p = 0; p < op.n_parts; ++p) if (!same(op.part[p])) return false;
+    for (int d = 0; d < op.n_y; ++d) if (!same(op.y_out[d])) return false;
+    for (int d = 0; d < op.n_r; ++d) if (!same(op.r_out[d])) return false;
     return true;
 }
 
@@ -206,8 +236,22 @@ cudaError_t dispatch(const AllreduceOperands &op, const uint16_t *w, int64_t T, 
     for (int d = 0; d < op.n_r; ++d) pick.pointer(op.r_out[d]);
     if (pick.vec == 16) {
         cudaError_t err = cudaSuccess;
-        if (launch_wide<DT>(op, w, T, H, eps, stream, &err)) return err;
+        if (launch_wide<DT, false>(op, w, T, H, eps, stream, &err)) return err;
         pick.vec = 8;  // everything that is 32-byte aligned is 16-byte aligned
+    }
+    // Rows of less than 16-byte alignment go to the ragged kernel (figures there), except where the 8-byte
+    // forms are the faster ones: few rows, whose latency their smaller code serves better (1.8 against 2.1 us
+    // at [16, 4100] with 2 partials, 3.3 against 4.2 us at [140, 4100] with 4, 4.35 against 4.6 us at [64, 8188] with 8; but 7.5 -> 6.1 us at [16, 14332]
+    // with 8, 5.8 -> 3.8 us at fp32 [16, 4098]), two or three partials up to 512 rows (4.05 against 4.5 us at
+    // [400, 4100]; 9.1 -> 7.1 us at [512, 4100] with 4), and binary32 rows of more than 10240 units, where
+    // one block per SM is left (41.2 against 45.9 us at fp32 [1024, 8190] with 4; 27.5 -> 13.2 us at [512, 5001]).
+    const int64_t units = static_cast<int64_t>(H) * Storage<DT>::UNITS;
+    const bool few = T <= 148;  // a block per SM at most
+    const bool narrow_form = pick.vec == 4 && (DT == ASTRA_FP32 ? units > 10240 || (op.n_parts < 4 && few)
+                                                                : (op.n_parts < 4 && T <= 512) || (units <= 8192 && few));
+    if (pick.vec < 8 && !narrow_form && rows_together(op)) {
+        cudaError_t err = cudaSuccess;
+        if (launch_wide<DT, true>(op, w, T, H, eps, stream, &err)) return err;
     }
     switch (pick.vec) {
         case 8: return choose_shape<DT, 8>(op, w, T, H, eps, stream);

@@ -191,6 +191,131 @@ fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands
     }
 }
 
+// Rows that start at any element (odd widths), all operands at the same place within 32 bytes: body in
+// 32-byte vectors, edge one unit per lane of the first two warps, weight shifted, as in
+// fused_add_rmsnorm_ragged_kernel; partials and shapes as in the kernel above.  The edge's partials
+// are fetched group by group beside the body's.  (The plain loads and stores stay per-thread here too: a
+// partial or a destination may be another GPU's memory.)
+// Measured L2-cold, bf16, against the 2-, 4- and 8-byte vector kernels: see the launch code.
+template <int DT, int VPT, int GROUP>
+__global__ void __launch_bounds__(allreduce_reg_max_threads(16 * VPT, GROUP))
+fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOperands op,
+                                          const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
+    constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
+    constexpr bool EDGE_LAST = GROUP == 4, EARLY_W = GROUP > 4;
+    __shared__ float slots[kMaxWarps];
+    const int units = H * UNITS;
+    const int64_t row = static_cast<int64_t>(blockIdx.x) * units;
+    const int n = op.n_parts;
+    if (threadIdx.x == 0) prefetch_l2_range(op.r + row, static_cast<int64_t>(units) * 2);
+    const RaggedRow g = ragged_row<UNITS>(op.r + row, weight, units, static_cast<int>(threadIdx.x));
+    const int64_t body = row + g.first;
+    grid_dependency_wait();
+    grid_launch_dependents();
+
+    Pack<UV> pr[VPT];
+    Pack<UNITS> er, ew;
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int v = threadIdx.x + i * blockDim.x;
+        if (v < g.nvec) pr[i] = load<UV, Ld::Stream>(op.r + body + v * UV);
+    }
+    if (!EDGE_LAST && g.edge >= 0) {
+        er = load<UNITS, Ld::Stream>(op.r + row + g.edge);
+        ew = load<UNITS, Ld::Keep>(weight + g.edge);
+    }
+    float s[VPT][VEC], es[1] = {0.f};
+#pragma unroll
+    for (int p0 = 0; p0 < kMaxParts; p0 += GROUP) {
+        if (p0 >= n) break;
+        Pack<UV> px[GROUP][VPT];
+        Pack<UNITS> ex[GROUP];
+#pragma unroll
+        for (int q = 0; q < GROUP; ++q) {
+            if (p0 + q < n) {
+                const uint16_t *base = op.part[p0 + q];
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) {
+                    const int v = threadIdx.x + i * blockDim.x;
+                    if (v < g.nvec) px[q][i] = load<UV, Ld::Stream>(base + body + v * UV);
+                }
+                if (!EDGE_LAST && g.edge >= 0) ex[q] = load<UNITS, Ld::Stream>(base + row + g.edge);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < GROUP; ++q) {
+            if (p0 + q < n) {
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) {
+                    const int v = threadIdx.x + i * blockDim.x;
+                    if (v < g.nvec) {
+                        float fx[VEC];
+                        widen<DT, VEC>(px[q][i], fx);
+                        if (p0 + q == 0) {
+#pragma unroll
+                            for (int k = 0; k < VEC; ++k) s[i][k] = fx[k];
+                        } else {
+                            accumulate(s[i], fx);
+                        }
+                    }
+                }
+                if (!EDGE_LAST && g.edge >= 0) {
+                    float fx[1];
+                    widen<DT, 1>(ex[q], fx);
+                    if (p0 + q == 0) es[0] = fx[0];
+                    else accumulate(es, fx);
+                }
+            }
+        }
+    }
+
+    float acc = 0.f;
+    float2 acc2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int v = threadIdx.x + i * blockDim.x;
+        if (v < g.nvec) {
+            float fr[VEC];
+            widen<DT, VEC>(pr[i], fr);
+            add_and_square(s[i], fr, s[i], acc, acc2);
+            store_to_all<UV>(op.r_out, op.n_r, body + v * UV, narrow<DT, VEC>(s[i]));
+        }
+    }
+    if (EDGE_LAST && g.edge >= 0) {
+        er = load<UNITS, Ld::Stream>(op.r + row + g.edge);
+        ew = load<UNITS, Ld::Keep>(weight + g.edge);
+#pragma unroll
+        for (int p0 = 0; p0 < kMaxParts; p0 += 8) {
+            if (p0 >= n) break;
+            Pack<UNITS> ex[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (p0 + q < n) ex[q] = load<UNITS, Ld::Stream>(op.part[p0 + q] + row + g.edge);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (p0 + q < n) {
+                    float fx[1];
+                    widen<DT, 1>(ex[q], fx);
+                    if (p0 + q == 0) es[0] = fx[0];
+                    else accumulate(es, fx);
+                }
+            }
+        }
+    }
+    if (g.edge >= 0) {
+        float fr[1];
+        widen<DT, 1>(er, fr);
+        add_and_square(es, fr, es, acc, acc2);
+        store_to_all<UNITS>(op.r_out, op.n_r, row + g.edge, narrow<DT, 1>(es));
+    }
+    auto store_y = [&](int at, const auto &v) {
+        store_to_all<std::decay_t<decltype(v)>::UNITS_PER_PACK>(op.y_out, op.n_y, row + at, v);
+    };
+    ASTRA_FOR_SHIFT(g.shift, UNITS,
+                    (ragged_finish<SHIFT, DT, VPT, EARLY_W>(g, weight, acc + (acc2.x + acc2.y), eps, inv_H, slots, s, es, ew,
+                                                          store_y)))
+}
+
 // The rank-order sum of one vector position, GROUP partial loads in flight at a time.
 template <int DT, int VEC, int GROUP>
 __device__ __forceinline__ void rank_order_sum(const AllreduceOperands &op, int64_t at, float (&s)[VEC]) {

@@ -9,6 +9,7 @@ import oracle
 import paper_2509_07506_b200 as astra
 from paper_2509_07506_b200 import workloads as wl
 from parity import check_values
+from test_gpu_allreduce import run_allreduce
 from test_gpu_parity import f64, run_rmsnorm, run_silu
 from test_gpu_strided import pitched, untouched
 
@@ -60,3 +61,10 @@ def test_rmsnorm_ragged_pitches(pads):
     check_values(f64(yv.cpu()), oy, FP16, what="rmsnorm ragged pitches")
     for buf in (xb, rb, yb, ob):
         assert untouched(buf, 0, H)
+
+
+@pytest.mark.parametrize("dtype", [BF16, FP16, FP32])
+@pytest.mark.parametrize("n_parts", [2, 4, 9])
+@pytest.mark.parametrize("T,H,offset", [(3, 2049, 0), (16, 4099, 1), (129, 2051, 6), (9, 8189, 15), (5, 16383, 0), (4, 1027, 3)])
+def test_allreduce_rmsnorm_ragged_rows(n_parts, T, H, offset, dtype):
+    run_allreduce(wl.allreduce_rmsnorm_inputs(T, H, n_parts, dtype, seed=H + n_parts), offset=offset)
