@@ -217,15 +217,20 @@ cudaError_t launch_merge_strided(uint16_t *v_out, float *lse_out, const uint16_t
     constexpr int VEC = UVEC / Storage<DT>::UNITS;
     const int64_t nvec = D / UVEC;
     const int64_t rows_per_launch = kMaxVecsPerLaunch / nvec;
+    const int64_t T = rows_total / Hh;
+    auto dense_tensor = [&](int64_t st_t, int64_t st_h) { return (Hh == 1 || st_h == D) && (T == 1 || st_t == Hh * D); };
+    const bool dense = dense_tensor(st.va_t, st.va_h) && dense_tensor(st.vb_t, st.vb_h) && dense_tensor(st.vo_t, st.vo_h);
     for (int64_t r0 = 0; r0 < rows_total; r0 += rows_per_launch) {
         const int64_t rows = (rows_total - r0 < rows_per_launch) ? (rows_total - r0) : rows_per_launch;
         const uint32_t total = static_cast<uint32_t>(rows * nvec);
         const uint32_t tile = THREADS * UNROLL;
         const uint32_t blocks = (total + tile - 1) / tile;
+        const FastDiv per_row = FastDiv::make(static_cast<uint32_t>(nvec)), heads = FastDiv::make(static_cast<uint32_t>(Hh));
         const cudaError_t err =
-            launch(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS>, blocks, THREADS, stream,
-                   v_out, lse_out, v_a, lse_a, v_b, lse_b, total, static_cast<uint32_t>(r0),
-                   FastDiv::make(static_cast<uint32_t>(nvec)), FastDiv::make(static_cast<uint32_t>(Hh)), st);
+            dense ? launch(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, true>, blocks, THREADS, stream,
+                           v_out, lse_out, v_a, lse_a, v_b, lse_b, total, static_cast<uint32_t>(r0), per_row, heads, st)
+                  : launch(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, false>, blocks, THREADS, stream,
+                           v_out, lse_out, v_a, lse_a, v_b, lse_b, total, static_cast<uint32_t>(r0), per_row, heads, st);
         if (err != cudaSuccess) return err;
     }
   }

@@ -116,7 +116,10 @@ namespace astra {
 // Same computation for arbitrarily strided tensors (head_dim contiguous): row = token * Hh + head is
 // split again into (token, head) to address each tensor by its own strides.  This is the form for
 // head-major scores ([Hh, T]) or values that are slices of a wider buffer.
-template <int DT, int VEC, int UNROLL, int THREADS>
+// DENSE_VALUES: the three value tensors are dense [T, Hh, D] (the usual case of head-major scores), so their
+// vectors are addressed flat and a block's share of each input is one contiguous range, which it asks for
+// ahead of the dependency wait, as above; otherwise a thread per row asks for that row.
+template <int DT, int VEC, int UNROLL, int THREADS, bool DENSE_VALUES>
 __global__ void __launch_bounds__(THREADS)
 merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
                                      const uint16_t *v_a, const float *lse_a,
@@ -124,9 +127,28 @@ merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
                                      uint32_t total_vecs, uint32_t row0, FastDiv nvec, FastDiv heads,
                                      MergeStrides st) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
-    const uint32_t base = blockIdx.x * (THREADS * UNROLL) + threadIdx.x;
+    const uint32_t first = blockIdx.x * (THREADS * UNROLL);
+    const uint32_t base = first + threadIdx.x;
+    const uint32_t count = min(static_cast<uint32_t>(THREADS * UNROLL), total_vecs - first);
+    const int64_t flat0 = static_cast<int64_t>(row0) * nvec.d;  // the launch's first vector in a dense tensor
+    if constexpr (DENSE_VALUES) {
+        if (threadIdx.x == 0) {
+            prefetch_l2_range(v_a + (flat0 + first) * UV, static_cast<int64_t>(count) * UV * 2);
+            prefetch_l2_range(v_b + (flat0 + first) * UV, static_cast<int64_t>(count) * UV * 2);
+        }
+    } else {
+        const uint32_t lrow = nvec.div(first) + threadIdx.x;
+        if (lrow <= nvec.div(first + count - 1)) {
+            const uint32_t row = row0 + lrow, t = heads.div(row), h = row - t * heads.d;
+            const int64_t bytes = static_cast<int64_t>(nvec.d) * UV * 2;
+            prefetch_l2_range(v_a + (t * st.va_t + h * st.va_h), bytes);
+            prefetch_l2_range(v_b + (t * st.vb_t + h * st.vb_h), bytes);
+        }
+    }
     grid_dependency_wait();
     grid_launch_dependents();
+    Pack<UV> a[UNROLL], b[UNROLL];
+    float sa[UNROLL], sb[UNROLL];
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j) {
         const uint32_t v = base + j * THREADS;
@@ -136,18 +158,32 @@ merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
             const uint32_t row = row0 + lrow;  // rows of this launch start at row0
             const uint32_t t = heads.div(row);
             const uint32_t h = row - t * heads.d;
-            const Pack<UV> a = load<UV, Ld::Stream>(v_a + (t * st.va_t + h * st.va_h + col));
-            const Pack<UV> b = load<UV, Ld::Stream>(v_b + (t * st.vb_t + h * st.vb_h + col));
-            const MergeWeights mw = merge_weights(lse_a[t * st.sa_t + h * st.sa_h], lse_b[t * st.sb_t + h * st.sb_h]);
+            a[j] = load<UV, Ld::Stream>(v_a + (DENSE_VALUES ? (flat0 + v) * UV : t * st.va_t + h * st.va_h + col));
+            b[j] = load<UV, Ld::Stream>(v_b + (DENSE_VALUES ? (flat0 + v) * UV : t * st.vb_t + h * st.vb_h + col));
+            sa[j] = lse_a[t * st.sa_t + h * st.sa_h];
+            sb[j] = lse_b[t * st.sb_t + h * st.sb_h];
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < UNROLL; ++j) {
+        const uint32_t v = base + j * THREADS;
+        if (v < total_vecs) {
+            const uint32_t lrow = nvec.div(v);
+            const int64_t col = static_cast<int64_t>(v - lrow * nvec.d) * UV;
+            const uint32_t row = row0 + lrow;
+            const uint32_t t = heads.div(row);
+            const uint32_t h = row - t * heads.d;
+            const MergeWeights mw = merge_weights(sa[j], sb[j]);
             float fa[VEC], fb[VEC], fo[VEC];
-            widen<DT, VEC>(a, fa);
-            widen<DT, VEC>(b, fb);
+            widen<DT, VEC>(a[j], fa);
+            widen<DT, VEC>(b[j], fb);
 #pragma unroll
             for (int i = 0; i < VEC; ++i) {
                 const float ta = mw.use_a ? fa[i] * mw.wa : 0.f;
                 fo[i] = mw.use_b ? fmaf(fb[i], mw.wb, ta) : ta;
             }
-            store<UV, St::Stream>(v_out + (t * st.vo_t + h * st.vo_h + col), narrow<DT, VEC>(fo));
+            store<UV, St::Stream>(v_out + (DENSE_VALUES ? (flat0 + v) * UV : t * st.vo_t + h * st.vo_h + col),
+                                  narrow<DT, VEC>(fo));
             if (lse_out != nullptr && col == 0) lse_out[t * st.so_t + h * st.so_h] = mw.lse;
         }
     }
