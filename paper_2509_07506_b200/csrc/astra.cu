@@ -402,7 +402,11 @@ bool launch_rmsnorm_wide(const RmsnormOperands &op, const uint16_t *w, int64_t T
         o.r += t0 * op.r_pitch;
         o.y += t0 * op.y_pitch;
         o.r_out += t0 * op.r_out_pitch;
-        *err = launch(fused_add_rmsnorm_reg_kernel<DT, VEC, VPT>, rows, threads, stream, o, w, H, eps, inv_H);
+        if (T <= kWideVectorDecodeRows && threads <= 256)  // the decode form
+            *err = launch(fused_add_rmsnorm_reg_kernel<DT, VEC, VPT, Ld::Stream, St::Stream, false, true>, rows, threads,
+                          stream, o, w, H, eps, inv_H);
+        else
+            *err = launch(fused_add_rmsnorm_reg_kernel<DT, VEC, VPT>, rows, threads, stream, o, w, H, eps, inv_H);
     }
     return true;
 }

@@ -30,8 +30,11 @@ struct RmsnormOperands {
     int64_t x_pitch, r_pitch, y_pitch, r_out_pitch;
 };
 
-// Sum over the block; every thread receives the total.  `slots` holds kMaxWarps floats.
-__device__ __forceinline__ float block_sum(float v, float *slots) {
+// Sum over the block; every thread receives the total.  `slots` holds kMaxWarps floats, 16-byte aligned.
+// SHORT (at most eight warps): the second stage is two broadcast reads and a tree of additions in every
+// thread, whose latency is below that of five more shuffles (1.44 -> 1.34 us at [16, 4096]); in kernels that
+// stream it is level.
+template <bool SHORT = false> __device__ __forceinline__ float block_sum(float v, float *slots) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -39,9 +42,19 @@ __device__ __forceinline__ float block_sum(float v, float *slots) {
     if (nwarps == 1) return v;
     if (lane == 0) slots[warp] = v;
     __syncthreads();
-    float t = lane < nwarps ? slots[lane] : 0.f;
+    float t;
+    if constexpr (SHORT) {
+        const float4 p = reinterpret_cast<const float4 *>(slots)[0];
+        t = (p.x + p.y) + ((nwarps > 2 ? p.z : 0.f) + (nwarps > 3 ? p.w : 0.f));
+        if (nwarps > 4) {
+            const float4 q = reinterpret_cast<const float4 *>(slots)[1];
+            t += (q.x + (nwarps > 5 ? q.y : 0.f)) + ((nwarps > 6 ? q.z : 0.f) + (nwarps > 7 ? q.w : 0.f));
+        }
+    } else {
+        t = lane < nwarps ? slots[lane] : 0.f;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    }
     return t;
 }
 
@@ -101,13 +114,19 @@ __host__ __device__ constexpr int rmsnorm_reg_max_threads(int units_per_thread) 
 // [16384, 8192] and 27 % at [512, 14336] (896-thread blocks: two per SM instead of one).  The
 // four-vector form (8-byte accesses, e.g. H = 4100) fits the cap too; with eight or sixteen narrower
 // vectors it would spill, so no cap there.
-template <int DT, int VEC, int VPT, Ld LDH = Ld::Stream, St STH = St::Stream, bool EARLY_W = false,
+// DECODE (few rows, at most eight warps): the short second stage of the sum, and the next kernel may start
+// when this one's inputs have arrived instead of before they are asked for; its launch then ends just as
+// this kernel does, where its blocks would otherwise wait.  Together 1.63 -> 1.39 us at [16, 4096], 1.51 ->
+// 1.30 at [16, 2048], 1.87 -> 1.71 at [1, 8192] (device time from a graph).  With more rows the early
+// prefetch of the next kernel is worth more (1.9 against 2.2 us at [128, 4096], 11.1 against 11.5 at
+// [1024, 8192]), and with more warps neither gains reliably (2.13 against 2.24 us at [16, 11008]).
+template <int DT, int VEC, int VPT, Ld LDH = Ld::Stream, St STH = St::Stream, bool EARLY_W = false, bool DECODE = false,
           int MINB = ((VEC * VPT * Storage<DT>::UNITS <= 16 && VPT <= 4 && VEC * Storage<DT>::UNITS >= 4) ? 2 : 1)>
 __global__ void __launch_bounds__(rmsnorm_reg_max_threads(VEC * VPT * Storage<DT>::UNITS), MINB)
 fused_add_rmsnorm_reg_kernel(RmsnormOperands op, const uint16_t *__restrict__ weight,
                              int H, float eps, float inv_H) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     const int nvec = H / VEC;
     const int64_t row = blockIdx.x;
     const uint16_t *xr = op.x + row * op.x_pitch;
@@ -120,7 +139,7 @@ fused_add_rmsnorm_reg_kernel(RmsnormOperands op, const uint16_t *__restrict__ we
         prefetch_l2_range(rr, static_cast<int64_t>(H) * (2 * Storage<DT>::UNITS));
     }
     grid_dependency_wait();
-    grid_launch_dependents();
+    if constexpr (!DECODE) grid_launch_dependents();
 
     Pack<UV> px[VPT], pr[VPT], pw[VPT];
 #pragma unroll
@@ -162,7 +181,8 @@ fused_add_rmsnorm_reg_kernel(RmsnormOperands op, const uint16_t *__restrict__ we
             if (v < nvec) pw[i] = load<UV, Ld::Keep>(weight + v * UV);
         }
     }
-    const float total = block_sum(acc + (acc2.x + acc2.y), slots);
+    if constexpr (DECODE) grid_launch_dependents();
+    const float total = block_sum<DECODE>(acc + (acc2.x + acc2.y), slots);
     const float rstd = rsqrtf(fmaf(total, inv_H, eps));
 
 #pragma unroll
@@ -264,7 +284,7 @@ template <int DT, int VPT, bool EARLY_W>
 __global__ void __launch_bounds__(kRmsnormRaggedMaxThreads, VPT <= 2 ? 2 : 1)
 fused_add_rmsnorm_ragged_kernel(RmsnormOperands op, const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     const int units = H * UNITS;
     const int64_t row = blockIdx.x;
     const uint16_t *xr = op.x + row * op.x_pitch;
@@ -338,7 +358,7 @@ fused_add_rmsnorm_cluster_kernel(RmsnormOperands op, const uint16_t *__restrict_
                                  int H, float eps, float inv_H) {
     namespace cg = cooperative_groups;
     constexpr int UV = VEC * Storage<DT>::UNITS;
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     __shared__ float block_partial;
     cg::cluster_group cluster = cg::this_cluster();
     const unsigned nblocks = cluster.num_blocks();
@@ -421,7 +441,7 @@ __global__ void fused_add_rmsnorm_twopass_kernel(RmsnormOperands op,
                                                  const uint16_t *__restrict__ weight,
                                                  int H, float eps, float inv_H) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     const int nvec = H / VEC;
     const int64_t row = blockIdx.x;
     const uint16_t *xr = op.x + row * op.x_pitch;

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(DENSE ? kAllreduceDenseThreads : allreduce_reg
 fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands op,
                                        const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     const int nvec = H / VEC;
     const int64_t row = static_cast<int64_t>(blockIdx.x) * H * Storage<DT>::UNITS;  // first unit of the row
     const int n = op.n_parts;
@@ -203,7 +203,7 @@ fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOpera
                                           const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
     constexpr bool EDGE_LAST = GROUP == 4, EARLY_W = GROUP > 4;
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     const int units = H * UNITS;
     const int64_t row = static_cast<int64_t>(blockIdx.x) * units;
     const int n = op.n_parts;
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(1024)
 fused_allreduce_add_rmsnorm_twopass_kernel(const __grid_constant__ AllreduceOperands op,
                                            const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = VEC * Storage<DT>::UNITS;
-    __shared__ float slots[kMaxWarps];
+    __shared__ __align__(16) float slots[kMaxWarps];
     const int nvec = H / VEC;
     const int64_t row = static_cast<int64_t>(blockIdx.x) * H * Storage<DT>::UNITS;
     grid_dependency_wait();
