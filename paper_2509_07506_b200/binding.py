@@ -1,7 +1,8 @@
 """Python binding of the C ABI in ``include/astra.h`` (argument marshalling only).
 
 Each function takes torch CUDA tensors, checks what the C side cannot see (device, dtype,
-contiguity, shapes that agree), passes raw device pointers and the current stream to
+contiguity, shapes that agree; in the ``_astra_fastcall`` extension for the ordinary case, here for
+every other and to say what is wrong), passes raw device pointers and the current stream to
 ``libastra.so`` and raises :class:`AstraError` on a non-zero status.  All arithmetic happens in
 the CUDA kernels; there is no fallback of any kind: if the shared library is missing, importing
 this module's functions raises.
@@ -98,9 +99,9 @@ _fast = None  # the _astra_fastcall extension module, once loaded
 
 def _load_fastcall(lib) -> None:
     """Import the `_astra_fastcall` extension from the package directory and give it the addresses of
-    the entry points resolved above.  It re-issues prepared calls without going through ctypes (about
-    1 us less host time per launch) and, like the library, it is required: a missing or stale module
-    is an error, not a reason to take another route."""
+    the entry points resolved above.  It issues direct calls after checking the tensors itself (see
+    ``_direct``) and re-issues prepared calls, both without going through ctypes and, like the library,
+    it is required: a missing or stale module is an error, not a reason to take another route."""
     global _fast
     try:
         from . import _astra_fastcall as fast
@@ -114,7 +115,10 @@ def _load_fastcall(lib) -> None:
                           "`python -m paper_2509_07506_b200.build`")
     for kind, fn in ((fast.KIND_RMSNORM, lib.astra_fused_add_rmsnorm), (fast.KIND_SILU, lib.astra_silu_and_mul),
                      (fast.KIND_MERGE, lib.astra_merge_attn_states_lse),
-                     (fast.KIND_ALLREDUCE_RMSNORM, lib.astra_fused_allreduce_add_rmsnorm)):
+                     (fast.KIND_ALLREDUCE_RMSNORM, lib.astra_fused_allreduce_add_rmsnorm),
+                     (fast.KIND_RMSNORM_EX, lib.astra_fused_add_rmsnorm_ex), (fast.KIND_SILU_EX, lib.astra_silu_and_mul_ex),
+                     (fast.KIND_MERGE_EX, lib.astra_merge_attn_states_lse_ex),
+                     (fast.KIND_ALLREDUCE_RMSNORM_EX, lib.astra_fused_allreduce_add_rmsnorm_ex)):
         fast.bind(kind, ctypes.cast(fn, ctypes.c_void_p).value)
     _fast = fast
 
@@ -199,14 +203,12 @@ class _on_device:
 class PreparedCall:
     """One validated call, kept ready to be issued again.
 
-    The plain functions below check every tensor, read its address and convert the arguments on
-    each call; for the small shapes of decode steps that host work takes longer than the kernel.
-    A prepared call does all of it once: it keeps the converted arguments in a C struct of the
+    The plain functions below check every tensor and read its address on each call.  A prepared call does all of it once: it keeps the converted arguments in a C struct of the
     ``_astra_fastcall`` extension (and references to the tensors, so their addresses stay valid) and
     ``__call__`` only looks up the current stream and hands the struct to the entry point, without
     ctypes in between.  The C entry point still checks every argument on every launch.  The tensors'
     contents may change between calls; their addresses, shapes and dtypes are fixed at preparation.
-    Results are identical to the plain call's, which is itself ``prepare(...)()``.
+    Results are identical to the plain call's.
     ``via_ctypes()`` issues the same call through ctypes (kept to compare the two routes).
     """
 
@@ -256,6 +258,27 @@ def _stream_of(dev: int) -> int:
 _raw_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
+def _direct(what: str, *args) -> bool:
+    """Issue a call through the extension's own checks of the tensors.  True once it has been launched;
+    False, with nothing launched, where an operand is not the ordinary case (or the library is not
+    loaded yet): the caller then takes the route below, whose checks name what is wrong."""
+    if _fast is None:
+        return False
+    st = getattr(_fast, what)(*args)
+    if st is None:
+        return False
+    if st != ASTRA_OK:
+        raise AstraError(st, _ENTRY_NAMES[what])
+    return True
+
+
+_ENTRY_NAMES = {"rmsnorm": "astra_fused_add_rmsnorm", "silu": "astra_silu_and_mul", "merge": "astra_merge_attn_states_lse",
+                "allreduce_rmsnorm": "astra_fused_allreduce_add_rmsnorm",
+                **{f"{k}_ex": f"{n}_ex" for k, n in (("rmsnorm", "astra_fused_add_rmsnorm"), ("silu", "astra_silu_and_mul"),
+                                                    ("merge", "astra_merge_attn_states_lse"),
+                                                    ("allreduce_rmsnorm", "astra_fused_allreduce_add_rmsnorm"))}}
+
+
 def _ptr(t: Optional[torch.Tensor]):
     return ctypes.c_void_p(t.data_ptr()) if t is not None else None
 
@@ -282,7 +305,8 @@ def prepare_fused_add_rmsnorm(x: torch.Tensor, residual: torch.Tensor, weight: t
 def astra_fused_add_rmsnorm(x: torch.Tensor, residual: torch.Tensor, weight: torch.Tensor,
                             eps: float, stream: Optional[torch.cuda.Stream] = None) -> None:
     """In place: residual <- x + residual, x <- RMSNorm(x + residual) * weight.  x, residual [T, H]."""
-    prepare_fused_add_rmsnorm(x, residual, weight, eps)(stream)
+    if not _direct("rmsnorm", x, residual, weight, eps, stream):
+        prepare_fused_add_rmsnorm(x, residual, weight, eps)(stream)
 
 
 def prepare_silu_and_mul(out: torch.Tensor, input: torch.Tensor) -> PreparedCall:
@@ -302,7 +326,8 @@ def prepare_silu_and_mul(out: torch.Tensor, input: torch.Tensor) -> PreparedCall
 def astra_silu_and_mul(out: torch.Tensor, input: torch.Tensor,
                        stream: Optional[torch.cuda.Stream] = None) -> None:
     """out[T, D] <- SiLU(input[:, :D]) * input[:, D:]."""
-    prepare_silu_and_mul(out, input)(stream)
+    if not _direct("silu", out, input, stream):
+        prepare_silu_and_mul(out, input)(stream)
 
 
 def prepare_merge_attn_states_lse(v_out: torch.Tensor, lse_out: Optional[torch.Tensor],
@@ -335,7 +360,8 @@ def astra_merge_attn_states_lse(v_out: torch.Tensor, lse_out: Optional[torch.Ten
                                 v_b: torch.Tensor, lse_b: torch.Tensor,
                                 stream: Optional[torch.cuda.Stream] = None) -> None:
     """v_out, lse_out <- merge of (v_a, lse_a) and (v_b, lse_b).  v_* [T, Hh, D]; lse_* [T, Hh] fp32."""
-    prepare_merge_attn_states_lse(v_out, lse_out, v_a, lse_a, v_b, lse_b)(stream)
+    if not _direct("merge", v_out, lse_out, v_a, lse_a, v_b, lse_b, stream):
+        prepare_merge_attn_states_lse(v_out, lse_out, v_a, lse_a, v_b, lse_b)(stream)
 
 
 def prepare_fused_allreduce_add_rmsnorm(y: torch.Tensor, residual: torch.Tensor, parts, weight: torch.Tensor,
@@ -371,7 +397,8 @@ def astra_fused_allreduce_add_rmsnorm(y: torch.Tensor, residual: torch.Tensor, p
     in that order in binary32 and the residual last.  The partials may live on other GPUs whose
     memory this process can address; y, residual and weight live on the GPU that runs the kernel.
     The call waits for nothing: order it after the partials have been written."""
-    prepare_fused_allreduce_add_rmsnorm(y, residual, parts, weight, eps)(stream)
+    if not _direct("allreduce_rmsnorm", y, residual, parts, weight, eps, stream):
+        prepare_fused_allreduce_add_rmsnorm(y, residual, parts, weight, eps)(stream)
 
 
 def astra_fused_allreduce_add_rmsnorm_ex(y_outs, residual_outs, residual: torch.Tensor, parts, weight: torch.Tensor,
@@ -383,6 +410,8 @@ def astra_fused_allreduce_add_rmsnorm_ex(y_outs, residual_outs, residual: torch.
     full buffers.  ``residual`` and ``weight`` live on the GPU that runs the kernel; partials and
     destinations may live on other GPUs whose memory this process can address.  The call waits for
     nothing and the destinations' owners must not read them before it has completed."""
+    if _direct("allreduce_rmsnorm_ex", y_outs, residual_outs, residual, parts, weight, eps, stream):
+        return
     parts, y_outs, residual_outs = list(parts), list(y_outs), list(residual_outs)
     _check(residual, "residual")
     code = _code(residual, "residual")
@@ -432,6 +461,8 @@ def astra_fused_add_rmsnorm_ex(y: torch.Tensor, residual_out: torch.Tensor, x: t
                                stream: Optional[torch.cuda.Stream] = None) -> None:
     """y <- RMSNorm(x + residual) * weight, residual_out <- x + residual; [T, H] tensors whose rows
     may be pitched (slices of wider buffers).  y may be x and residual_out may be residual."""
+    if _direct("rmsnorm_ex", y, residual_out, x, residual, weight, eps, stream):
+        return
     if x.dim() != 2:
         raise ValueError("x must be [T, H]")
     code = _code(x, "x")
@@ -451,6 +482,8 @@ def astra_fused_add_rmsnorm_ex(y: torch.Tensor, residual_out: torch.Tensor, x: t
 def astra_silu_and_mul_ex(out: torch.Tensor, gate: torch.Tensor, up: torch.Tensor,
                           stream: Optional[torch.cuda.Stream] = None) -> None:
     """out[T, D] <- SiLU(gate) * up with separately addressed (possibly pitched) operands."""
+    if _direct("silu_ex", out, gate, up, stream):
+        return
     if gate.dim() != 2:
         raise ValueError("gate must be [T, D]")
     code = _code(gate, "gate")
@@ -471,6 +504,8 @@ def astra_merge_attn_states_lse_ex(v_out: torch.Tensor, lse_out: Optional[torch.
                                    stream: Optional[torch.cuda.Stream] = None) -> None:
     """Merge for strided tensors: values [T, Hh, D] with D contiguous, scores [T, Hh] with any
     non-negative strides (e.g. the transposed view of a head-major [Hh, T] tensor)."""
+    if _direct("merge_ex", v_out, lse_out, v_a, lse_a, v_b, lse_b, stream):
+        return
     if v_a.dim() != 3:
         raise ValueError("v_a must be [T, Hh, D]")
     code = _code(v_a, "v_a")

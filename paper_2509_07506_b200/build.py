@@ -1,6 +1,6 @@
 """Build ``libastra.so`` (the CUDA kernels and their C ABI) for sm_100a with nvcc, the ablation
-library beside it, and ``_astra_fastcall`` (a small CPython extension that re-issues prepared calls
-without ctypes) with the host C compiler.
+library beside it, and ``_astra_fastcall`` (a small CPython extension that issues calls without ctypes
+or Python-level checks) with the host compilers.
 
 Usage: ``python -m paper_2509_07506_b200.build [--force]``.  The shared objects are written next
 to this file; nothing is installed outside the source tree.
@@ -25,7 +25,7 @@ FASTCALL_PATH = os.path.join(PKG_DIR, "_astra_fastcall.so")
 
 SOURCES = ["astra.cu", "astra_allreduce.cu"]
 ABLATION_SOURCES = ["ablation.cu"]
-FASTCALL_SOURCES = ["fastcall.c"]
+FASTCALL_SOURCES = ["fastcall.c", "torchcall.cpp"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-std=c++17", "-lineinfo",
@@ -44,7 +44,7 @@ def _nvcc() -> str:
 
 def _inputs():
     files = [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE) if f.endswith(".h")]
-    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".h", ".c"))]
+    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".h", ".c", ".cpp"))]
     return files
 
 
@@ -103,19 +103,45 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return _compile(LIB_PATH, SOURCES, force, verbose)
 
 
+def _fastcall_is_stale() -> bool:
+    """The extension reads torch's tensor objects, so it belongs to one torch release as well as to one
+    state of the sources."""
+    import torch
+    if is_stale(FASTCALL_PATH):
+        return True
+    with open(FASTCALL_PATH, "rb") as fh:
+        return b"astra-torch:" + torch.__version__.encode() + b";" not in fh.read()
+
+
 def build_fastcall(force: bool = False) -> str:
-    """Compile the _astra_fastcall extension (plain C against the CPython headers) if it is missing
-    or was built from other sources; returns its path."""
-    if not force and not is_stale(FASTCALL_PATH):
+    """Compile the _astra_fastcall extension (against the CPython and torch headers) if it is missing or
+    was built from other sources or for another torch; returns its path."""
+    if not force and not _fastcall_is_stale():
         return FASTCALL_PATH
-    cc = shutil.which("gcc") or shutil.which("cc")
-    if cc is None:
-        raise RuntimeError("no C compiler found: _astra_fastcall cannot be built")
+    import torch
+    from torch.utils import cpp_extension
+    cc, cxx = shutil.which("gcc") or shutil.which("cc"), shutil.which("g++") or shutil.which("c++")
+    if cc is None or cxx is None:
+        raise RuntimeError("no C and C++ compilers found: _astra_fastcall cannot be built")
+    common = ["-O2", "-fPIC", "-fvisibility=hidden", f'-DASTRA_BUILD_ID="{source_hash()}"',
+              f'-DASTRA_TORCH_VERSION="{torch.__version__}"', "-I", sysconfig.get_paths()["include"], "-I", INCLUDE, "-I", CSRC]
+    torch_dirs = [flag for d in cpp_extension.include_paths("cuda") for flag in ("-isystem", d)]
     tmp = FASTCALL_PATH + f".tmp{os.getpid()}"
-    cmd = [cc, "-O2", "-std=c11", "-fPIC", "-shared", "-fvisibility=hidden", f'-DASTRA_BUILD_ID="{source_hash()}"',
-           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE, "-o", tmp]
-    cmd += [os.path.join(CSRC, s) for s in FASTCALL_SOURCES]
-    subprocess.check_call(cmd)
+    objects = []
+    try:
+        for src in FASTCALL_SOURCES:
+            obj = f"{tmp}.{src}.o"
+            objects.append(obj)
+            lang = [cc, "-std=c11"] if src.endswith(".c") else [
+                cxx, "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *torch_dirs]
+            subprocess.check_call([*lang, *common, "-c", "-o", obj, os.path.join(CSRC, src)])
+        lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+        subprocess.check_call([cxx, "-shared", "-o", tmp, *objects, "-L", lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
+                               "-ltorch_python"])
+    finally:
+        for obj in objects:
+            if os.path.exists(obj):
+                os.remove(obj)
     os.replace(tmp, FASTCALL_PATH)
     return FASTCALL_PATH
 
