@@ -239,6 +239,10 @@ class PreparedCall:
         if st != ASTRA_OK:
             raise AstraError(st, self.name)
 
+    def footprint(self):
+        """``((address, bytes, is_written), ...)``: the memory a launch reads and writes."""
+        return _fast.footprint(self._ready)
+
     def via_ctypes(self, stream: Optional[torch.cuda.Stream] = None) -> None:
         """The same launch issued through ctypes instead of the extension module."""
         handle = stream.cuda_stream if stream is not None else _stream_of(self._device)

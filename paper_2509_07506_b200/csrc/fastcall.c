@@ -173,6 +173,40 @@ static PyObject *fc_launch(PyObject *self, PyObject *const *args, Py_ssize_t nar
     return PyLong_FromLong((long)st);
 }
 
+/* footprint(prepared) -> ((address, bytes, is_written), ...): the memory the call reads and writes */
+static PyObject *fc_footprint(PyObject *self, PyObject *arg) {
+    if (!Py_IS_TYPE(arg, &PreparedType)) {
+        PyErr_SetString(PyExc_TypeError, "footprint(prepared)");
+        return NULL;
+    }
+    const Prepared *p = (const Prepared *)arg;
+    const int64_t elem = p->dtype == ASTRA_FP32 ? 4 : 2;
+    const int64_t all = p->ext[0] * p->ext[1] * elem, row = p->ext[1] * elem;
+    const void *at[6 + MAX_PARTS] = {p->ptr[0], p->ptr[1], p->ptr[2], p->ptr[3], p->ptr[4], p->ptr[5]};
+    int64_t bytes[6 + MAX_PARTS] = {0};
+    int n, written = 2;  /* the first `written` pointers are outputs */
+    switch (p->kind) {
+        case KIND_SILU:
+            n = 2, written = 1, bytes[0] = all, bytes[1] = 2 * all;
+            break;
+        case KIND_MERGE:
+            n = 6, bytes[0] = bytes[2] = bytes[4] = all * p->ext[2], bytes[1] = bytes[3] = bytes[5] = p->ext[0] * p->ext[1] * 4;
+            break;
+        default:  /* the two norms; the all-reduce form has its partials besides */
+            n = 3, bytes[0] = bytes[1] = all, bytes[2] = row;
+            for (int i = 0; i < p->n_parts; ++i) at[n] = p->parts[i], bytes[n++] = all;
+            break;
+    }
+    PyObject *out = PyTuple_New(n);
+    for (int i = 0; out != NULL && i < n; ++i) {
+        PyObject *item = Py_BuildValue("(KLi)", (unsigned long long)(uintptr_t)at[i], (long long)(at[i] ? bytes[i] : 0),
+                                       i < written);
+        if (item == NULL) Py_CLEAR(out);
+        else PyTuple_SET_ITEM(out, i, item);
+    }
+    return out;
+}
+
 static PyObject *fc_build_id(PyObject *self, PyObject *noargs) {
     return PyUnicode_FromString(astra_fastcall_build_marker + sizeof("astra-build-id:") - 1);
 }
@@ -191,6 +225,7 @@ static PyMethodDef methods[] = {
     DIRECT("merge_ex", tc_merge_ex, "merge_ex(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream)"),
     DIRECT("allreduce_rmsnorm_ex", tc_allreduce_ex,
            "allreduce_rmsnorm_ex(y_outs, residual_outs, residual, parts, weight, eps, stream)"),
+    {"footprint", fc_footprint, METH_O, "footprint(prepared) -> ((address, bytes, is_written), ...)"},
     {"build_id", fc_build_id, METH_NOARGS, "hash of the sources this module was compiled from"},
     {NULL, NULL, 0, NULL},
 };

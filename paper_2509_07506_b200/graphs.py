@@ -9,17 +9,78 @@ torch's graph object is used for capture and replay: device plumbing, no arithme
 """
 from __future__ import annotations
 
-from typing import Optional, Sequence
+import bisect
+from typing import List, Optional, Sequence
 
 import torch
 
 from .binding import PreparedCall
 
+# Calls that share no memory one of them writes are captured into parallel branches, two at most.  Each call
+# of a dependent sequence is a chain of latencies (launch, first bytes, reduction, completion) that leaves
+# most of the GPU idle while it waits; a second sequence fills that time.  Measured per decode layer (norm,
+# merge, norm, activation, the norms over one residual) with 1 / 2 / 4 branches: 4.41 / 2.59 / 2.64 us at 1 token
+# of width 4096, 4.98 / 3.07 / 2.97 at 16, 9.69 / 7.16 / 7.08 at 256, 14.8 / 10.3 / 10.8 at 512, and still
+# 27.7 / 23.3 / 23.4 at 1024 and 216 / 209 / 210 at 8192 tokens, where the gain is the filled ends of the grids.
+MAX_BRANCHES = 2
+
+
+def independent_groups(footprints: Sequence[Sequence[tuple]]) -> List[int]:
+    """A group number per call (0, 1, ... in order of first appearance) such that two calls of different
+    groups touch no common byte that either of them writes.  ``footprints[i]`` lists the
+    ``(address, bytes, is_written)`` ranges of call i."""
+    parent = list(range(len(footprints)))
+
+    def root(i: int) -> int:
+        while parent[i] != i:
+            parent[i] = parent[parent[i]]
+            i = parent[i]
+        return i
+
+    # maximal runs of overlapping written ranges: everything in one run belongs together
+    starts: List[int] = []
+    ends: List[int] = []
+    owner: List[int] = []
+    for begin, size, call in sorted((a, n, i) for i, fp in enumerate(footprints) for a, n, w in fp if w and n):
+        if ends and begin < ends[-1]:
+            ends[-1] = max(ends[-1], begin + size)
+            parent[root(call)] = root(owner[-1])
+        else:
+            starts.append(begin)
+            ends.append(begin + size)
+            owner.append(call)
+    for call, fp in enumerate(footprints):
+        for begin, size, written in fp:
+            if written or not size:
+                continue
+            k = bisect.bisect_right(ends, begin)          # the first run that ends beyond the range's start
+            while k < len(starts) and starts[k] < begin + size:
+                parent[root(call)] = root(owner[k])
+                k += 1
+    number: dict = {}
+    return [number.setdefault(root(i), len(number)) for i in range(len(footprints))]
+
+
+def _branches(calls: Sequence[PreparedCall]) -> List[int]:
+    """The branch each call is captured into; all zeros (one sequence) where a call is not one of ours."""
+    if any(type(c) is not PreparedCall for c in calls):
+        return [0] * len(calls)
+    footprints = [c.footprint() for c in calls]
+    groups = independent_groups(footprints)
+    sizes = [groups.count(g) for g in range(max(groups) + 1)]
+    load, branch_of = [0] * min(MAX_BRANCHES, len(sizes)), [0] * len(sizes)
+    for g in sorted(range(len(sizes)), key=lambda g: -sizes[g]):
+        branch_of[g] = min(range(len(load)), key=load.__getitem__)
+        load[branch_of[g]] += sizes[g]
+    return [branch_of[g] for g in groups]
+
 
 class CapturedCalls:
     """``CapturedCalls([call_a, call_b, ...])`` runs the prepared calls once eagerly on a side stream
-    (so that lazy initialisation happens outside the capture), then captures them in order;
-    ``replay()`` re-issues the whole sequence on the current stream with one launch.  The tensors the
+    (so that lazy initialisation happens outside the capture), then captures them;
+    ``replay()`` re-issues the whole sequence on the current stream with one launch, with the results of
+    the calls issued in order: calls that depend on one another through a tensor stay in that order, and
+    calls that share no written memory may run at the same time.  The tensors the
     calls were prepared on are the graph's inputs and outputs.  The eager warm-up run has already
     executed every call once when the constructor returns (in-place calls such as fused_add_rmsnorm
     have then modified their operands), so fill the inputs after constructing, and refill them in
@@ -36,10 +97,16 @@ class CapturedCalls:
             for call in self.calls:       # warm-up outside the capture
                 call(side)
             side.synchronize()
+            branches = _branches(self.calls)
+            streams = [side] + [torch.cuda.Stream(self.device) for _ in range(max(branches))]
             self.graph = torch.cuda.CUDAGraph()
             with torch.cuda.graph(self.graph, stream=side):
-                for call in self.calls:
-                    call(side)
+                for s in streams[1:]:
+                    s.wait_stream(side)
+                for call, branch in zip(self.calls, branches):
+                    call(streams[branch])
+                for s in streams[1:]:
+                    side.wait_stream(s)
         torch.cuda.current_stream(self.device).wait_stream(side)
 
     def replay(self) -> None:
