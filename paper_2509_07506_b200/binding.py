@@ -100,7 +100,7 @@ _fast = None  # the _astra_fastcall extension module, once loaded
 def _load_fastcall(lib) -> None:
     """Import the `_astra_fastcall` extension from the package directory and give it the addresses of
     the entry points resolved above.  It issues direct calls after checking the tensors itself (see
-    ``_direct``) and re-issues prepared calls, both without going through ctypes and, like the library,
+    ``_raise_refusal``) and re-issues prepared calls, both without going through ctypes and, like the library,
     it is required: a missing or stale module is an error, not a reason to take another route."""
     global _fast
     try:
@@ -262,25 +262,12 @@ def _stream_of(dev: int) -> int:
 _raw_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
-def _direct(what: str, *args) -> bool:
-    """Issue a call through the extension's own checks of the tensors.  True once it has been launched;
-    False, with nothing launched, where an operand is not the ordinary case (or the library is not
-    loaded yet): the caller then takes the route below, whose checks name what is wrong."""
-    if _fast is None:
-        return False
-    st = getattr(_fast, what)(*args)
-    if st is None:
-        return False
-    if st != ASTRA_OK:
-        raise AstraError(st, _ENTRY_NAMES[what])
-    return True
-
-
-_ENTRY_NAMES = {"rmsnorm": "astra_fused_add_rmsnorm", "silu": "astra_silu_and_mul", "merge": "astra_merge_attn_states_lse",
-                "allreduce_rmsnorm": "astra_fused_allreduce_add_rmsnorm",
-                **{f"{k}_ex": f"{n}_ex" for k, n in (("rmsnorm", "astra_fused_add_rmsnorm"), ("silu", "astra_silu_and_mul"),
-                                                    ("merge", "astra_merge_attn_states_lse"),
-                                                    ("allreduce_rmsnorm", "astra_fused_allreduce_add_rmsnorm"))}}
+# A direct call goes through the extension's own checks of the tensors first.  Status 0: launched.  None, with
+# nothing launched: an operand is not the ordinary case (or the library is not loaded yet), and the route
+# below, whose checks name what is wrong, is taken.
+def _raise_refusal(st: Optional[int], name: str) -> None:
+    if st is not None:
+        raise AstraError(st, name)
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -309,7 +296,9 @@ def prepare_fused_add_rmsnorm(x: torch.Tensor, residual: torch.Tensor, weight: t
 def astra_fused_add_rmsnorm(x: torch.Tensor, residual: torch.Tensor, weight: torch.Tensor,
                             eps: float, stream: Optional[torch.cuda.Stream] = None) -> None:
     """In place: residual <- x + residual, x <- RMSNorm(x + residual) * weight.  x, residual [T, H]."""
-    if not _direct("rmsnorm", x, residual, weight, eps, stream):
+    st = _fast.rmsnorm(x, residual, weight, eps, stream) if _fast is not None else None
+    if st != ASTRA_OK:
+        _raise_refusal(st, "astra_fused_add_rmsnorm")
         prepare_fused_add_rmsnorm(x, residual, weight, eps)(stream)
 
 
@@ -330,7 +319,9 @@ def prepare_silu_and_mul(out: torch.Tensor, input: torch.Tensor) -> PreparedCall
 def astra_silu_and_mul(out: torch.Tensor, input: torch.Tensor,
                        stream: Optional[torch.cuda.Stream] = None) -> None:
     """out[T, D] <- SiLU(input[:, :D]) * input[:, D:]."""
-    if not _direct("silu", out, input, stream):
+    st = _fast.silu(out, input, stream) if _fast is not None else None
+    if st != ASTRA_OK:
+        _raise_refusal(st, "astra_silu_and_mul")
         prepare_silu_and_mul(out, input)(stream)
 
 
@@ -364,7 +355,9 @@ def astra_merge_attn_states_lse(v_out: torch.Tensor, lse_out: Optional[torch.Ten
                                 v_b: torch.Tensor, lse_b: torch.Tensor,
                                 stream: Optional[torch.cuda.Stream] = None) -> None:
     """v_out, lse_out <- merge of (v_a, lse_a) and (v_b, lse_b).  v_* [T, Hh, D]; lse_* [T, Hh] fp32."""
-    if not _direct("merge", v_out, lse_out, v_a, lse_a, v_b, lse_b, stream):
+    st = _fast.merge(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream) if _fast is not None else None
+    if st != ASTRA_OK:
+        _raise_refusal(st, "astra_merge_attn_states_lse")
         prepare_merge_attn_states_lse(v_out, lse_out, v_a, lse_a, v_b, lse_b)(stream)
 
 
@@ -401,7 +394,9 @@ def astra_fused_allreduce_add_rmsnorm(y: torch.Tensor, residual: torch.Tensor, p
     in that order in binary32 and the residual last.  The partials may live on other GPUs whose
     memory this process can address; y, residual and weight live on the GPU that runs the kernel.
     The call waits for nothing: order it after the partials have been written."""
-    if not _direct("allreduce_rmsnorm", y, residual, parts, weight, eps, stream):
+    st = _fast.allreduce_rmsnorm(y, residual, parts, weight, eps, stream) if _fast is not None else None
+    if st != ASTRA_OK:
+        _raise_refusal(st, "astra_fused_allreduce_add_rmsnorm")
         prepare_fused_allreduce_add_rmsnorm(y, residual, parts, weight, eps)(stream)
 
 
@@ -414,8 +409,10 @@ def astra_fused_allreduce_add_rmsnorm_ex(y_outs, residual_outs, residual: torch.
     full buffers.  ``residual`` and ``weight`` live on the GPU that runs the kernel; partials and
     destinations may live on other GPUs whose memory this process can address.  The call waits for
     nothing and the destinations' owners must not read them before it has completed."""
-    if _direct("allreduce_rmsnorm_ex", y_outs, residual_outs, residual, parts, weight, eps, stream):
+    st = _fast.allreduce_rmsnorm_ex(y_outs, residual_outs, residual, parts, weight, eps, stream) if _fast is not None else None
+    if st == ASTRA_OK:
         return
+    _raise_refusal(st, "astra_fused_allreduce_add_rmsnorm_ex")
     parts, y_outs, residual_outs = list(parts), list(y_outs), list(residual_outs)
     _check(residual, "residual")
     code = _code(residual, "residual")
@@ -465,8 +462,10 @@ def astra_fused_add_rmsnorm_ex(y: torch.Tensor, residual_out: torch.Tensor, x: t
                                stream: Optional[torch.cuda.Stream] = None) -> None:
     """y <- RMSNorm(x + residual) * weight, residual_out <- x + residual; [T, H] tensors whose rows
     may be pitched (slices of wider buffers).  y may be x and residual_out may be residual."""
-    if _direct("rmsnorm_ex", y, residual_out, x, residual, weight, eps, stream):
+    st = _fast.rmsnorm_ex(y, residual_out, x, residual, weight, eps, stream) if _fast is not None else None
+    if st == ASTRA_OK:
         return
+    _raise_refusal(st, "astra_fused_add_rmsnorm_ex")
     if x.dim() != 2:
         raise ValueError("x must be [T, H]")
     code = _code(x, "x")
@@ -486,8 +485,10 @@ def astra_fused_add_rmsnorm_ex(y: torch.Tensor, residual_out: torch.Tensor, x: t
 def astra_silu_and_mul_ex(out: torch.Tensor, gate: torch.Tensor, up: torch.Tensor,
                           stream: Optional[torch.cuda.Stream] = None) -> None:
     """out[T, D] <- SiLU(gate) * up with separately addressed (possibly pitched) operands."""
-    if _direct("silu_ex", out, gate, up, stream):
+    st = _fast.silu_ex(out, gate, up, stream) if _fast is not None else None
+    if st == ASTRA_OK:
         return
+    _raise_refusal(st, "astra_silu_and_mul_ex")
     if gate.dim() != 2:
         raise ValueError("gate must be [T, D]")
     code = _code(gate, "gate")
@@ -508,8 +509,10 @@ def astra_merge_attn_states_lse_ex(v_out: torch.Tensor, lse_out: Optional[torch.
                                    stream: Optional[torch.cuda.Stream] = None) -> None:
     """Merge for strided tensors: values [T, Hh, D] with D contiguous, scores [T, Hh] with any
     non-negative strides (e.g. the transposed view of a head-major [Hh, T] tensor)."""
-    if _direct("merge_ex", v_out, lse_out, v_a, lse_a, v_b, lse_b, stream):
+    st = _fast.merge_ex(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream) if _fast is not None else None
+    if st == ASTRA_OK:
         return
+    _raise_refusal(st, "astra_merge_attn_states_lse_ex")
     if v_a.dim() != 3:
         raise ValueError("v_a must be [T, Hh, D]")
     code = _code(v_a, "v_a")
