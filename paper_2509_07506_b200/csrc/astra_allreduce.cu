@@ -21,10 +21,19 @@ constexpr int kDeepGroup = 8;    // and few rows
 // UVEC is the vector width in units, VPT the vectors per thread.
 // `dense` selects the instantiation whose registers are capped so that five 256-thread blocks fit an
 // SM; it exists for the streaming shape (two loads in flight, 16 units per thread) only.
-template <int DT, int UVEC, int VPT, int GROUP>
+// `LATE_R`: two 32-byte vectors, the residual requested last.
+template <int DT, int UVEC, int VPT, int GROUP, bool LATE_R = false>
 cudaError_t launch_reg(const AllreduceOperands &op, const uint16_t *w, unsigned rows, int threads, int H,
                        float eps, float inv_H, bool dense, cudaStream_t stream) {
-    if constexpr (UVEC >= 4 && UVEC >= Storage<DT>::UNITS && UVEC * VPT <= 32) {
+    if constexpr (LATE_R) {
+        if constexpr (UVEC == 16 && VPT == 2)
+            return launch(fused_allreduce_add_rmsnorm_reg_kernel<DT, UVEC / Storage<DT>::UNITS, VPT, GROUP, false, true>, rows,
+                          threads, stream, op, w, H, eps, inv_H);
+    } else if constexpr (GROUP == 1) {  // wide binary32 rows only
+        if constexpr (DT == ASTRA_FP32 && UVEC == 16 && VPT == 4)
+            return launch(fused_allreduce_add_rmsnorm_reg_kernel<DT, UVEC / Storage<DT>::UNITS, VPT, GROUP>, rows, threads,
+                          stream, op, w, H, eps, inv_H);
+    } else if constexpr (UVEC >= 4 && UVEC >= Storage<DT>::UNITS && UVEC * VPT <= 32) {
         if constexpr (GROUP == 2 && UVEC == 8 && VPT == 2) {  // the measured case: 16-byte vectors, no spill at 48 registers
             if (dense && threads <= kAllreduceDenseThreads)
                 return launch(fused_allreduce_add_rmsnorm_reg_kernel<DT, UVEC / Storage<DT>::UNITS, VPT, GROUP, true>,
@@ -72,17 +81,20 @@ inline int pick_vpt(int nvec, int start_units, int *threads_out) {
     return vpt;
 }
 
-// The ragged kernel (rows that start anywhere): 32-byte vectors, one or two per thread.
-template <int DT, int UVEC, int VPT, int GROUP>
+// The ragged kernel (rows that start anywhere): 32-byte vectors, as many per thread as above.
+template <int DT, int UVEC, int VPT, int GROUP, bool LATE_R>
 cudaError_t launch_ragged(const AllreduceOperands &op, const uint16_t *w, unsigned rows, int threads, int H, float eps,
                           float inv_H, cudaStream_t stream) {
-    if constexpr (UVEC == 16 && VPT <= 2 && !(GROUP == kDeepGroup && VPT > 1))
-        return launch(fused_allreduce_add_rmsnorm_ragged_kernel<DT, VPT, GROUP>, rows, threads, stream, op, w, H, eps, inv_H);
+    constexpr bool built = LATE_R ? VPT == 2 : GROUP == 1 ? VPT == 4 && DT == ASTRA_FP32
+                                             : GROUP == kDeepGroup ? VPT == 1 : VPT <= 2;
+    if constexpr (UVEC == 16 && built)
+        return launch(fused_allreduce_add_rmsnorm_ragged_kernel<DT, VPT, GROUP, LATE_R>, rows, threads, stream, op, w, H, eps,
+                      inv_H);
     return cudaErrorInvalidValue;
 }
 
 // Launches over all rows (split where the grid limit requires).  vpt = 0 selects the two-sweep kernel.
-template <int DT, int UVEC, int GROUP, bool RAGGED = false>
+template <int DT, int UVEC, int GROUP, bool RAGGED = false, bool LATE_R = false>
 cudaError_t launch_rows(AllreduceOperands op, const uint16_t *w, int64_t T, int H, float eps, int vpt,
                         int threads, cudaStream_t stream) {
   if constexpr (UVEC >= Storage<DT>::UNITS) {
@@ -105,8 +117,15 @@ cudaError_t launch_rows(AllreduceOperands op, const uint16_t *w, int64_t T, int 
         o.r += t0 * row_units;
         cudaError_t err;
         if constexpr (RAGGED) {
-            err = vpt == 1 ? launch_ragged<DT, UVEC, 1, GROUP>(o, w, rows, threads, H, eps, inv_H, stream)
-                           : launch_ragged<DT, UVEC, 2, GROUP>(o, w, rows, threads, H, eps, inv_H, stream);
+            err = vpt == 1   ? launch_ragged<DT, UVEC, 1, GROUP, LATE_R>(o, w, rows, threads, H, eps, inv_H, stream)
+                  : vpt == 2 ? launch_ragged<DT, UVEC, 2, GROUP, LATE_R>(o, w, rows, threads, H, eps, inv_H, stream)
+                             : launch_ragged<DT, UVEC, 4, GROUP, LATE_R>(o, w, rows, threads, H, eps, inv_H, stream);
+            if (err != cudaSuccess) return err;
+            continue;
+        }
+        if constexpr (LATE_R || GROUP == 1) {
+            err = vpt == 2 ? launch_reg<DT, UVEC, 2, GROUP, LATE_R>(o, w, rows, threads, H, eps, inv_H, dense, stream)
+                           : launch_reg<DT, UVEC, 4, GROUP, LATE_R>(o, w, rows, threads, H, eps, inv_H, dense, stream);
             if (err != cudaSuccess) return err;
             continue;
         }
@@ -145,30 +164,43 @@ cudaError_t choose_shape(const AllreduceOperands &op, const uint16_t *w, int64_t
 // against the 16-byte form at [8192, 4096]: 50.6 -> 49.2 us with 2 partials, 70.8 -> 66.6 us with 4,
 // 110.9 -> 104.7 us with 8; at [1024, 4096]: 8.3 -> 7.7, 10.9 -> 10.3, 16.2 -> 15.9 us.
 //
-// Four shapes: one or two vectors per thread (16 or 32 units), two or four partial loads in flight
-// (four only from four partials on).  What decides between them is how many bytes of loads an SM has
-// in flight, i.e. resident blocks x threads x bytes per thread, with the resident blocks set by the
-// registers (56 / 96 / 72 / 128 per thread as compiled for sm_100a, allocated in eights, 65536 per
-// SM).  The measurements across H = 2048 ... 16384 fit one rule: take the first shape, in the order
-// below, that keeps about 90 KB in flight per SM; if none does, the one with the most.  Examples:
+// Five shapes: one or two vectors per thread (16 or 32 units), two or four partial loads in flight
+// (four only from four partials on), and two of each with the residual requested last.  What decides
+// between them is how many bytes of loads an SM has in flight, i.e. resident blocks x threads x bytes per
+// thread, with the resident blocks set by the registers (as compiled for sm_100a, allocated in eights,
+// 65536 per SM).  The measurements across H = 2048 ... 16384 fit one rule: take the first shape, in the
+// order below, that keeps about 90 KB in flight per SM; if none does, the one with the most.  Examples:
 // H = 4096 takes one vector and four in flight (three 256-thread blocks per SM); H = 8192 with four
 // in flight would leave one 512-thread block per SM, so it takes two vectors in 256-thread blocks
 // (78.8 -> 68.0 us with 4 partials, 117.3 -> 105.6 us with 8); H = 10240 with two in flight takes two
 // vectors in 320-thread blocks (two per SM) rather than one 640-thread block (61.6 against 76.7 us);
-// H = 16384 takes one vector in one 1024-thread block (143.1 against 155.8 us with 4 partials).
+// H = 11008 ... 14336 take the late residual (79.7 -> 67.9 us at [4096, 11008] with 2 partials, more at the
+// kernel; but 2.7 against 3.2 us at [16, 11008], where every SM has one row at most); H = 16384 takes one vector in one 1024-thread block (143.1 against 155.8 us with 4 partials).
+// Binary32 rows need fewer registers (5120 elements take one vector in two 640-thread blocks: 25.1 -> 23.1 us at
+// [1024, 5120] with 4 partials).
+// Binary32 rows of more than 16384 units take four vectors per thread, one load in flight, in one block
+// of up to 512 threads per SM, instead of two sweeps: 73.5 -> 52.6, 105.8 -> 73.5, 191 -> 112.5 us at [1024, 16384]
+// with 2 / 4 / 8 partials (48.6 / 68.1 / 107 us at 6.9 TB/s), 17.5 -> 9.5 us at [16, 16384] with 8.
 // Returns false where no shape applies (rows too narrow for 128-thread blocks, or too wide).
 struct WideShape {
     int vpt, group, regs, max_threads, min_threads;
+    bool late = false;  // the residual is requested after the partials
 };
 #ifndef ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS
 #define ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS 128
 #endif
 constexpr int64_t kDeepQueueRows = ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS;
-constexpr WideShape kWideShapes[] = {
-    {1, 4, 72, 512, 128}, {2, 4, 128, 256, 64}, {1, 2, 56, 1024, 128}, {2, 2, 96, 512, 64}};
-// The same shapes of the ragged kernel, with its registers (the last one takes fewer for binary32).
-template <int DT> constexpr WideShape kRaggedShapes[] = {
-    {1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, DT == ASTRA_FP32 ? 96 : 120, 512, 64}};
+constexpr int64_t kOneBlockRows = 148;  // rows up to which every SM of a B200 has one block at most
+constexpr int kWideShapeCount = 5;
+template <int DT> constexpr WideShape kWideShapes[kWideShapeCount] = {
+    {1, 4, 72, 512, 128}, {2, 4, 128, 256, 64}, {1, 2, 56, 1024, 128}, {2, 2, 96, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}};
+template <> constexpr WideShape kWideShapes<ASTRA_FP32>[kWideShapeCount] = {
+    {1, 4, 64, 512, 128}, {2, 4, 112, 256, 64}, {1, 2, 48, 1024, 128}, {2, 2, 80, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}};
+// The same shapes of the ragged kernel, with its registers.
+template <int DT> constexpr WideShape kRaggedShapes[kWideShapeCount] = {
+    {1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 120, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}};
+template <> constexpr WideShape kRaggedShapes<ASTRA_FP32>[kWideShapeCount] = {
+    {1, 4, 64, 512, 64}, {2, 4, 120, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 96, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}};
 constexpr int64_t kWideBytesInFlight = 90 * 1024;
 
 template <int DT, bool RAGGED>
@@ -192,14 +224,15 @@ bool launch_wide(const AllreduceOperands &op, const uint16_t *w, int64_t T, int 
     }
     int best = -1, best_threads = 0;
     int64_t best_bytes = 0;
-    for (int c = 0; c < 4; ++c) {
-        const WideShape &sh = RAGGED ? kRaggedShapes<DT>[c] : kWideShapes[c];
+    for (int c = 0; c < kWideShapeCount; ++c) {
+        const WideShape &sh = RAGGED ? kRaggedShapes<DT>[c] : kWideShapes<DT>[c];
         if (sh.group > kStreamGroup && op.n_parts < sh.group) continue;
+        if (sh.late && T <= kOneBlockRows) continue;  // a second block per SM has no row to work on then
         const int threads = round_up_to((nvec + sh.vpt - 1) / sh.vpt, 32);
         if (threads > sh.max_threads || threads < sh.min_threads) continue;
         const int by_regs = 65536 / (sh.regs * threads), by_threads = 2048 / threads;
         const int blocks = by_regs < by_threads ? by_regs : by_threads;
-        const int64_t bytes = static_cast<int64_t>(blocks) * threads * sh.vpt * (sh.group + 1) * 32;
+        const int64_t bytes = static_cast<int64_t>(blocks) * threads * sh.vpt * (sh.group + (sh.late ? 0 : 1)) * 32;
         if (bytes > best_bytes) {
             best = c;
             best_bytes = bytes;
@@ -207,9 +240,20 @@ bool launch_wide(const AllreduceOperands &op, const uint16_t *w, int64_t T, int 
         }
         if (bytes >= kWideBytesInFlight) break;  // the first shape that reaches it is also the largest so far
     }
-    if (best < 0) return false;
-    const WideShape &sh = RAGGED ? kRaggedShapes<DT>[best] : kWideShapes[best];
-    if (sh.group == 4)
+    if (best < 0) {
+        if constexpr (DT == ASTRA_FP32) {
+            const int threads = round_up_to((nvec + 3) / 4, 32);
+            if (nvec > 1024 && threads <= allreduce_reg_max_threads(64, 1)) {
+                *err = launch_rows<DT, UVEC, 1, RAGGED>(op, w, T, H, eps, 4, threads, stream);
+                return true;
+            }
+        }
+        return false;
+    }
+    const WideShape &sh = RAGGED ? kRaggedShapes<DT>[best] : kWideShapes<DT>[best];
+    if (sh.late)
+        *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED, true>(op, w, T, H, eps, sh.vpt, best_threads, stream);
+    else if (sh.group == 4)
         *err = launch_rows<DT, UVEC, 4, RAGGED>(op, w, T, H, eps, sh.vpt, best_threads, stream);
     else
         *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED>(op, w, T, H, eps, sh.vpt, best_threads, stream);
@@ -241,14 +285,16 @@ cudaError_t dispatch(const AllreduceOperands &op, const uint16_t *w, int64_t T, 
     }
     // Rows of less than 16-byte alignment go to the ragged kernel (figures there), except where the 8-byte
     // forms are the faster ones: few rows, whose latency their smaller code serves better (1.8 against 2.1 us
-    // at [16, 4100] with 2 partials, 3.3 against 4.2 us at [140, 4100] with 4, 4.35 against 4.6 us at [64, 8188] with 8; but 7.5 -> 6.1 us at [16, 14332]
-    // with 8, 5.8 -> 3.8 us at fp32 [16, 4098]), two or three partials up to 512 rows (4.05 against 4.5 us at
-    // [400, 4100]; 9.1 -> 7.1 us at [512, 4100] with 4), and binary32 rows of more than 10240 units, where
-    // one block per SM is left (41.2 against 45.9 us at fp32 [1024, 8190] with 4; 27.5 -> 13.2 us at [512, 5001]).
+    // at [16, 4100] with 2 partials, 3.3 against 4.2 us at [140, 4100] with 4, 4.35 against 4.6 us at [64, 8188]
+    // with 8; but 7.5 -> 6.1 us at [16, 14332] with 8, 5.8 -> 3.8 us at fp32 [16, 4098]), two or three partials
+    // up to 512 rows (4.05 against 4.5 us at [400, 4100]; 9.1 -> 7.1 us at [512, 4100] with 4), and binary32 rows
+    // of 10241 to 16384 units (41.2 against 45.9 us at fp32 [1024, 8190] with 4; 27.5 -> 13.2 us at [512, 5001]
+    // and 130 -> 80 us at [1024, 16382], which take two sweeps otherwise).
     const int64_t units = static_cast<int64_t>(H) * Storage<DT>::UNITS;
-    const bool few = T <= 148;  // a block per SM at most
-    const bool narrow_form = pick.vec == 4 && (DT == ASTRA_FP32 ? units > 10240 || (op.n_parts < 4 && few)
-                                                                : (op.n_parts < 4 && T <= 512) || (units <= 8192 && few));
+    const bool few = T <= kOneBlockRows;
+    const bool narrow_form =
+        pick.vec == 4 && (DT == ASTRA_FP32 ? (units > 10240 && units <= 16384) || (op.n_parts < 4 && few && units <= 16384)
+                                           : (op.n_parts < 4 && T <= 512) || (units <= 8192 && few));
     if (pick.vec < 8 && !narrow_form && rows_together(op)) {
         cudaError_t err = cudaSuccess;
         if (launch_wide<DT, true>(op, w, T, H, eps, stream, &err)) return err;

@@ -74,8 +74,10 @@ __device__ __forceinline__ void accumulate(float (&s)[VEC], const float (&x)[VEC
 // fits; that matters for rows of more than 8192 units, where one fat block per SM with one vector per
 // thread beat two vectors per thread in half as many threads by 3 to 9 % (e.g. 157.9 -> 143.1 us at
 // [4096, 16384] with 4 partials, 82.2 -> 77.4 us at [4096, 11008] with 2).
+// One load in flight serves binary32 rows of up to 64 units per thread (32 sums).
 __host__ __device__ constexpr int allreduce_reg_max_threads(int units, int group) {
-    return group > 4 ? (units <= 16 ? 512 : 128)
+    return group == 1 ? 512
+         : group > 4 ? (units <= 16 ? 512 : 128)
          : group > 2 ? (units <= 8 ? 1024 : (units <= 16 ? 512 : 256))
                      : (units <= 16 ? 1024 : 512);
 }
@@ -91,9 +93,20 @@ __host__ __device__ constexpr int allreduce_reg_max_threads(int units, int group
 constexpr int kAllreduceDenseThreads = 256;
 constexpr int kAllreduceDenseBlocks = 5;
 
-template <int DT, int VEC, int VPT, int GROUP, bool DENSE = false>
-__global__ void __launch_bounds__(DENSE ? kAllreduceDenseThreads : allreduce_reg_max_threads(VEC * VPT * Storage<DT>::UNITS, GROUP),
-                                  DENSE ? kAllreduceDenseBlocks : 1)
+//
+// LATE_R requests the residual after the partials instead of with the first of them, which frees its
+// registers while they are summed: two vectors per thread with two partial loads in flight then take 72
+// registers instead of 96 and two blocks of up to 448 threads fit an SM instead of one.  For rows of 10241
+// to 14336 units, where every other shape leaves one block per SM that idles at its barrier, L2-cold, with
+// 2 / 4 / 8 partials: 79.7 -> 67.9, 112.7 -> 92.2, 171.0 -> 145.3 us at [4096, 11008] (65.4 / 91.5 / 143.8 us at
+// 6.9 TB/s) and 93.2 -> 86.1, 133.2 -> 119.4, 203.5 -> 188.2 us at [4096, 14336]; no gain where two blocks fit
+// anyway (61.1 against 62.8 us at [4096, 10240]).
+constexpr int kAllreduceLateThreads = 448;
+
+template <int DT, int VEC, int VPT, int GROUP, bool DENSE = false, bool LATE_R = false>
+__global__ void __launch_bounds__(LATE_R ? kAllreduceLateThreads : DENSE ? kAllreduceDenseThreads
+                                                                  : allreduce_reg_max_threads(VEC * VPT * Storage<DT>::UNITS, GROUP),
+                                  LATE_R ? 2 : DENSE ? kAllreduceDenseBlocks : 1)
 fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands op,
                                        const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
@@ -108,12 +121,16 @@ fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands
     grid_launch_dependents();
 
     // the residual is consumed last but requested first, together with the first group of partials
+    // (LATE_R: after the last one)
     Pack<UV> pr[VPT];
+    auto fetch_residual = [&] {
 #pragma unroll
-    for (int i = 0; i < VPT; ++i) {
-        const int v = threadIdx.x + i * blockDim.x;
-        if (v < nvec) pr[i] = load<UV, Ld::Stream>(op.r + row + v * UV);
-    }
+        for (int i = 0; i < VPT; ++i) {
+            const int v = threadIdx.x + i * blockDim.x;
+            if (v < nvec) pr[i] = load<UV, Ld::Stream>(op.r + row + v * UV);
+        }
+    };
+    if constexpr (!LATE_R) fetch_residual();
 
     // The loop over groups is unrolled to the largest supported count and left by a break: every copy
     // then has a constant p0 (the first one initialises the sums without a test) and the compiler may
@@ -157,6 +174,7 @@ fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands
         }
     }
 
+    if constexpr (LATE_R) fetch_residual();
     float acc = 0.f;
     float2 acc2 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -197,12 +215,13 @@ fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands
 // are fetched group by group beside the body's.  (The plain loads and stores stay per-thread here too: a
 // partial or a destination may be another GPU's memory.)
 // Measured L2-cold, bf16, against the 2-, 4- and 8-byte vector kernels: see the launch code.
-template <int DT, int VPT, int GROUP>
-__global__ void __launch_bounds__(allreduce_reg_max_threads(16 * VPT, GROUP))
+template <int DT, int VPT, int GROUP, bool LATE_R = false>
+__global__ void __launch_bounds__(LATE_R ? kAllreduceLateThreads : VPT == 4 ? 512 : allreduce_reg_max_threads(16 * VPT, GROUP),
+                                  LATE_R ? 2 : 1)
 fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOperands op,
                                           const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
-    constexpr bool EDGE_LAST = GROUP == 4, EARLY_W = GROUP > 4;
+    constexpr bool EDGE_LAST = GROUP == 4 || GROUP == 1 || LATE_R, EARLY_W = GROUP > 4;
     __shared__ __align__(16) float slots[kMaxWarps];
     const int units = H * UNITS;
     const int64_t row = static_cast<int64_t>(blockIdx.x) * units;
@@ -215,11 +234,14 @@ fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOpera
 
     Pack<UV> pr[VPT];
     Pack<UNITS> er, ew;
+    auto fetch_residual = [&] {
 #pragma unroll
-    for (int i = 0; i < VPT; ++i) {
-        const int v = threadIdx.x + i * blockDim.x;
-        if (v < g.nvec) pr[i] = load<UV, Ld::Stream>(op.r + body + v * UV);
-    }
+        for (int i = 0; i < VPT; ++i) {
+            const int v = threadIdx.x + i * blockDim.x;
+            if (v < g.nvec) pr[i] = load<UV, Ld::Stream>(op.r + body + v * UV);
+        }
+    };
+    if constexpr (!LATE_R) fetch_residual();
     if (!EDGE_LAST && g.edge >= 0) {
         er = load<UNITS, Ld::Stream>(op.r + row + g.edge);
         ew = load<UNITS, Ld::Keep>(weight + g.edge);
@@ -269,6 +291,7 @@ fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOpera
         }
     }
 
+    if constexpr (LATE_R) fetch_residual();
     float acc = 0.f;
     float2 acc2 = make_float2(0.f, 0.f);
 #pragma unroll

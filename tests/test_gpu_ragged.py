@@ -68,3 +68,17 @@ def test_rmsnorm_ragged_pitches(pads):
 @pytest.mark.parametrize("T,H,offset", [(3, 2049, 0), (16, 4099, 1), (129, 2051, 6), (9, 8189, 15), (5, 16383, 0), (4, 1027, 3)])
 def test_allreduce_rmsnorm_ragged_rows(n_parts, T, H, offset, dtype):
     run_allreduce(wl.allreduce_rmsnorm_inputs(T, H, n_parts, dtype, seed=H + n_parts), offset=offset)
+
+
+@pytest.mark.parametrize("n_parts", [2, 8])
+@pytest.mark.parametrize("T,H,dtype,offset", [(150, 10256, BF16, 0), (149, 11008, FP16, 0), (151, 14336, BF16, 0), (150, 14335, BF16, 0),
+                                              (150, 5632, FP32, 0), (3, 8200, FP32, 0), (2, 16384, FP32, 0), (3, 16383, FP32, 2)])
+def test_allreduce_rmsnorm_wide_rows(n_parts, T, H, dtype, offset):
+    """Rows whose residual is requested last (10241 to 14336 units, more rows than SMs) and binary32 rows of
+    more than 16384 units, aligned and not."""
+    run_allreduce(wl.allreduce_rmsnorm_inputs(T, H, n_parts, dtype, seed=H + n_parts), offset=offset)
+
+
+@pytest.mark.parametrize("T,H", [(65, 8200), (64, 8200), (66, 16384), (65, 11008)])
+def test_rmsnorm_wide_aligned_fp32_rows(T, H):
+    run_rmsnorm(wl.rmsnorm_inputs(T, H, FP32, eps=1e-5, seed=H + T))
