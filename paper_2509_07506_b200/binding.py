@@ -113,6 +113,9 @@ def _load_fastcall(lib) -> None:
     if os.path.isdir(_build.CSRC) and os.path.isdir(_build.INCLUDE) and fast.build_id() != _build.source_hash():
         raise ImportError(f"{FASTCALL_PATH} was built from other sources: rebuild it with "
                           "`python -m paper_2509_07506_b200.build`")
+    if fast.torch_version() != torch.__version__:  # it reads torch's tensor objects
+        raise ImportError(f"{FASTCALL_PATH} was built for torch {fast.torch_version()}, this is {torch.__version__}: rebuild "
+                          "it with `python -m paper_2509_07506_b200.build`")
     for kind, fn in ((fast.KIND_RMSNORM, lib.astra_fused_add_rmsnorm), (fast.KIND_SILU, lib.astra_silu_and_mul),
                      (fast.KIND_MERGE, lib.astra_merge_attn_states_lse),
                      (fast.KIND_ALLREDUCE_RMSNORM, lib.astra_fused_allreduce_add_rmsnorm),

@@ -211,6 +211,11 @@ static PyObject *fc_build_id(PyObject *self, PyObject *noargs) {
     return PyUnicode_FromString(astra_fastcall_build_marker + sizeof("astra-build-id:") - 1);
 }
 
+static PyObject *fc_torch_version(PyObject *self, PyObject *noargs) {
+    const char *v = astra_torch_marker + sizeof("astra-torch:") - 1;
+    return PyUnicode_FromStringAndSize(v, (Py_ssize_t)strlen(v) - 1);
+}
+
 static PyMethodDef methods[] = {
     {"bind", fc_bind, METH_VARARGS, "bind(kind, address): set the entry point of one kind of call"},
     {"prepare", fc_prepare, METH_VARARGS, "prepare(kind, pointers, extents, eps, dtype, parts) -> Prepared"},
@@ -227,6 +232,7 @@ static PyMethodDef methods[] = {
            "allreduce_rmsnorm_ex(y_outs, residual_outs, residual, parts, weight, eps, stream)"),
     {"footprint", fc_footprint, METH_O, "footprint(prepared) -> ((address, bytes, is_written), ...)"},
     {"build_id", fc_build_id, METH_NOARGS, "hash of the sources this module was compiled from"},
+    {"torch_version", fc_torch_version, METH_NOARGS, "torch release this module was compiled against"},
     {NULL, NULL, 0, NULL},
 };
 

@@ -21,6 +21,7 @@ extern "C" {
 #endif
 
 extern void *astra_entry_points[KIND_COUNT];
+extern const char astra_torch_marker[];  /* "astra-torch:<release>;" */
 
 PyObject *tc_rmsnorm(PyObject *, PyObject *const *, Py_ssize_t);
 PyObject *tc_silu(PyObject *, PyObject *const *, Py_ssize_t);

@@ -326,7 +326,6 @@ PyObject *tc_merge_ex(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
 }
 
 // The torch release this file was compiled against; the build script finds it in the built file.
-extern const char astra_torch_marker[];
 __attribute__((used)) const char astra_torch_marker[] = "astra-torch:" ASTRA_TORCH_VERSION ";";
 
 }  // extern "C"
