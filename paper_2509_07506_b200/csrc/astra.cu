@@ -416,7 +416,7 @@ bool launch_rmsnorm_wide(const RmsnormOperands &op, const uint16_t *w, int64_t T
 #ifndef ASTRA_RMSNORM_RAGGED_MIN_UNITS
 #define ASTRA_RMSNORM_RAGGED_MIN_UNITS 1024
 #endif
-constexpr int64_t kRmsnormRaggedMinUnits = ASTRA_RMSNORM_RAGGED_MIN_UNITS;  // at least 64 threads with one vector each
+constexpr int64_t kRmsnormRaggedMinUnits = ASTRA_RMSNORM_RAGGED_MIN_UNITS;
 
 template <int DT, int VPT, bool EARLY_W>
 cudaError_t launch_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T, int H, int threads, float eps,
@@ -436,14 +436,7 @@ cudaError_t launch_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, 
     return cudaSuccess;
 }
 
-// False where the ragged kernel does not apply.  One vector per thread up to 320 threads, then two (up to
-// 512 threads), then, for binary32 rows only (half the sums per unit), four: 21.3 us with one and 21.6 with two
-// at [4096, 4099], 45.1 and 41.4 us at [4096, 8188], 39.2 and 28.8 us at [2048, 11007].  Two also where that
-// makes one wave of what would be a little more (5 blocks of 256 threads per SM at 48 registers against 8
-// of 128 at 64: 6.8 -> 6.6 us at [1024, 4101]).  A few wide rows of 8-byte vectors are left to the clusters,
-// which spread each over several SMs (3.1 against 4.9 us at fp32 [16, 16382], 4.9 and 5.1 at 64 rows, 9.5 and
-// 6.5 at 128).
-constexpr int64_t kRmsnormRaggedWideRows = 64;
+// False where the ragged kernel does not apply.
 template <int DT>
 bool try_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T, int H, int vec, float eps,
                         cudaStream_t stream, cudaError_t *err) {
@@ -454,13 +447,11 @@ bool try_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T,
                           (reinterpret_cast<uintptr_t>(op.y) - at) % 32 == 0 &&
                           (reinterpret_cast<uintptr_t>(op.r_out) - at) % 32 == 0;
     if (!together || Hu < kRmsnormRaggedMinUnits) return false;
-    const int64_t nvec = Hu / 16;
-    auto threads_for = [&](int v) { const int64_t t = (nvec + v - 1) / v; return static_cast<int>((t + 31) / 32 * 32); };
-    const int64_t wave1 = 148 * (65536 / (48 * threads_for(1))), wave2 = 148 * (65536 / (64 * threads_for(2)));
-    if (nvec <= 320 && !(T > wave1 && T <= wave2)) *err = launch_rmsnorm_ragged<DT, 1, true>(op, w, T, H, threads_for(1), eps, stream);
-    else if (nvec <= 2 * kRmsnormRaggedMaxThreads) *err = launch_rmsnorm_ragged<DT, 2, false>(op, w, T, H, threads_for(2), eps, stream);
-    else if (DT == ASTRA_FP32 && nvec <= 4 * kRmsnormRaggedMaxThreads && !(vec == 4 && T <= kRmsnormRaggedWideRows)) {
-        if constexpr (DT == ASTRA_FP32) *err = launch_rmsnorm_ragged<DT, 4, false>(op, w, T, H, threads_for(4), eps, stream);
+    const RaggedShape sh = rmsnorm_ragged_shape(T, Hu, DT == ASTRA_FP32, vec == 4);
+    if (sh.vpt == 1) *err = launch_rmsnorm_ragged<DT, 1, true>(op, w, T, H, sh.threads, eps, stream);
+    else if (sh.vpt == 2) *err = launch_rmsnorm_ragged<DT, 2, false>(op, w, T, H, sh.threads, eps, stream);
+    else if (sh.vpt == 4) {
+        if constexpr (DT == ASTRA_FP32) *err = launch_rmsnorm_ragged<DT, 4, false>(op, w, T, H, sh.threads, eps, stream);
     } else return false;
     return true;
 }

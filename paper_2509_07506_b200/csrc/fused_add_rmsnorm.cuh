@@ -200,7 +200,7 @@ fused_add_rmsnorm_reg_kernel(RmsnormOperands op, const uint16_t *__restrict__ we
 // ---------------------------------------------------------------------------------------------
 // Rows that start at any element (odd widths): x, residual and the outputs start at the same place within
 // a 32-byte granule, row by row, so the granules that lie inside the row (its body) are 32-byte accesses
-// of all four; the few units before and after them (the edge, at most 61) are one element per lane of the
+// of all four; the few units before and after them (the edge, at most 46) are one element per lane of the
 // first two warps.  Only the weight, which starts the same way for every row, lies at an offset to them:
 // its two granules per body vector are loaded whole and shifted, by an amount that is the row's.
 // ---------------------------------------------------------------------------------------------
@@ -210,8 +210,8 @@ struct RaggedRow {
     int edge;         // this thread's edge unit, or -1
 };
 
-// The share of thread `thread` of a row of `units` units at `row`.  Body vectors whose weight granules would pass the weight's ends are left
-// to the edge: at most 31 units before the body and 30 after it.
+// The share of thread `thread` of a row of `units` units at `row`.  Body vectors whose weight granules would pass
+// the weight's ends are left to the edge: at most 30 units before the body or 30 after it, 46 together.
 template <int UNITS>
 __host__ __device__ __forceinline__ RaggedRow ragged_row(const uint16_t *row, const uint16_t *weight, int units, int thread) {
     constexpr int UV = 16;
@@ -271,7 +271,7 @@ __device__ __forceinline__ void ragged_finish(const RaggedRow &g, const uint16_t
 
 // HBM-bound like the aligned kernel, of which it moves the same bytes in the same widths; what it pays for
 // the row's place is the second weight granule, a funnel shift per word of weight and two warps' edge.
-// Launched with at least 64 threads (the edge), VPT vectors per thread covering units / 16 of them.
+// Launched with rmsnorm_ragged_shape's blocks, VPT vectors per thread covering units / 16 of them.
 // Measured L2-cold, fp16, against the kernels for 2-, 4- and 8-byte vectors: 41.8 -> 21.3 us at [4096, 4099]
 // (19.5 us at 6.9 TB/s), 99.4 -> 28.8 us at [2048, 11007], 142 -> 41.0 us at [2048, 16383], 12.3 -> 6.9 us at
 // [1024, 4101], 2.9 -> 2.0 us at [16, 4099], 25.0 -> 21.3 us at [4096, 4098], 79.7 -> 78.8 us at [16384, 4100];
@@ -279,7 +279,34 @@ __device__ __forceinline__ void ragged_finish(const RaggedRow &g, const uint16_t
 // 29.2 us at [4096, 4099] and [2048, 11007]), run-time shifts by selects (22.6 and 40.4 us), the edge as
 // partial vectors in the main loop (29.8 and 54.6 us: its branches serialise the loads).
 // Two vectors per thread hold the sums of 16384 units in two blocks of 512 threads per SM at 64 registers.
-constexpr int kRmsnormRaggedMaxThreads = 512;
+constexpr int kRmsnormRaggedMaxThreads = 512, kRmsnormRaggedMinThreads = 64;
+
+// Vectors per thread and block size for T rows of `units` units; vpt = 0 where the ragged kernel does not
+// apply.  A block has at least 64 threads, one per unit of the longest edge, also where fewer could hold the body.
+// One vector per thread up to 320 threads, then two (up to 512 threads), then, for binary32 rows only (half
+// the sums per unit), four: 21.3 us with one and 21.6 with two at [4096, 4099], 45.1 and 41.4 us at [4096, 8188],
+// 39.2 and 28.8 us at [2048, 11007].  Two also where that makes one wave of what would be a little more (5
+// blocks of 256 threads per SM at 48 registers against 8 of 128 at 64: 6.8 -> 6.6 us at [1024, 4101]).  A few wide
+// rows of 8-byte vectors are left to the clusters, which spread each over several SMs (3.1 against 4.9 us at
+// fp32 [16, 16382], 4.9 and 5.1 at 64 rows, 9.5 and 6.5 at 128).
+struct RaggedShape {
+    int vpt, threads;
+};
+constexpr int64_t kRmsnormRaggedWideRows = 64;
+inline RaggedShape rmsnorm_ragged_shape(int64_t T, int64_t units, bool binary32, bool vec8_byte) {
+    const int64_t nvec = units / 16;
+    auto threads_for = [&](int v) {
+        const int64_t t = ((nvec + v - 1) / v + 31) / 32 * 32;
+        return static_cast<int>(t < kRmsnormRaggedMinThreads ? kRmsnormRaggedMinThreads : t);
+    };
+    const int64_t wave1 = 148 * (65536 / (48 * threads_for(1))), wave2 = 148 * (65536 / (64 * threads_for(2)));
+    if (nvec <= 320 && !(T > wave1 && T <= wave2)) return {1, threads_for(1)};
+    if (nvec <= 2 * kRmsnormRaggedMaxThreads) return {2, threads_for(2)};
+    if (binary32 && nvec <= 4 * kRmsnormRaggedMaxThreads && !(vec8_byte && T <= kRmsnormRaggedWideRows))
+        return {4, threads_for(4)};
+    return {0, 0};
+}
+
 template <int DT, int VPT, bool EARLY_W>
 __global__ void __launch_bounds__(kRmsnormRaggedMaxThreads, VPT <= 2 ? 2 : 1)
 fused_add_rmsnorm_ragged_kernel(RmsnormOperands op, const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {

@@ -39,6 +39,15 @@ def test_fuzz_fused_add_rmsnorm(T, H, dtype, offset, seed):
     run_rmsnorm(wl.rmsnorm_inputs(T, H, dtype, eps=1e-5, seed=seed), offset=offset)
 
 
+@pytest.mark.parametrize("T,H,dtype,offset,seed", cases(5, 90, widths=[1025, 1027, 1030, 1034, 1038, 1041, 2051, 2058, 3075, 4099, 4101,
+                                                                       4100, 5119, 5126, 8191, 8196, 11007, 16383]))
+def test_fuzz_fused_add_rmsnorm_with_a_weight_of_its_own(T, H, dtype, offset, seed):
+    """Widths that start rows anywhere, the weight at an offset drawn apart from the rows'."""
+    rng = random.Random(seed)
+    T = rng.choice([T, T, rng.randrange(1, MAX_ELEMS // H)])  # every block shape has its own range of rows
+    run_rmsnorm(wl.rmsnorm_inputs(T, H, dtype, eps=1e-5, seed=seed), offset=offset, weight_offset=rng.randrange(16))
+
+
 @pytest.mark.parametrize("T,D,dtype,offset,seed", cases(2, 90))
 def test_fuzz_silu_and_mul(T, D, dtype, offset, seed):
     if 2 * T * D > MAX_ELEMS:

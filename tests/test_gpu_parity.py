@@ -63,9 +63,11 @@ def fold(total: dict, part: dict) -> dict:
     return total
 
 
-def run_rmsnorm(inp: wl.RmsnormInputs, offset=0, stream=None):
-    """Runs the library on the input and compares EVERY row with the oracle (in row chunks)."""
-    gx, gr, gw = Guarded(inp.x, offset), Guarded(inp.residual, offset), Guarded(inp.weight, offset)
+def run_rmsnorm(inp: wl.RmsnormInputs, offset=0, stream=None, weight_offset=None):
+    """Runs the library on the input and compares EVERY row with the oracle (in row chunks).  The weight lies at
+    `weight_offset` (elements beyond a 256-byte boundary), like the rows unless given."""
+    gx, gr = Guarded(inp.x, offset), Guarded(inp.residual, offset)
+    gw = Guarded(inp.weight, offset if weight_offset is None else weight_offset)
     astra.astra_fused_add_rmsnorm(gx.t, gr.t, gw.t, inp.eps, stream=stream)
     torch.cuda.synchronize()
     for g in (gx, gr, gw):

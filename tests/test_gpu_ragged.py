@@ -48,6 +48,15 @@ def test_rmsnorm_ragged_rows(T, H, offset, dtype):
     run_rmsnorm(wl.rmsnorm_inputs(T, H, dtype, eps=1e-5, seed=H + offset), offset=offset)
 
 
+@pytest.mark.parametrize("dtype", [BF16, FP16])
+@pytest.mark.parametrize("T,H,weight_row", [(4000, 1025, 7), (4000, 1030, 1), (4000, 1038, 3), (3109, 1025, 11), (1500, 2051, 5),
+                                            (1030, 4101, 2)])
+def test_rmsnorm_ragged_rows_with_a_weight_of_their_own(T, H, weight_row, dtype):
+    """The weight as a row of a wider [L, H] tensor, which starts at another place within 32 bytes than the first
+    row, at the row counts where two vectors per thread make one wave."""
+    run_rmsnorm(wl.rmsnorm_inputs(T, H, dtype, eps=1e-5, seed=T + H), weight_offset=weight_row * H)
+
+
 @pytest.mark.parametrize("pads", [(0, 0, 0, 0), (16, 128, 0, 32), (16, 8, 0, 0)])
 def test_rmsnorm_ragged_pitches(pads):
     """Pitches that keep the four tensors together modulo 32 bytes, and (last) pitches that do not."""

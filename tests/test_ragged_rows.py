@@ -1,7 +1,7 @@
 """Index arithmetic of the kernels for rows that start at any element, run on the host: the geometry
-functions of the kernel headers are compiled into a small program that walks every alignment of every
-operand, widths around multiples of the vector size, and all threads, and checks that each unit of a row
-belongs to exactly one thread, that every access lies inside its tensor and is aligned to its size."""
+functions of the kernel headers and the launch rule are compiled into a small program that walks every
+alignment of every operand, widths around multiples of the vector size, every block shape that the rule gives
+them, and all threads, and checks that each unit of a row belongs to exactly one thread, that every access lies inside its tensor and is aligned to its size."""
 import subprocess
 
 
@@ -9,6 +9,8 @@ from paper_2509_07506_b200 import build as astra_build
 
 PROGRAM = r"""
 #include <cstdio>
+#include <set>
+#include <utility>
 #include <vector>
 #include "fused_add_rmsnorm.cuh"
 #include "silu_and_mul.cuh"
@@ -66,14 +68,24 @@ template <int UNITS> static void silu_rows(long o0, long a0, long b0, int rows, 
 }
 
 int main() {
-    for (int units : {1024, 1025, 1039, 1040, 1041, 1055, 1056, 2051, 5120, 5135, 5136})
-        for (long row = 0; row < 16; ++row)
-            for (long weight = 0; weight < 16; ++weight) {
-                const int one = (units / 16 + 31) / 32 * 32, two = ((units / 16 + 1) / 2 + 31) / 32 * 32;
-                norm_row<1>(row, weight, units, 1, one);
-                norm_row<1>(row, weight, units, 2, two < 64 ? 64 : two);
-                if (units % 2 == 0 && row % 2 == 0 && weight % 2 == 0) norm_row<2>(row, weight, units, 1, one);
+    // every shape that the launch rule gives a width at any row count
+    std::set<int> widths = {1055, 1056, 1057, 2051, 4099, 5120, 5135, 5136, 8191, 16383, 16399, 16400, 32767, 32782};
+    for (int units = 1024; units <= 1041; ++units) widths.insert(units);
+    for (int units : widths)
+        for (bool binary32 : {false, true}) {
+            std::set<std::pair<int, int>> shapes;
+            for (int T = 1; T <= 6000; ++T) {
+                const RaggedShape sh = rmsnorm_ragged_shape(T, units, binary32, T % 2 == 0);
+                if (sh.vpt > 0) shapes.insert({sh.vpt, sh.threads});
             }
+            expect(binary32 || units >= 16400 || !shapes.empty(), "shape", units, 0, 0, 0);
+            for (auto [vpt, threads] : shapes)
+                for (long row = 0; row < 16; ++row)
+                    for (long weight = 0; weight < 16; ++weight) {
+                        if (!binary32) norm_row<1>(row, weight, units, vpt, threads);
+                        else if (units % 2 == 0 && row % 2 == 0 && weight % 2 == 0) norm_row<2>(row, weight, units, vpt, threads);
+                    }
+        }
     for (int D : {512, 513, 514, 519, 520, 527})
         for (int rows : {1, 2, 3, 5})
             for (long o = 0; o < 8; ++o)
