@@ -130,7 +130,9 @@ struct Table {
     Table &operator=(const Table &) = delete;
 };
 
-// The launch itself runs without the interpreter lock: it blocks while the GPU's queue is full.
+// The strided and two-shot forms launch without the interpreter lock, as they did through ctypes.  The plain
+// forms keep it, as prepared calls do: whoever gives it up beside a thread that computes in Python waits a
+// whole switch interval (5 ms) to have it back, 1000 times the call.
 template <typename CALL> astra_status_t unlocked(CALL call) {
     PyThreadState *state = PyEval_SaveThread();
     const astra_status_t st = call();
@@ -172,9 +174,7 @@ PyObject *tc_rmsnorm(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const stream = stream_of(a[4], x);
         void *const p_x = x.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_fused_add_rmsnorm)>(KIND_RMSNORM);
-        return unlocked([&] {
-            return fn(p_x, r, w, T, H, eps, dt, stream);
-        });
+        return fn(p_x, r, w, T, H, eps, dt, stream);
     });
 }
 
@@ -189,9 +189,7 @@ PyObject *tc_silu(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const stream = stream_of(a[2], in);
         void *const p_in = in.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_silu_and_mul)>(KIND_SILU);
-        return unlocked([&] {
-            return fn(out, p_in, T, D, dt, stream);
-        });
+        return fn(out, p_in, T, D, dt, stream);
     });
 }
 
@@ -208,9 +206,7 @@ PyObject *tc_merge(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const stream = stream_of(a[6], va);
         void *const p_va = va.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_merge_attn_states_lse)>(KIND_MERGE);
-        return unlocked([&] {
-            return fn(vo, static_cast<float *>(so), p_va, static_cast<float *>(sa), vb, static_cast<float *>(sb), T, Hh, D, dt, stream);
-        });
+        return fn(vo, static_cast<float *>(so), p_va, static_cast<float *>(sa), vb, static_cast<float *>(sb), T, Hh, D, dt, stream);
     });
 }
 
@@ -227,9 +223,7 @@ PyObject *tc_allreduce(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const stream = stream_of(a[5], y);
         void *const p_y = y.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_fused_allreduce_add_rmsnorm)>(KIND_ALLREDUCE_RMSNORM);
-        return unlocked([&] {
-            return fn(p_y, r, parts.p, parts.n, w, T, H, eps, dt, stream);
-        });
+        return fn(p_y, r, parts.p, parts.n, w, T, H, eps, dt, stream);
     });
 }
 

@@ -1,5 +1,9 @@
 """The extension's own checks of direct calls: what is not the ordinary case is left to the binding's
 Python route (nothing launched, None returned), so that every refusal keeps its error."""
+import sys
+import threading
+import time
+
 import pytest
 import torch
 
@@ -137,3 +141,43 @@ def test_wrappers_and_modes_take_the_bindings_own_route(fast):
     torch.func.vmap(lambda v: (seen.append(fast.rmsnorm(v, r, w, 1e-6, None)), v)[1])(torch.stack([x, x]))
     assert seen == [None]
     torch.cuda.synchronize()
+
+
+@pytest.mark.gpu
+def test_plain_calls_keep_the_interpreter_lock(fast):
+    """Beside a thread that computes in Python, a call that gave the lock up would wait for it for a whole switch
+    interval; so many calls in a row would take `n` of them."""
+    x, r, w = norm()
+    va, sa = torch.randn(3, 4, 16, device="cuda"), torch.randn(3, 4, device="cuda")
+    vo, so, y = torch.empty_like(va), torch.empty_like(sa), torch.empty_like(x)
+    inp, out = torch.randn(3, 64, device="cuda"), torch.empty(3, 32, device="cuda")
+
+    def every():
+        binding.astra_fused_add_rmsnorm(x, r, w, 1e-6)
+        binding.astra_silu_and_mul(out, inp)
+        binding.astra_merge_attn_states_lse(vo, so, va, sa, va, sa)
+        binding.astra_fused_allreduce_add_rmsnorm(y, r, [x, x], w, 1e-6)
+
+    every()
+    torch.cuda.synchronize()
+    done = threading.Event()
+
+    def compute():
+        while not done.is_set():
+            pass
+    interval, n = 0.05, 20
+    before = sys.getswitchinterval()
+    other = threading.Thread(target=compute, daemon=True)
+    sys.setswitchinterval(interval)
+    try:
+        other.start()
+        start = time.perf_counter()
+        for _ in range(n // 4):
+            every()
+        took = time.perf_counter() - start
+    finally:
+        done.set()
+        sys.setswitchinterval(before)
+        other.join()
+    torch.cuda.synchronize()
+    assert took < n * interval / 4  # the lock may still be asked for once or twice in between
