@@ -25,6 +25,7 @@
 #include <torch/version.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "astra.h"
 #include "fastcall.h"
@@ -133,9 +134,11 @@ struct Table {
 // The strided and two-shot forms launch without the interpreter lock, as they did through ctypes.  The plain
 // forms keep it, as prepared calls do: whoever gives it up beside a thread that computes in Python waits a
 // whole switch interval (5 ms) to have it back, 1000 times the call.
-template <typename CALL> astra_status_t unlocked(CALL call) {
+// Everything they pass has been read before the lock is given up: plain values only.
+template <typename FN, typename... ARGS> astra_status_t unlocked(FN fn, ARGS... args) {
+    static_assert((std::is_scalar_v<ARGS> && ...), "no object is looked at without the interpreter lock");
     PyThreadState *state = PyEval_SaveThread();
-    const astra_status_t st = call();
+    const astra_status_t st = fn(args...);
     PyEval_RestoreThread(state);
     return st;
 }
@@ -240,9 +243,7 @@ PyObject *tc_allreduce_ex(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const stream = stream_of(a[6], r);
         void *const p_r = r.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_fused_allreduce_add_rmsnorm_ex)>(KIND_ALLREDUCE_RMSNORM_EX);
-        return unlocked([&] {
-            return fn(ys.p, ys.n, rs.p, rs.n, p_r, parts.p, parts.n, w, T, H, eps, dt, stream);
-        });
+        return unlocked(fn, ys.p, ys.n, rs.p, rs.n, p_r, parts.p, parts.n, w, T, H, eps, dt, stream);
     });
 }
 
@@ -263,9 +264,7 @@ PyObject *tc_rmsnorm_ex(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const p_x = x.mutable_data_ptr();
         void *const p_r = r.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_fused_add_rmsnorm_ex)>(KIND_RMSNORM_EX);
-        return unlocked([&] {
-            return fn(p_y, p_ro, p_x, p_r, w, T, H, pitch(y), pitch(ro), pitch(x), pitch(r), eps, dt, stream);
-        });
+        return unlocked(fn, p_y, p_ro, p_x, p_r, w, T, H, pitch(y), pitch(ro), pitch(x), pitch(r), eps, dt, stream);
     });
 }
 
@@ -282,9 +281,7 @@ PyObject *tc_silu_ex(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const p_gate = gate.mutable_data_ptr();
         void *const p_up = up.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_silu_and_mul_ex)>(KIND_SILU_EX);
-        return unlocked([&] {
-            return fn(p_out, p_gate, p_up, gate.size(0), gate.size(1), pitch(out), pitch(gate), pitch(up), dt, stream);
-        });
+        return unlocked(fn, p_out, p_gate, p_up, gate.size(0), gate.size(1), pitch(out), pitch(gate), pitch(up), dt, stream);
     });
 }
 
@@ -313,9 +310,8 @@ PyObject *tc_merge_ex(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
         void *const p_va = va.mutable_data_ptr();
         void *const p_vb = vb.mutable_data_ptr();
         const auto fn = entry<decltype(&astra_merge_attn_states_lse_ex)>(KIND_MERGE_EX);
-        return unlocked([&] {
-            return fn(p_vo, static_cast<float *>(score[2]), p_va, static_cast<float *>(score[0]), p_vb, static_cast<float *>(score[1]), T, Hh, D, st, dt, stream);
-        });
+        return unlocked(fn, p_vo, static_cast<float *>(score[2]), p_va, static_cast<float *>(score[0]), p_vb,
+                        static_cast<float *>(score[1]), T, Hh, D, st, dt, stream);
     });
 }
 
