@@ -25,6 +25,7 @@
 #include <torch/version.h>
 
 #include <algorithm>
+#include <exception>
 #include <type_traits>
 
 #include "astra.h"
@@ -124,7 +125,9 @@ struct Table {
         for (int i = 0; i < count; ++i) p[i] = dense(PySequence_Fast_GET_ITEM(seq, i), like, like.sizes(), true);
         for (; n < count; ++n) held[n] = Py_NewRef(PySequence_Fast_GET_ITEM(seq, n));
     }
+    // Not where the thread is being taken down: it does not hold the lock then, and the process is ending.
     ~Table() {
+        if (!PyGILState_Check()) return;
         while (n > 0) Py_DECREF(held[--n]);
     }
     Table(const Table &) = delete;
@@ -155,10 +158,12 @@ template <typename CALL> PyObject *guarded(Py_ssize_t nargs, Py_ssize_t want, CA
     }
     try {
         return PyLong_FromLong(static_cast<long>(call()));
-    } catch (...) {  // an unusual operand, or torch refused an access: the binding's own route decides
-        PyErr_Clear();
-        Py_RETURN_NONE;
+    } catch (const Unusual &) {
+    } catch (const std::exception &) {  // torch refused an access
     }
+    // (Nothing else is caught: at the interpreter's end, a thread that comes for the lock again is unwound.)
+    PyErr_Clear();  // the binding's own route decides
+    Py_RETURN_NONE;
 }
 
 }  // namespace

@@ -1,5 +1,7 @@
 """The extension's own checks of direct calls: what is not the ordinary case is left to the binding's
 Python route (nothing launched, None returned), so that every refusal keeps its error."""
+import os
+import subprocess
 import sys
 import threading
 import time
@@ -181,3 +183,27 @@ def test_plain_calls_keep_the_interpreter_lock(fast):
         other.join()
     torch.cuda.synchronize()
     assert took < n * interval / 4  # the lock may still be asked for once or twice in between
+
+
+@pytest.mark.gpu
+def test_threads_in_a_call_at_the_interpreters_end():
+    """A daemon thread that is in an unlocked launch when the interpreter ends is unwound when it comes for the
+    lock; the process ends with its own status all the same."""
+    code = """if True:
+        import sys, threading, time, torch
+        import paper_2509_07506_b200 as astra
+        x, r, w = (torch.zeros(s, device="cuda") for s in ((2, 64), (2, 64), 64))
+        ys, rs = [torch.zeros_like(x) for _ in range(2)], [torch.zeros_like(x) for _ in range(2)]
+        def work():
+            while True:
+                astra.astra_fused_add_rmsnorm_ex(ys[0], rs[0], x, r, w, 1e-6)
+                astra.astra_fused_allreduce_add_rmsnorm_ex(ys, rs, r, [x], w, 1e-6)
+        for _ in range(4):
+            threading.Thread(target=work, daemon=True).start()
+        time.sleep(0.5)
+        torch.cuda.synchronize()
+        sys.exit(7)
+    """
+    root = os.path.dirname(os.path.dirname(os.path.abspath(binding.__file__)))
+    done = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 7, (done.returncode, done.stderr[-2000:])
