@@ -1,7 +1,7 @@
 """Python binding of the C ABI in ``include/astra.h`` (argument marshalling only).
 
 Each function takes torch CUDA tensors, checks what the C side cannot see (device, dtype,
-contiguity, shapes that agree; in the ``_astra_fastcall`` extension for the ordinary case, here for
+contiguity, shapes that agree; in the ``_astra_torchcall`` extension for the ordinary case, here for
 every other and to say what is wrong), passes raw device pointers and the current stream to
 ``libastra.so`` and raises :class:`AstraError` on a non-zero status.  All arithmetic happens in
 the CUDA kernels; there is no fallback of any kind: if the shared library is missing, importing
@@ -11,12 +11,14 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from typing import Optional
 
 import torch
 
 LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libastra.so")
 FASTCALL_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_astra_fastcall.so")
+TORCHCALL_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_astra_torchcall.so")
 
 ASTRA_BF16 = 0
 ASTRA_FP16 = 1
@@ -94,14 +96,15 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
-_fast = None  # the _astra_fastcall extension module, once loaded
+_fast = None  # the _astra_fastcall extension module, once loaded, with the direct calls of _astra_torchcall
+
+_DIRECT = ("rmsnorm", "silu", "merge", "allreduce_rmsnorm", "rmsnorm_ex", "silu_ex", "merge_ex", "allreduce_rmsnorm_ex")
 
 
 def _load_fastcall(lib) -> None:
     """Import the `_astra_fastcall` extension from the package directory and give it the addresses of
-    the entry points resolved above.  It issues direct calls after checking the tensors itself (see
-    ``_raise_refusal``) and re-issues prepared calls, both without going through ctypes and, like the library,
-    it is required: a missing or stale module is an error, not a reason to take another route."""
+    the entry points resolved above.  It re-issues prepared calls without going through ctypes and, like the
+    library, it is required: a missing or stale module is an error, not a reason to take another route."""
     global _fast
     try:
         from . import _astra_fastcall as fast
@@ -109,21 +112,47 @@ def _load_fastcall(lib) -> None:
         raise ImportError(
             f"{FASTCALL_PATH} is missing or cannot be loaded ({exc}): build it with "
             "`python -m paper_2509_07506_b200.build`") from exc
-    from . import build as _build
-    if os.path.isdir(_build.CSRC) and os.path.isdir(_build.INCLUDE) and fast.build_id() != _build.source_hash():
-        raise ImportError(f"{FASTCALL_PATH} was built from other sources: rebuild it with "
-                          "`python -m paper_2509_07506_b200.build`")
-    if fast.torch_version() != torch.__version__:  # it reads torch's tensor objects
-        raise ImportError(f"{FASTCALL_PATH} was built for torch {fast.torch_version()}, this is {torch.__version__}: rebuild "
-                          "it with `python -m paper_2509_07506_b200.build`")
-    for kind, fn in ((fast.KIND_RMSNORM, lib.astra_fused_add_rmsnorm), (fast.KIND_SILU, lib.astra_silu_and_mul),
-                     (fast.KIND_MERGE, lib.astra_merge_attn_states_lse),
-                     (fast.KIND_ALLREDUCE_RMSNORM, lib.astra_fused_allreduce_add_rmsnorm),
-                     (fast.KIND_RMSNORM_EX, lib.astra_fused_add_rmsnorm_ex), (fast.KIND_SILU_EX, lib.astra_silu_and_mul_ex),
-                     (fast.KIND_MERGE_EX, lib.astra_merge_attn_states_lse_ex),
-                     (fast.KIND_ALLREDUCE_RMSNORM_EX, lib.astra_fused_allreduce_add_rmsnorm_ex)):
-        fast.bind(kind, ctypes.cast(fn, ctypes.c_void_p).value)
+    _refuse_other_sources(fast, FASTCALL_PATH)
+    _bind_entry_points(fast, lib)
+    direct = _load_torchcall(lib)
+    for name in _DIRECT:
+        setattr(fast, name, getattr(direct, name) if direct is not None else lambda *args: None)
     _fast = fast
+
+
+def _load_torchcall(lib):
+    """The `_astra_torchcall` extension, which issues direct calls after checking the tensors itself (see
+    ``_raise_refusal``), or None where there is none for this torch: it reads torch's C++ objects, so it belongs to
+    the release it was compiled against.  Direct calls then take this module's route, 3 to 24 us slower."""
+    from . import build as _build
+    built_for = _build.torchcall_torch(TORCHCALL_PATH)
+    try:
+        if built_for != str(torch.__version__):
+            raise ImportError("it is missing" if built_for is None else f"it was built for torch {built_for}")
+        from . import _astra_torchcall as direct
+    except ImportError as exc:
+        warnings.warn(f"{TORCHCALL_PATH} is not used with torch {torch.__version__} ({exc}); direct calls are slower than they "
+                      "need be until `python -m paper_2509_07506_b200.build` has run", RuntimeWarning, stacklevel=4)
+        return None
+    _refuse_other_sources(direct, TORCHCALL_PATH)
+    _bind_entry_points(direct, lib)
+    return direct
+
+
+def _refuse_other_sources(module, path: str) -> None:
+    from . import build as _build
+    if os.path.isdir(_build.CSRC) and os.path.isdir(_build.INCLUDE) and module.build_id() != _build.source_hash():
+        raise ImportError(f"{path} was built from other sources: rebuild it with `python -m paper_2509_07506_b200.build`")
+
+
+def _bind_entry_points(module, lib) -> None:
+    for kind, fn in (("RMSNORM", lib.astra_fused_add_rmsnorm), ("SILU", lib.astra_silu_and_mul),
+                     ("MERGE", lib.astra_merge_attn_states_lse), ("ALLREDUCE_RMSNORM", lib.astra_fused_allreduce_add_rmsnorm),
+                     ("RMSNORM_EX", lib.astra_fused_add_rmsnorm_ex), ("SILU_EX", lib.astra_silu_and_mul_ex),
+                     ("MERGE_EX", lib.astra_merge_attn_states_lse_ex),
+                     ("ALLREDUCE_RMSNORM_EX", lib.astra_fused_allreduce_add_rmsnorm_ex)):
+        if hasattr(module, f"KIND_{kind}"):
+            module.bind(getattr(module, f"KIND_{kind}"), ctypes.cast(fn, ctypes.c_void_p).value)
 
 
 def _refuse_stale(lib) -> None:

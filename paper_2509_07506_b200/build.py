@@ -1,6 +1,7 @@
 """Build ``libastra.so`` (the CUDA kernels and their C ABI) for sm_100a with nvcc, the ablation
-library beside it, and ``_astra_fastcall`` (a small CPython extension that issues calls without ctypes
-or Python-level checks) with the host compilers.
+library beside it, and with the host compilers two small CPython extensions that issue calls without
+ctypes: ``_astra_fastcall`` (prepared calls) and ``_astra_torchcall`` (direct calls on the tensors of the
+installed torch).
 
 Usage: ``python -m paper_2509_07506_b200.build [--force]``.  The shared objects are written next
 to this file; nothing is installed outside the source tree.
@@ -22,10 +23,12 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB_PATH = os.path.join(PKG_DIR, "libastra.so")
 ABLATION_LIB_PATH = os.path.join(PKG_DIR, "libastra_ablation.so")
 FASTCALL_PATH = os.path.join(PKG_DIR, "_astra_fastcall.so")
+TORCHCALL_PATH = os.path.join(PKG_DIR, "_astra_torchcall.so")
 
 SOURCES = ["astra.cu", "astra_allreduce.cu"]
 ABLATION_SOURCES = ["ablation.cu"]
-FASTCALL_SOURCES = ["fastcall.c", "torchcall.cpp"]
+FASTCALL_SOURCE = "fastcall.c"
+TORCHCALL_SOURCE = "torchcall.cpp"
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-std=c++17", "-lineinfo",
@@ -97,53 +100,61 @@ def _compile(lib_path: str, sources, force: bool, verbose: bool, extra_flags=())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile libastra.so (and the _astra_fastcall extension the binding loads with it) if missing or
-    built from other sources; returns the library's path."""
+    """Compile libastra.so (and the extensions the binding loads with it) if missing or built from other
+    sources; returns the library's path."""
     build_fastcall(force)
+    try:
+        build_torchcall(force)
+    except (RuntimeError, OSError, subprocess.CalledProcessError) as exc:  # no torch headers, say: direct calls do without
+        print(f"_astra_torchcall not built, direct calls take the slower route: {exc}", file=sys.stderr)
     return _compile(LIB_PATH, SOURCES, force, verbose)
 
 
-def _fastcall_is_stale() -> bool:
-    """The extension reads torch's tensor objects, so it belongs to one torch release as well as to one
-    state of the sources."""
-    import torch
-    if is_stale(FASTCALL_PATH):
-        return True
-    with open(FASTCALL_PATH, "rb") as fh:
-        return b"astra-torch:" + torch.__version__.encode() + b";" not in fh.read()
-
-
 def build_fastcall(force: bool = False) -> str:
-    """Compile the _astra_fastcall extension (against the CPython and torch headers) if it is missing or
-    was built from other sources or for another torch; returns its path."""
-    if not force and not _fastcall_is_stale():
+    """Compile the _astra_fastcall extension (plain C against the CPython headers) if it is missing or was
+    built from other sources; returns its path."""
+    if not force and not is_stale(FASTCALL_PATH):
         return FASTCALL_PATH
-    import torch
-    from torch.utils import cpp_extension
-    cc, cxx = shutil.which("gcc") or shutil.which("cc"), shutil.which("g++") or shutil.which("c++")
-    if cc is None or cxx is None:
-        raise RuntimeError("no C and C++ compilers found: _astra_fastcall cannot be built")
-    common = ["-O2", "-fPIC", "-fvisibility=hidden", f'-DASTRA_BUILD_ID="{source_hash()}"',
-              f'-DASTRA_TORCH_VERSION="{torch.__version__}"', "-I", sysconfig.get_paths()["include"], "-I", INCLUDE, "-I", CSRC]
-    torch_dirs = [flag for d in cpp_extension.include_paths("cuda") for flag in ("-isystem", d)]
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if cc is None:
+        raise RuntimeError("no C compiler found: _astra_fastcall cannot be built")
     tmp = FASTCALL_PATH + f".tmp{os.getpid()}"
-    objects = []
-    try:
-        for src in FASTCALL_SOURCES:
-            obj = f"{tmp}.{src}.o"
-            objects.append(obj)
-            lang = [cc, "-std=c11"] if src.endswith(".c") else [
-                cxx, "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *torch_dirs]
-            subprocess.check_call([*lang, *common, "-c", "-o", obj, os.path.join(CSRC, src)])
-        lib = os.path.join(os.path.dirname(torch.__file__), "lib")
-        subprocess.check_call([cxx, "-shared", "-o", tmp, *objects, "-L", lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
-                               "-ltorch_python"])
-    finally:
-        for obj in objects:
-            if os.path.exists(obj):
-                os.remove(obj)
+    subprocess.check_call([cc, "-O2", "-std=c11", "-shared", "-fPIC", "-fvisibility=hidden", f'-DASTRA_BUILD_ID="{source_hash()}"',
+                           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE, "-I", CSRC, "-o", tmp,
+                           os.path.join(CSRC, FASTCALL_SOURCE)])
     os.replace(tmp, FASTCALL_PATH)
     return FASTCALL_PATH
+
+
+def torchcall_torch(path: str = TORCHCALL_PATH):
+    """The torch release a built _astra_torchcall belongs to (read from the file, without loading it), or None."""
+    try:
+        with open(path, "rb") as fh:
+            m = re.search(rb"astra-torch:([^;]+);", fh.read())
+    except OSError:
+        return None
+    return m.group(1).decode() if m else None
+
+
+def build_torchcall(force: bool = False) -> str:
+    """Compile the _astra_torchcall extension (against the CPython and torch headers) if it is missing or
+    was built from other sources or for another torch; returns its path."""
+    import torch
+    if not force and not is_stale(TORCHCALL_PATH) and torchcall_torch() == str(torch.__version__):
+        return TORCHCALL_PATH
+    from torch.utils import cpp_extension
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        raise RuntimeError("no C++ compiler found")
+    tmp = TORCHCALL_PATH + f".tmp{os.getpid()}"
+    subprocess.check_call([cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DASTRA_BUILD_ID="{source_hash()}"',
+                           f'-DASTRA_TORCH_VERSION="{torch.__version__}"', "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+                           "-I", CSRC, *(flag for d in cpp_extension.include_paths("cuda") for flag in ("-isystem", d)),
+                           "-o", tmp, os.path.join(CSRC, TORCHCALL_SOURCE), "-L", os.path.join(os.path.dirname(torch.__file__), "lib"),
+                           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, TORCHCALL_PATH)
+    return TORCHCALL_PATH
 
 
 def ensure_built(ablation: bool = False) -> str:
@@ -168,4 +179,5 @@ def build_ablation(force: bool = False, verbose: bool = False) -> str:
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
     print(FASTCALL_PATH)
+    print(TORCHCALL_PATH)
     print(build_ablation(force="--force" in sys.argv, verbose="-v" in sys.argv))

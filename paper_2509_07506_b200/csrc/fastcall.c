@@ -8,7 +8,8 @@
  * the entry point.  It only marshals: every argument check of the C ABI still runs inside the entry
  * point on every launch, and nothing is computed here.
  *
- * Direct calls on tensors are in torchcall.cpp, the other half of the module.
+ * Direct calls on tensors are in torchcall.cpp, an extension of its own: it belongs to one torch release,
+ * this one to none.
  *
  * The module does not link against libastra.so.  The binding hands it the addresses of the entry
  * points it has already resolved (`bind`), so there is one copy of the library in the process and
@@ -38,7 +39,7 @@ typedef astra_status_t (*merge_fn)(void *, float *, const void *, const float *,
 typedef astra_status_t (*allreduce_fn)(void *, void *, const void *const *, int32_t, const void *, int64_t,
                                        int64_t, float, astra_dtype_t, void *);
 
-void *astra_entry_points[KIND_COUNT];
+static void *entry_points[KIND_PREPARED];
 
 typedef struct {
     PyObject_HEAD
@@ -73,13 +74,13 @@ static PyObject *fc_bind(PyObject *self, PyObject *args) {
     int kind;
     PyObject *addr;
     if (!PyArg_ParseTuple(args, "iO", &kind, &addr)) return NULL;
-    if (kind < 0 || kind >= KIND_COUNT) {
+    if (kind < 0 || kind >= KIND_PREPARED) {
         PyErr_SetString(PyExc_ValueError, "unknown kind of call");
         return NULL;
     }
     void *p;
     if (as_address(addr, &p) < 0) return NULL;
-    astra_entry_points[kind] = p;
+    entry_points[kind] = p;
     Py_RETURN_NONE;
 }
 
@@ -99,7 +100,7 @@ static PyObject *fc_prepare(PyObject *self, PyObject *args) {
         PyErr_SetString(PyExc_ValueError, "unknown kind of call");
         return NULL;
     }
-    if (astra_entry_points[kind] == NULL) {
+    if (entry_points[kind] == NULL) {
         PyErr_SetString(PyExc_RuntimeError, "no entry point bound for this kind of call");
         return NULL;
     }
@@ -148,7 +149,7 @@ static PyObject *fc_launch(PyObject *self, PyObject *const *args, Py_ssize_t nar
     void *stream = PyLong_AsVoidPtr(args[1]);
     if (stream == NULL && PyErr_Occurred()) return NULL;
     const astra_dtype_t dt = (astra_dtype_t)p->dtype;
-    void *fn = astra_entry_points[p->kind];
+    void *fn = entry_points[p->kind];
     if (fn == NULL) {  /* unbound again since the call was prepared */
         PyErr_SetString(PyExc_RuntimeError, "no entry point bound for this kind of call");
         return NULL;
@@ -211,28 +212,12 @@ static PyObject *fc_build_id(PyObject *self, PyObject *noargs) {
     return PyUnicode_FromString(astra_fastcall_build_marker + sizeof("astra-build-id:") - 1);
 }
 
-static PyObject *fc_torch_version(PyObject *self, PyObject *noargs) {
-    const char *v = astra_torch_marker + sizeof("astra-torch:") - 1;
-    return PyUnicode_FromStringAndSize(v, (Py_ssize_t)strlen(v) - 1);
-}
-
 static PyMethodDef methods[] = {
     {"bind", fc_bind, METH_VARARGS, "bind(kind, address): set the entry point of one kind of call"},
     {"prepare", fc_prepare, METH_VARARGS, "prepare(kind, pointers, extents, eps, dtype, parts) -> Prepared"},
     {"launch", (PyCFunction)(void (*)(void))fc_launch, METH_FASTCALL, "launch(prepared, stream_handle) -> status"},
-#define DIRECT(name, fn, doc) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL, doc " -> status, or None: not the ordinary case"}
-    DIRECT("rmsnorm", tc_rmsnorm, "rmsnorm(x, residual, weight, eps, stream)"),
-    DIRECT("silu", tc_silu, "silu(out, input, stream)"),
-    DIRECT("merge", tc_merge, "merge(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream)"),
-    DIRECT("allreduce_rmsnorm", tc_allreduce, "allreduce_rmsnorm(y, residual, parts, weight, eps, stream)"),
-    DIRECT("rmsnorm_ex", tc_rmsnorm_ex, "rmsnorm_ex(y, residual_out, x, residual, weight, eps, stream)"),
-    DIRECT("silu_ex", tc_silu_ex, "silu_ex(out, gate, up, stream)"),
-    DIRECT("merge_ex", tc_merge_ex, "merge_ex(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream)"),
-    DIRECT("allreduce_rmsnorm_ex", tc_allreduce_ex,
-           "allreduce_rmsnorm_ex(y_outs, residual_outs, residual, parts, weight, eps, stream)"),
     {"footprint", fc_footprint, METH_O, "footprint(prepared) -> ((address, bytes, is_written), ...)"},
     {"build_id", fc_build_id, METH_NOARGS, "hash of the sources this module was compiled from"},
-    {"torch_version", fc_torch_version, METH_NOARGS, "torch release this module was compiled against"},
     {NULL, NULL, 0, NULL},
 };
 
@@ -253,9 +238,5 @@ PyMODINIT_FUNC PyInit__astra_fastcall(void) {
     PyModule_AddIntConstant(m, "KIND_SILU", KIND_SILU);
     PyModule_AddIntConstant(m, "KIND_MERGE", KIND_MERGE);
     PyModule_AddIntConstant(m, "KIND_ALLREDUCE_RMSNORM", KIND_ALLREDUCE_RMSNORM);
-    PyModule_AddIntConstant(m, "KIND_RMSNORM_EX", KIND_RMSNORM_EX);
-    PyModule_AddIntConstant(m, "KIND_SILU_EX", KIND_SILU_EX);
-    PyModule_AddIntConstant(m, "KIND_MERGE_EX", KIND_MERGE_EX);
-    PyModule_AddIntConstant(m, "KIND_ALLREDUCE_RMSNORM_EX", KIND_ALLREDUCE_RMSNORM_EX);
     return m;
 }

@@ -1,7 +1,5 @@
-/* Shared by the two halves of the _astra_fastcall extension (fastcall.c and torchcall.cpp). */
+/* Kinds of calls, shared by the _astra_fastcall (fastcall.c) and _astra_torchcall (torchcall.cpp) extensions. */
 #pragma once
-
-#include <Python.h>
 
 enum {  /* the first KIND_PREPARED kinds can be prepared */
     KIND_RMSNORM = 0,
@@ -15,23 +13,3 @@ enum {  /* the first KIND_PREPARED kinds can be prepared */
     KIND_ALLREDUCE_RMSNORM_EX = 7,
     KIND_COUNT = 8
 };
-
-#ifdef __cplusplus
-extern "C" {
-#endif
-
-extern void *astra_entry_points[KIND_COUNT];
-extern const char astra_torch_marker[];  /* "astra-torch:<release>;" */
-
-PyObject *tc_rmsnorm(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_silu(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_merge(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_allreduce(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_rmsnorm_ex(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_silu_ex(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_merge_ex(PyObject *, PyObject *const *, Py_ssize_t);
-PyObject *tc_allreduce_ex(PyObject *, PyObject *const *, Py_ssize_t);
-
-#ifdef __cplusplus
-}
-#endif

@@ -1,5 +1,6 @@
-// Direct calls of the astra.h ABI on torch tensors, without Python-level checks: the second half of the
-// _astra_fastcall extension.
+// _astra_torchcall -- a CPython extension for direct calls of the astra.h ABI on torch tensors, without
+// Python-level checks.  It reads torch's C++ objects and so belongs to one torch release; with another one the
+// binding leaves it unloaded and takes its own route.
 //
 // A direct call from the binding's Python code costs 3.5 to 12 us of attribute reads, checks and argument
 // conversions, more than the launch and far more than the kernel of a decode-sized shape.  Each function
@@ -31,9 +32,15 @@
 #include "astra.h"
 #include "fastcall.h"
 
+#ifndef ASTRA_BUILD_ID
+#define ASTRA_BUILD_ID "unidentified"
+#endif
+
 namespace {
 
 constexpr int kMaxTable = 16;
+
+void *entry_points[KIND_COUNT];
 
 // What a call that is not the ordinary case answers instead of a status.  (A value and not an exception: such
 // calls go on to the Python route on every call, 12 us for a generator of partials, and a C++ exception adds 2.)
@@ -159,7 +166,7 @@ template <typename FN, typename... ARGS> astra_status_t unlocked(FN fn, ARGS... 
 }
 
 // The entry point of one kind of call, or null where none is bound.
-template <typename FN> FN entry(int kind) { return reinterpret_cast<FN>(astra_entry_points[kind]); }
+template <typename FN> FN entry(int kind) { return reinterpret_cast<FN>(entry_points[kind]); }
 
 template <typename CALL> PyObject *guarded(Py_ssize_t nargs, Py_ssize_t want, CALL call) {
     if (nargs != want) {
@@ -176,10 +183,6 @@ template <typename CALL> PyObject *guarded(Py_ssize_t nargs, Py_ssize_t want, CA
     PyErr_Clear();  // the binding's own route decides
     Py_RETURN_NONE;
 }
-
-}  // namespace
-
-extern "C" {
 
 // rmsnorm(x, residual, weight, eps, stream)
 PyObject *tc_rmsnorm(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
@@ -328,7 +331,63 @@ PyObject *tc_merge_ex(PyObject *, PyObject *const *a, Py_ssize_t nargs) {
     });
 }
 
-// The torch release this file was compiled against; the build script finds it in the built file.
-__attribute__((used)) const char astra_torch_marker[] = "astra-torch:" ASTRA_TORCH_VERSION ";";
+// What this file was compiled from and against; the build script and the binding find both in the built file.
+__attribute__((used)) const char build_marker[] = "astra-build-id:" ASTRA_BUILD_ID;
+__attribute__((used)) const char torch_marker[] = "astra-torch:" ASTRA_TORCH_VERSION ";";
 
-}  // extern "C"
+PyObject *tc_build_id(PyObject *, PyObject *) {
+    return PyUnicode_FromString(build_marker + sizeof("astra-build-id:") - 1);
+}
+
+// bind(kind, address): the entry point that calls of this kind go to
+PyObject *tc_bind(PyObject *, PyObject *args) {
+    int kind;
+    PyObject *address;
+    if (!PyArg_ParseTuple(args, "iO", &kind, &address)) return nullptr;
+    if (kind < 0 || kind >= KIND_COUNT) {
+        PyErr_SetString(PyExc_ValueError, "unknown kind of call");
+        return nullptr;
+    }
+    void *p = address == Py_None ? nullptr : PyLong_AsVoidPtr(address);
+    if (p == nullptr && PyErr_Occurred()) return nullptr;
+    entry_points[kind] = p;
+    Py_RETURN_NONE;
+}
+
+#define DIRECT(name, fn, doc) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL, doc " -> status, or None: not the ordinary case"}
+PyMethodDef methods[] = {
+    {"bind", tc_bind, METH_VARARGS, "bind(kind, address): set the entry point of one kind of call"},
+    DIRECT("rmsnorm", tc_rmsnorm, "rmsnorm(x, residual, weight, eps, stream)"),
+    DIRECT("silu", tc_silu, "silu(out, input, stream)"),
+    DIRECT("merge", tc_merge, "merge(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream)"),
+    DIRECT("allreduce_rmsnorm", tc_allreduce, "allreduce_rmsnorm(y, residual, parts, weight, eps, stream)"),
+    DIRECT("rmsnorm_ex", tc_rmsnorm_ex, "rmsnorm_ex(y, residual_out, x, residual, weight, eps, stream)"),
+    DIRECT("silu_ex", tc_silu_ex, "silu_ex(out, gate, up, stream)"),
+    DIRECT("merge_ex", tc_merge_ex, "merge_ex(v_out, lse_out, v_a, lse_a, v_b, lse_b, stream)"),
+    DIRECT("allreduce_rmsnorm_ex", tc_allreduce_ex,
+           "allreduce_rmsnorm_ex(y_outs, residual_outs, residual, parts, weight, eps, stream)"),
+    {"build_id", tc_build_id, METH_NOARGS, "hash of the sources this module was compiled from"},
+    {nullptr, nullptr, 0, nullptr},
+};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_astra_torchcall", "direct calls of the astra C ABI on torch tensors", -1, methods,
+                      nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__astra_torchcall(void) {
+    PyObject *m = PyModule_Create(&module);
+    if (m == nullptr) return nullptr;
+    const struct { const char *name; int kind; } kinds[] = {
+        {"KIND_RMSNORM", KIND_RMSNORM}, {"KIND_SILU", KIND_SILU}, {"KIND_MERGE", KIND_MERGE},
+        {"KIND_ALLREDUCE_RMSNORM", KIND_ALLREDUCE_RMSNORM}, {"KIND_RMSNORM_EX", KIND_RMSNORM_EX},
+        {"KIND_SILU_EX", KIND_SILU_EX}, {"KIND_MERGE_EX", KIND_MERGE_EX},
+        {"KIND_ALLREDUCE_RMSNORM_EX", KIND_ALLREDUCE_RMSNORM_EX}};
+    for (const auto &k : kinds) {
+        if (PyModule_AddIntConstant(m, k.name, k.kind) < 0) {
+            Py_DECREF(m);
+            return nullptr;
+        }
+    }
+    return m;
+}

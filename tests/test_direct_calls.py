@@ -34,6 +34,30 @@ def test_operands_that_are_not_cuda_tensors_are_left_to_the_binding(fast):
         fast.rmsnorm(t, t)
 
 
+@pytest.mark.parametrize("missing", [False, True])
+def test_another_torch_does_without_direct_calls(monkeypatch, fast, missing):
+    """An extension of another torch release, or none, is left out with a warning; the library, prepared calls and
+    the binding's own route need neither."""
+    t = torch.zeros((2, 8), dtype=torch.bfloat16)
+    try:
+        with monkeypatch.context() as m:
+            m.setattr(binding, "_lib", None)
+            if missing:
+                m.setattr(binding, "TORCHCALL_PATH", binding.TORCHCALL_PATH + ".none")
+            else:
+                m.setattr(torch, "__version__", "0.1.2")
+            with pytest.warns(RuntimeWarning, match="missing" if missing else "built for torch"):
+                binding.load_library()
+            assert binding._fast.silu(t, t, None) is None and binding._fast.build_id()
+            assert type(binding._fast.silu) is not type(binding._fast.build_id)
+            with pytest.raises(TypeError, match="CUDA"):
+                binding.astra_fused_add_rmsnorm(t, t, t[0], 1e-6)
+    finally:
+        binding._lib = None
+        binding.load_library()
+    assert type(binding._fast.silu) is type(binding._fast.build_id)
+
+
 def test_leaving_a_call_to_the_binding_costs_no_more_than_the_call(fast):
     """A refusal comes on top of the Python route on every such call; as a C++ exception it cost 20 to 40 empty
     calls of the extension."""
