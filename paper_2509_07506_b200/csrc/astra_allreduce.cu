@@ -14,9 +14,6 @@ using namespace astra::host;
 
 inline int round_up_to(int v, int m) { return (v + m - 1) / m * m; }
 
-constexpr int kStreamGroup = 2;  // partial loads in flight: long streams,
-constexpr int kDeepGroup = 8;    // and few rows
-
 // Register-resident rows hold at most 32 16-bit units per thread in vectors of 8, 16 or 32 bytes.
 // UVEC is the vector width in units, VPT the vectors per thread.
 // `dense` selects the instantiation whose registers are capped so that five 256-thread blocks fit an
@@ -160,103 +157,24 @@ cudaError_t choose_shape(const AllreduceOperands &op, const uint16_t *w, int64_t
   return cudaErrorInvalidValue;
 }
 
-// Streaming sizes whose operands are 32-byte aligned throughout: 32-byte accesses.  Measured L2-cold
-// against the 16-byte form at [8192, 4096]: 50.6 -> 49.2 us with 2 partials, 70.8 -> 66.6 us with 4,
-// 110.9 -> 104.7 us with 8; at [1024, 4096]: 8.3 -> 7.7, 10.9 -> 10.3, 16.2 -> 15.9 us.
-//
-// Five shapes: one or two vectors per thread (16 or 32 units), two or four partial loads in flight
-// (four only from four partials on), and two of each with the residual requested last.  What decides
-// between them is how many bytes of loads an SM has in flight, i.e. resident blocks x threads x bytes per
-// thread, with the resident blocks set by the registers (as compiled for sm_100a, allocated in eights,
-// 65536 per SM).  The measurements across H = 2048 ... 16384 fit one rule: take the first shape, in the
-// order below, that keeps about 90 KB in flight per SM; if none does, the one with the most.  Examples:
-// H = 4096 takes one vector and four in flight (three 256-thread blocks per SM); H = 8192 with four
-// in flight would leave one 512-thread block per SM, so it takes two vectors in 256-thread blocks
-// (78.8 -> 68.0 us with 4 partials, 117.3 -> 105.6 us with 8); H = 10240 with two in flight takes two
-// vectors in 320-thread blocks (two per SM) rather than one 640-thread block (61.6 against 76.7 us);
-// H = 11008 ... 14336 take the late residual (79.7 -> 67.9 us at [4096, 11008] with 2 partials, more at the
-// kernel; but 2.7 against 3.2 us at [16, 11008], where every SM has one row at most); H = 16384 takes one vector in one 1024-thread block (143.1 against 155.8 us with 4 partials).
-// Binary32 rows need fewer registers (5120 elements take one vector in two 640-thread blocks: 25.1 -> 23.1 us at
-// [1024, 5120] with 4 partials).
-// Binary32 rows of more than 16384 units take four vectors per thread, one load in flight, in one block
-// of up to 512 threads per SM, instead of two sweeps: 73.5 -> 52.6, 105.8 -> 73.5, 191 -> 112.5 us at [1024, 16384]
-// with 2 / 4 / 8 partials (48.6 / 68.1 / 107 us at 6.9 TB/s), 17.5 -> 9.5 us at [16, 16384] with 8.
-// Returns false where no shape applies (rows too narrow for 128-thread blocks, or too wide).
-struct WideShape {
-    int vpt, group, regs, max_threads, min_threads;
-    bool late = false;  // the residual is requested after the partials
-};
-#ifndef ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS
-#define ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS 128
-#endif
-constexpr int64_t kDeepQueueRows = ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS;
-constexpr int64_t kOneBlockRows = 148;  // rows up to which every SM of a B200 has one block at most
-constexpr int kWideShapeCount = 5;
-template <int DT> constexpr WideShape kWideShapes[kWideShapeCount] = {
-    {1, 4, 72, 512, 128}, {2, 4, 128, 256, 64}, {1, 2, 56, 1024, 128}, {2, 2, 96, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}};
-template <> constexpr WideShape kWideShapes<ASTRA_FP32>[kWideShapeCount] = {
-    {1, 4, 64, 512, 128}, {2, 4, 112, 256, 64}, {1, 2, 48, 1024, 128}, {2, 2, 80, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}};
-// The same shapes of the ragged kernel, with its registers.
-template <int DT> constexpr WideShape kRaggedShapes[kWideShapeCount] = {
-    {1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 120, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}};
-template <> constexpr WideShape kRaggedShapes<ASTRA_FP32>[kWideShapeCount] = {
-    {1, 4, 64, 512, 64}, {2, 4, 120, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 96, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}};
-constexpr int64_t kWideBytesInFlight = 90 * 1024;
-
+// Streaming sizes whose operands are 32-byte aligned throughout (RAGGED: lie together within 32 bytes): 32-byte
+// accesses in the shape that allreduce_wide_shape gives.  False where there is none.
 template <int DT, bool RAGGED>
 bool launch_wide(const AllreduceOperands &op, const uint16_t *w, int64_t T, int H, float eps, cudaStream_t stream,
                  cudaError_t *err) {
     constexpr int UVEC = 16;
-    const int nvec = H / (UVEC / Storage<DT>::UNITS);  // whole vectors (a ragged row has no more inside it)
-    // Few rows and more than four partials: all of a row's partials in one round trip (eight loads in
-    // flight, one vector per thread); with so few blocks the registers that costs do not matter.
-    // Device time from a graph, 8 partials, against the streaming shapes: 3.19 -> 2.70 us at [16, 4096],
-    // 4.17 -> 3.41 us at [16, 8192], 4.12 -> 3.85 us at [128, 4096]; slower from 192 rows on (7.93 -> 8.89 us
-    // at [192, 8192]).  With up to four partials the streaming shapes are the fastest at every row
-    // count (1.65 / 1.98 us at [16, 4096] with 2 / 4 partials, where the 16-byte shapes took 2.08 / 2.40).
-    // (The ragged kernel's four-in-flight shape fetches its edge last, so there four partials count as many.)
-    if (T <= kDeepQueueRows && op.n_parts > (RAGGED ? 3 : 4)) {
-        const int threads = round_up_to(nvec, 32);
-        if (threads >= (RAGGED ? 64 : 128) && threads <= allreduce_reg_max_threads(16, kDeepGroup)) {
-            *err = launch_rows<DT, UVEC, kDeepGroup, RAGGED>(op, w, T, H, eps, 1, threads, stream);
-            return true;
-        }
-    }
-    int best = -1, best_threads = 0;
-    int64_t best_bytes = 0;
-    for (int c = 0; c < kWideShapeCount; ++c) {
-        const WideShape &sh = RAGGED ? kRaggedShapes<DT>[c] : kWideShapes<DT>[c];
-        if (sh.group > kStreamGroup && op.n_parts < sh.group) continue;
-        if (sh.late && T <= kOneBlockRows) continue;  // a second block per SM has no row to work on then
-        const int threads = round_up_to((nvec + sh.vpt - 1) / sh.vpt, 32);
-        if (threads > sh.max_threads || threads < sh.min_threads) continue;
-        const int by_regs = 65536 / (sh.regs * threads), by_threads = 2048 / threads;
-        const int blocks = by_regs < by_threads ? by_regs : by_threads;
-        const int64_t bytes = static_cast<int64_t>(blocks) * threads * sh.vpt * (sh.group + (sh.late ? 0 : 1)) * 32;
-        if (bytes > best_bytes) {
-            best = c;
-            best_bytes = bytes;
-            best_threads = threads;
-        }
-        if (bytes >= kWideBytesInFlight) break;  // the first shape that reaches it is also the largest so far
-    }
-    if (best < 0) {
-        if constexpr (DT == ASTRA_FP32) {
-            const int threads = round_up_to((nvec + 3) / 4, 32);
-            if (nvec > 1024 && threads <= allreduce_reg_max_threads(64, 1)) {
-                *err = launch_rows<DT, UVEC, 1, RAGGED>(op, w, T, H, eps, 4, threads, stream);
-                return true;
-            }
-        }
-        return false;
-    }
-    const WideShape &sh = RAGGED ? kRaggedShapes<DT>[best] : kWideShapes<DT>[best];
-    if (sh.late)
-        *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED, true>(op, w, T, H, eps, sh.vpt, best_threads, stream);
+    const AllreduceShape sh = allreduce_wide_shape(T, H * Storage<DT>::UNITS, op.n_parts, DT == ASTRA_FP32, RAGGED);
+    if (sh.vpt == 0) return false;
+    if (sh.group == kDeepGroup)
+        *err = launch_rows<DT, UVEC, kDeepGroup, RAGGED>(op, w, T, H, eps, 1, sh.threads, stream);
+    else if (sh.late)
+        *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED, true>(op, w, T, H, eps, sh.vpt, sh.threads, stream);
     else if (sh.group == 4)
-        *err = launch_rows<DT, UVEC, 4, RAGGED>(op, w, T, H, eps, sh.vpt, best_threads, stream);
-    else
-        *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED>(op, w, T, H, eps, sh.vpt, best_threads, stream);
+        *err = launch_rows<DT, UVEC, 4, RAGGED>(op, w, T, H, eps, sh.vpt, sh.threads, stream);
+    else if (sh.group == kStreamGroup)
+        *err = launch_rows<DT, UVEC, kStreamGroup, RAGGED>(op, w, T, H, eps, sh.vpt, sh.threads, stream);
+    else if constexpr (DT == ASTRA_FP32)
+        *err = launch_rows<DT, UVEC, 1, RAGGED>(op, w, T, H, eps, sh.vpt, sh.threads, stream);
     return true;
 }
 

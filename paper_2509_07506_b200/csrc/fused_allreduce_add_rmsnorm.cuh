@@ -339,6 +339,101 @@ fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOpera
                                                           store_y)))
 }
 
+// Launch shapes of the two kernels in their 32-byte forms.  Measured L2-cold against the 16-byte form at [8192, 4096]: 50.6 -> 49.2 us with 2 partials, 70.8 -> 66.6 us with 4,
+// 110.9 -> 104.7 us with 8; at [1024, 4096]: 8.3 -> 7.7, 10.9 -> 10.3, 16.2 -> 15.9 us.
+//
+// Five shapes: one or two vectors per thread (16 or 32 units), two or four partial loads in flight
+// (four only from four partials on), and two of each with the residual requested last.  What decides
+// between them is how many bytes of loads an SM has in flight, i.e. resident blocks x threads x bytes per
+// thread, with the resident blocks set by the registers (as compiled for sm_100a).  The measurements across H = 2048 ... 16384 fit one rule: take the first shape, in the
+// order below, that keeps about 90 KB in flight per SM; if none does, the one with the most.  Examples:
+// H = 4096 takes one vector and four in flight (three 256-thread blocks per SM); H = 8192 with four
+// in flight would leave one 512-thread block per SM, so it takes two vectors in 256-thread blocks
+// (78.8 -> 68.0 us with 4 partials, 117.3 -> 105.6 us with 8); H = 10240 with two in flight takes two
+// vectors in 320-thread blocks (two per SM) rather than one 640-thread block (61.6 against 76.7 us);
+// H = 11008 ... 14336 take the late residual (79.7 -> 67.9 us at [4096, 11008] with 2 partials, more at the
+// kernel; but 2.7 against 3.2 us at [16, 11008], where every SM has one row at most); H = 16384 takes one vector in one 1024-thread block (143.1 against 155.8 us with 4 partials).
+// Binary32 rows need fewer registers (5120 elements take one vector in two 640-thread blocks: 25.1 -> 23.1 us at
+// [1024, 5120] with 4 partials).
+// Binary32 rows of more than 16384 units take four vectors per thread, one load in flight, in one block
+// of up to 512 threads per SM, instead of two sweeps: 73.5 -> 52.6, 105.8 -> 73.5, 191 -> 112.5 us at [1024, 16384]
+// with 2 / 4 / 8 partials (48.6 / 68.1 / 107 us at 6.9 TB/s), 17.5 -> 9.5 us at [16, 16384] with 8.
+struct WideShape {
+    int vpt, group, regs, max_threads, min_threads;
+    bool late = false;  // the residual is requested after the partials
+};
+constexpr int kStreamGroup = 2;  // partial loads in flight: long streams,
+constexpr int kDeepGroup = 8;    // and few rows
+#ifndef ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS
+#define ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS 128
+#endif
+constexpr int64_t kDeepQueueRows = ASTRA_ALLREDUCE_DEEP_QUEUE_ROWS;
+constexpr int64_t kOneBlockRows = 148;  // rows up to which every SM of a B200 has one block at most
+constexpr int kWideShapeCount = 5;
+constexpr WideShape kWideShapes[2][kWideShapeCount] = {
+    {{1, 4, 72, 512, 128}, {2, 4, 128, 256, 64}, {1, 2, 56, 1024, 128}, {2, 2, 96, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}},
+    {{1, 4, 64, 512, 128}, {2, 4, 112, 256, 64}, {1, 2, 48, 1024, 128}, {2, 2, 80, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}}};  // binary32
+// The same shapes of the ragged kernel, with its registers.
+constexpr WideShape kRaggedShapes[2][kWideShapeCount] = {
+    {{1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 120, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}},
+    {{1, 4, 64, 512, 64}, {2, 4, 120, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 96, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}}};
+constexpr int64_t kWideBytesInFlight = 90 * 1024;
+
+// Blocks that an SM holds at once.  Each of its four partitions has 16384 registers, hands them out warp by
+// warp in pieces of 256, and a block needs a place for each of its warps: 21 warps of 48 registers fit once, not
+// twice, although 2 * 21 * 32 * 48 registers are fewer than 65536 (counting them as two took fp32 [1024, 5152] with
+// 2 partials from 17.2 to 20.5 us).
+inline int resident_blocks(int regs, int threads) {
+    const int warps = (threads + 31) / 32;
+    const int by_regs = 4 * (16384 / ((regs * 32 + 255) / 256 * 256)) / warps, by_threads = 64 / warps;
+    return by_regs < by_threads ? by_regs : by_threads;
+}
+
+// Shape for T rows of `units` 16-bit units with n_parts partials; vpt = 0 where none applies (rows too narrow for
+// 128-thread blocks, ragged ones for 64, or too wide).
+struct AllreduceShape {
+    int vpt = 0, group = 0, threads = 0;
+    bool late = false;
+};
+inline AllreduceShape allreduce_wide_shape(int64_t T, int units, int n_parts, bool binary32, bool ragged) {
+    const int nvec = units / 16;  // whole vectors (a ragged row has no more inside it)
+    auto threads_for = [&](int vpt) { return ((nvec + vpt - 1) / vpt + 31) / 32 * 32; };
+    // Few rows and more than four partials: all of a row's partials in one round trip (eight loads in
+    // flight, one vector per thread); with so few blocks the registers that costs do not matter.
+    // Device time from a graph, 8 partials, against the streaming shapes: 3.19 -> 2.70 us at [16, 4096],
+    // 4.17 -> 3.41 us at [16, 8192], 4.12 -> 3.85 us at [128, 4096]; slower from 192 rows on (7.93 -> 8.89 us
+    // at [192, 8192]).  With up to four partials the streaming shapes are the fastest at every row
+    // count (1.65 / 1.98 us at [16, 4096] with 2 / 4 partials, where the 16-byte shapes took 2.08 / 2.40).
+    // (The ragged kernel's four-in-flight shape fetches its edge last, so there four partials count as many.)
+    if (T <= kDeepQueueRows && n_parts > (ragged ? 3 : 4) && threads_for(1) >= (ragged ? 64 : 128) &&
+        threads_for(1) <= allreduce_reg_max_threads(16, kDeepGroup))
+        return {1, kDeepGroup, threads_for(1)};
+    // Blocks without a row are not resident: binary32 rows of 11008 units keep one vector per thread up to 148 rows
+    // (4.7 against 6.5 us at [16, 6144] with 8 partials), and threads beyond the row's vectors have no loads.  The ragged kernel's edge wants both all the same
+    // (3.3 against 4.9 us at bf16 [500, 1059] with 2, 2.9 against 4.1 us at [150, 1603]).
+    const int64_t rows_per_sm = (T + kOneBlockRows - 1) / kOneBlockRows;
+    AllreduceShape best;
+    int64_t best_bytes = 0;
+    for (const WideShape &sh : (ragged ? kRaggedShapes : kWideShapes)[binary32]) {
+        if (sh.group > kStreamGroup && n_parts < sh.group) continue;
+        if (sh.late && T <= kOneBlockRows) continue;  // a second block per SM has no row to work on then
+        const int threads = threads_for(sh.vpt);
+        if (threads > sh.max_threads || threads < sh.min_threads) continue;
+        int64_t resident = resident_blocks(sh.regs, threads);
+        if (!ragged && resident > rows_per_sm) resident = rows_per_sm;
+        const int64_t vectors = ragged ? threads * sh.vpt : nvec;
+        const int64_t bytes = resident * vectors * (sh.group + (sh.late ? 0 : 1)) * 32;
+        if (bytes > best_bytes) {
+            best = {sh.vpt, sh.group, threads, sh.late};
+            best_bytes = bytes;
+        }
+        if (bytes >= kWideBytesInFlight) break;  // the first shape that reaches it is also the largest so far
+    }
+    if (best.vpt == 0 && binary32 && nvec > 1024 && threads_for(4) <= allreduce_reg_max_threads(64, 1))
+        return {4, 1, threads_for(4)};
+    return best;
+}
+
 // The rank-order sum of one vector position, GROUP partial loads in flight at a time.
 template <int DT, int VEC, int GROUP>
 __device__ __forceinline__ void rank_order_sum(const AllreduceOperands &op, int64_t at, float (&s)[VEC]) {
