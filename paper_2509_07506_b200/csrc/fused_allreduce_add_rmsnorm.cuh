@@ -215,9 +215,13 @@ fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands
 // are fetched group by group beside the body's.  (The plain loads and stores stay per-thread here too: a
 // partial or a destination may be another GPU's memory.)
 // Measured L2-cold, bf16, against the 2-, 4- and 8-byte vector kernels: see the launch code.
+// With four loads in flight the compiler is asked for no minimum of resident blocks: given one as a minimum it takes 76
+// and 134 registers (one and two vectors, 16-bit) instead of 64 and 128 with 16 and 28 bytes of spill, which
+// cost a block per SM: 96.8 -> 70.1 us at bf16 [4096, 7167] with 4 partials, 146 -> 113 at [4096, 8191] with 8, 46.6 ->
+// 40.6 at [4096, 4099] with 4, 47.7 -> 38.7 at fp32 [2048, 4095] with 4 (12.2 -> 13.6 at bf16 [500, 5123] with 8).
 template <int DT, int VPT, int GROUP, bool LATE_R = false>
 __global__ void __launch_bounds__(LATE_R ? kAllreduceLateThreads : VPT == 4 ? 512 : allreduce_reg_max_threads(16 * VPT, GROUP),
-                                  LATE_R ? 2 : 1)
+                                  LATE_R ? 2 : GROUP == 4 ? 0 : 1)
 fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOperands op,
                                           const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
@@ -375,8 +379,8 @@ constexpr WideShape kWideShapes[2][kWideShapeCount] = {
     {{1, 4, 64, 512, 128}, {2, 4, 112, 256, 64}, {1, 2, 48, 1024, 128}, {2, 2, 80, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}}};  // binary32
 // The same shapes of the ragged kernel, with its registers.
 constexpr WideShape kRaggedShapes[2][kWideShapeCount] = {
-    {{1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 120, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}},
-    {{1, 4, 64, 512, 64}, {2, 4, 120, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 96, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}}};
+    {{1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 112, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}},
+    {{1, 4, 64, 512, 64}, {2, 4, 120, 256, 64}, {1, 2, 56, 1024, 64}, {2, 2, 96, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}}};
 constexpr int64_t kWideBytesInFlight = 90 * 1024;
 
 // Blocks that an SM holds at once.  Each of its four partitions has 16384 registers, hands them out warp by
@@ -409,8 +413,9 @@ inline AllreduceShape allreduce_wide_shape(int64_t T, int units, int n_parts, bo
         threads_for(1) <= allreduce_reg_max_threads(16, kDeepGroup))
         return {1, kDeepGroup, threads_for(1)};
     // Blocks without a row are not resident: binary32 rows of 11008 units keep one vector per thread up to 148 rows
-    // (4.7 against 6.5 us at [16, 6144] with 8 partials), and threads beyond the row's vectors have no loads.  The ragged kernel's edge wants both all the same
-    // (3.3 against 4.9 us at bf16 [500, 1059] with 2, 2.9 against 4.1 us at [150, 1603]).
+    // (4.7 against 6.5 us at [16, 6144] with 8 partials), and threads beyond the row's vectors have no loads.  The
+    // ragged kernel's edge wants both all the same (3.3 against 4.9 us at bf16 [500, 1059] with 2, 2.9 against 4.1
+    // us at [150, 1603]), but no late residual for blocks that are not there (3.4 against 3.9 us at fp32 [150, 3202]).
     const int64_t rows_per_sm = (T + kOneBlockRows - 1) / kOneBlockRows;
     AllreduceShape best;
     int64_t best_bytes = 0;
@@ -420,7 +425,7 @@ inline AllreduceShape allreduce_wide_shape(int64_t T, int units, int n_parts, bo
         const int threads = threads_for(sh.vpt);
         if (threads > sh.max_threads || threads < sh.min_threads) continue;
         int64_t resident = resident_blocks(sh.regs, threads);
-        if (!ragged && resident > rows_per_sm) resident = rows_per_sm;
+        if ((!ragged || sh.late) && resident > rows_per_sm) resident = rows_per_sm;
         const int64_t vectors = ragged ? threads * sh.vpt : nvec;
         const int64_t bytes = resident * vectors * (sh.group + (sh.late ? 0 : 1)) * 32;
         if (bytes > best_bytes) {
