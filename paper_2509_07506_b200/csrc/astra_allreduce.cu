@@ -201,19 +201,9 @@ cudaError_t dispatch(const AllreduceOperands &op, const uint16_t *w, int64_t T, 
         if (launch_wide<DT, false>(op, w, T, H, eps, stream, &err)) return err;
         pick.vec = 8;  // everything that is 32-byte aligned is 16-byte aligned
     }
-    // Rows of less than 16-byte alignment go to the ragged kernel (figures there), except where the 8-byte
-    // forms are the faster ones: few rows, whose latency their smaller code serves better (1.8 against 2.1 us
-    // at [16, 4100] with 2 partials, 3.3 against 4.2 us at [140, 4100] with 4, 4.35 against 4.6 us at [64, 8188]
-    // with 8; but 7.5 -> 6.1 us at [16, 14332] with 8, 5.8 -> 3.8 us at fp32 [16, 4098]), two or three partials
-    // up to 512 rows (4.05 against 4.5 us at [400, 4100]; 9.1 -> 7.1 us at [512, 4100] with 4), and binary32 rows
-    // of 10241 to 16384 units (41.2 against 45.9 us at fp32 [1024, 8190] with 4; 27.5 -> 13.2 us at [512, 5001]
-    // and 130 -> 80 us at [1024, 16382], which take two sweeps otherwise).
-    const int64_t units = static_cast<int64_t>(H) * Storage<DT>::UNITS;
-    const bool few = T <= kOneBlockRows;
-    const bool narrow_form =
-        pick.vec == 4 && (DT == ASTRA_FP32 ? (units > 10240 && units <= 16384) || (op.n_parts < 4 && few && units <= 16384)
-                                           : (op.n_parts < 4 && T <= 512) || (units <= 8192 && few));
-    if (pick.vec < 8 && !narrow_form && rows_together(op)) {
+    // Rows of less than 16-byte alignment go to the ragged kernel, except where the narrow forms are the faster.
+    const int units = H * Storage<DT>::UNITS;
+    if (pick.vec < 8 && !allreduce_keeps_narrow(T, units, op.n_parts, DT == ASTRA_FP32, pick.vec) && rows_together(op)) {
         cudaError_t err = cudaSuccess;
         if (launch_wide<DT, true>(op, w, T, H, eps, stream, &err)) return err;
     }

@@ -439,6 +439,31 @@ inline AllreduceShape allreduce_wide_shape(int64_t T, int units, int n_parts, bo
     return best;
 }
 
+// Do T rows of `units` units that start at no 16-byte boundary stay with the 2-, 4- or 8-byte forms (vec = 1, 2, 4
+// units), or do they go to the ragged kernel?  Only 8-byte forms are ever the faster, and short rows of 4-byte ones
+// that are few.  Their smaller code starts sooner and they keep eight loads in flight up to 296 rows, which counts
+// while a row is short or the SMs have few.  Narrow against ragged, bf16: 2.6 and 4.1 us at [150, 1060] with 8
+// partials, 3.0 and 4.0 us at [150, 3076] with 4, 3.4 and 4.1 us at [800, 1060] with 2, 18.4 and 21.3 us at [3000, 3588]
+// with 2; but 4.4 and 3.8 us at [150, 4100] with 4, 6.3 and 4.9 us at [300, 2084] with 8, 25.7 and 22.9 us at [1500, 5124] with 4, and
+// anything from there on.  binary32: 2.2 and 2.6 us at [150, 802] with 2, 3.1 and 3.7 us at [150, 602] with 8; 4.4
+// and 2.9 us at [150, 2050] with 4, 9.9 and 8.6 us at [1500, 2050] with 2; from 10241 to 16384 units the narrow forms are
+// the faster throughout (41.2 against 45.9 us at [1024, 8190] with 4).
+inline bool allreduce_keeps_narrow(int64_t T, int units, int n_parts, bool binary32, int vec) {
+    const bool few = T <= kOneBlockRows, several = T <= 2 * kOneBlockRows, short_rows = units < 4096;
+    if (vec != 4) return vec == 2 && !binary32 && units < 1536 && n_parts < 4 && T <= 160;
+    if (!binary32) {
+        if (n_parts < 4) return T <= 512 || short_rows;
+        if (few) return units <= 8192;
+        if (n_parts < 6) return (short_rows && T <= 512) || units < 2560;
+        return short_rows && several;
+    }
+    if (units > 10240) return units <= 16384;
+    if (few) return n_parts < 4 || short_rows || units > 8704 || (T > 128 && (n_parts < 6 || units < 8192));
+    if (n_parts == 2) return (units < 8192 && T <= (units < 4608 ? 400 : 200)) || (short_rows && T <= 512) || units < 2048;
+    if (n_parts < 4) return (short_rows && T <= 512) || units < 2048;
+    return (short_rows && several) || (n_parts < 6 && units < 2560);
+}
+
 // The rank-order sum of one vector position, GROUP partial loads in flight at a time.
 template <int DT, int VEC, int GROUP>
 __device__ __forceinline__ void rank_order_sum(const AllreduceOperands &op, int64_t at, float (&s)[VEC]) {

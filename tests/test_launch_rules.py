@@ -1,0 +1,52 @@
+"""The rules that choose between a kernel for rows that start anywhere (or one that asks for its inputs ahead of
+time) and the plain forms, at sizes where one of the two was measured to be the slower: the rules are host
+functions of the kernel headers, compiled into a small program."""
+import subprocess
+
+from paper_2509_07506_b200 import build as astra_build
+
+PROGRAM = r"""
+#include <cstdio>
+#include "fused_allreduce_add_rmsnorm.cuh"
+using namespace astra;
+
+static int failures = 0;
+#define EXPECT(want, call) do { if ((call) != (want)) { ++failures; printf("%s is not %s\n", #call, #want); } } while (0)
+
+static void allreduce() {
+    // (rows, units, partials, binary32, units per access of the narrow form)
+    EXPECT(true, allreduce_keeps_narrow(150, 1060, 8, false, 4));
+    EXPECT(true, allreduce_keeps_narrow(150, 3076, 4, false, 4));
+    EXPECT(true, allreduce_keeps_narrow(296, 3588, 8, false, 4));
+    EXPECT(true, allreduce_keeps_narrow(800, 1060, 2, false, 4));
+    EXPECT(true, allreduce_keeps_narrow(3000, 3588, 2, false, 4));
+    EXPECT(true, allreduce_keeps_narrow(16, 4100, 8, false, 4));
+    EXPECT(false, allreduce_keeps_narrow(150, 4100, 4, false, 4));
+    EXPECT(false, allreduce_keeps_narrow(300, 2084, 8, false, 4));
+    EXPECT(false, allreduce_keeps_narrow(1500, 5124, 4, false, 4));
+    EXPECT(false, allreduce_keeps_narrow(16, 14332, 8, false, 4));
+    EXPECT(true, allreduce_keeps_narrow(150, 1604, 2, true, 4));
+    EXPECT(true, allreduce_keeps_narrow(150, 1204, 8, true, 4));
+    EXPECT(true, allreduce_keeps_narrow(16, 9220, 4, true, 4));
+    EXPECT(true, allreduce_keeps_narrow(1024, 16380, 4, true, 4));
+    EXPECT(false, allreduce_keeps_narrow(150, 4100, 4, true, 4));
+    EXPECT(false, allreduce_keeps_narrow(1500, 4100, 2, true, 4));
+    EXPECT(false, allreduce_keeps_narrow(1024, 16388, 4, true, 4));
+    for (int units : {1027, 4099, 16387})
+        for (int T : {1, 150, 4096}) EXPECT(false, allreduce_keeps_narrow(T, units, 4, false, 1));
+}
+
+int main() {
+    allreduce();
+    return failures != 0;
+}
+"""
+
+
+def test_rules_at_sizes_that_were_measured(tmp_path):
+    src, exe = tmp_path / "rules.cu", tmp_path / "rules"
+    src.write_text(PROGRAM)
+    subprocess.check_call([astra_build._nvcc(), "-std=c++17", "-O1", "-gencode", "arch=compute_100a,code=sm_100a",
+                           "-I", astra_build.INCLUDE, "-I", astra_build.CSRC, "-o", str(exe), str(src)])
+    done = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert done.returncode == 0, done.stdout
