@@ -447,7 +447,7 @@ bool try_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T,
                           (reinterpret_cast<uintptr_t>(op.y) - at) % 32 == 0 &&
                           (reinterpret_cast<uintptr_t>(op.r_out) - at) % 32 == 0;
     if (!together || Hu < kRmsnormRaggedMinUnits) return false;
-    const RaggedShape sh = rmsnorm_ragged_shape(T, Hu, DT == ASTRA_FP32, vec == 4);
+    const RaggedShape sh = rmsnorm_ragged_shape(T, Hu, DT == ASTRA_FP32, vec);
     if (sh.vpt == 1) *err = launch_rmsnorm_ragged<DT, 1, true>(op, w, T, H, sh.threads, eps, stream);
     else if (sh.vpt == 2) *err = launch_rmsnorm_ragged<DT, 2, false>(op, w, T, H, sh.threads, eps, stream);
     else if (sh.vpt == 4) {
@@ -467,11 +467,7 @@ cudaError_t dispatch_rmsnorm(const RmsnormOperands &op, const uint16_t *w, int64
         if (launch_rmsnorm_wide<DT>(op, w, T, H, eps, stream, &err)) return err;
         vec = 8;  // everything that is 32-byte aligned is 16-byte aligned
     }
-    // Aligned binary32 rows of more than 16384 units also hold their sums in one block there, which beats the
-    // clusters once there are rows for every SM: 51.6 -> 42.8 us at [1024, 16384], 35.6 -> 31.4 at [1024, 11008],
-    // 7.1 -> 6.5 at [128, 16384] (2.9 against 4.9 us at [16, 16384]).
-    const bool wide_fp32 = DT == ASTRA_FP32 && 2 * static_cast<int64_t>(H) > 32 * kRmsnormRaggedMaxThreads &&
-                           T > kRmsnormRaggedWideRows;
+    const bool wide_fp32 = DT == ASTRA_FP32 && 2 * static_cast<int64_t>(H) > 32 * kRmsnormRaggedMaxThreads;
     if (vec < 8 || wide_fp32) {
         cudaError_t err = cudaSuccess;
         if (try_rmsnorm_ragged<DT>(op, w, T, H, vec, eps, stream, &err)) return err;

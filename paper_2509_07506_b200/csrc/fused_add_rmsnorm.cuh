@@ -281,30 +281,70 @@ __device__ __forceinline__ void ragged_finish(const RaggedRow &g, const uint16_t
 // Two vectors per thread hold the sums of 16384 units in two blocks of 512 threads per SM at 64 registers.
 constexpr int kRmsnormRaggedMaxThreads = 512, kRmsnormRaggedMinThreads = 64;
 
+// Blocks that an SM holds at once.  Each of its four partitions has 16384 registers, hands them out warp by
+// warp in pieces of 256, and a block needs a place for each of its warps: 21 warps of 48 registers fit once, not
+// twice, although 2 * 21 * 32 * 48 registers are fewer than 65536 (counting them as two took fp32 [1024, 5152] with
+// 2 partials from 17.2 to 20.5 us).
+inline int resident_blocks(int regs, int threads) {
+    const int warps = (threads + 31) / 32;
+    const int by_regs = 4 * (16384 / ((regs * 32 + 255) / 256 * 256)) / warps, by_threads = 64 / warps;
+    return by_regs < by_threads ? by_regs : by_threads;
+}
+
+// Do T rows of `units` units stay with the other kernels, whose accesses there are of vec = 1, 2, 4 units (8: aligned
+// binary32 rows of more than 16384)?  `resident`: blocks of the ragged kernel per SM.
+// Odd rows never stay: 19 to 28 against 4 to 7 us at bf16 [400, 8195], 0.6 to 0.8 of the time elsewhere.  4-byte forms only
+// where rows are short and about as many as fill the SMs once with the narrow kernel's smaller blocks (1.9 against 2.1
+// us at bf16 [400, 1058], where the ragged kernel is at 0.7 to 0.9 of the time from 1800 units on).
+// The 8-byte forms move half the instructions of the 4-byte ones and are level or faster (1.9 against 2.1 us at bf16
+// [400, 1060], 2.3 and 2.6 at [256, 3164], 3.2 and 3.8 at fp32 [400, 2050]) except where the ragged kernel's one trip is a
+// short one (1.90 -> 1.71 us at bf16 [8, 4100]), its wider accesses stream (83.1 -> 81.5 us at [16384, 4100], 4.8 -> 4.1 at
+// [600, 4100]), or the rows fit the SMs in one wave of one kernel and not of the other (4.6 -> 4.2 us at bf16 [450, 8196],
+// 5.0 against 5.6 at [1500, 2084]).
+// Rows of more than 16384 units are otherwise clusters' or swept twice: 7.4 -> 3.7 us at bf16 [128, 16388], 51.6 -> 42.8 at
+// fp32 [1024, 16384], 35.6 -> 31.4 at [1024, 11008], 7.1 -> 6.5 at [128, 16384]; but clusters spread a row over several SMs and
+// are ahead while rows are few (3.1 against 4.9 us at fp32 [16, 16382], 4.9 and 5.1 at 64 rows, 9.5 and 6.5 at 128; 2.6
+// and 3.0 at bf16 [8, 16388]), and where one block fills an SM and a few rows start a second wave (6.1 against 6.8 us at
+// fp32 [149 ... 170, 11008]).
+inline bool rmsnorm_keeps_narrow(int64_t T, int64_t units, bool binary32, int vec, int resident) {
+    const int64_t rows_per_sm = (T + 147) / 148;
+    if (vec == 1) return false;
+    if (vec == 2) return units < 1536 && T >= 192 && T <= 560;
+    if (vec == 8 || units > 16400) return T <= 64 || (units > 18432 && units <= 26624 && T > 148 && T <= 176);
+    if (units > 16384) return T <= 32;
+    if (units < 2048) return true;
+    if (T <= 112) return binary32 ? T > 8 || units > 4608 : T * units > 270000 || units > 6144;
+    const int64_t narrow_resident = 64 / ((units + 511) / 512);  // 16 units per thread, every warp slot
+    if (T > 256 && rows_per_sm > narrow_resident && rows_per_sm <= resident) return false;
+    if (T > 256 && rows_per_sm <= narrow_resident && rows_per_sm > resident) return true;
+    if (T <= 512) return T <= 384 || units <= 4608 || units > 6144;
+    return (units < 2560 && T < 800) || (units > 6144 && units <= 10240);
+}
+
 // Vectors per thread and block size for T rows of `units` units; vpt = 0 where the ragged kernel does not
 // apply.  A block has at least 64 threads, one per unit of the longest edge, also where fewer could hold the body.
 // One vector per thread up to 320 threads, then two (up to 512 threads), then, for binary32 rows only (half
 // the sums per unit), four: 21.3 us with one and 21.6 with two at [4096, 4099], 45.1 and 41.4 us at [4096, 8188],
 // 39.2 and 28.8 us at [2048, 11007].  Two also where that makes one wave of what would be a little more (5
-// blocks of 256 threads per SM at 48 registers against 8 of 128 at 64: 6.8 -> 6.6 us at [1024, 4101]).  A few wide
-// rows of 8-byte vectors are left to the clusters, which spread each over several SMs (3.1 against 4.9 us at
-// fp32 [16, 16382], 4.9 and 5.1 at 64 rows, 9.5 and 6.5 at 128).
+// blocks of 256 threads per SM at 48 registers against 8 of 128 at 64: 6.8 -> 6.6 us at [1024, 4101]).
 struct RaggedShape {
     int vpt, threads;
 };
-constexpr int64_t kRmsnormRaggedWideRows = 64;
-inline RaggedShape rmsnorm_ragged_shape(int64_t T, int64_t units, bool binary32, bool vec8_byte) {
+inline RaggedShape rmsnorm_ragged_shape(int64_t T, int64_t units, bool binary32, int vec) {
     const int64_t nvec = units / 16;
     auto threads_for = [&](int v) {
         const int64_t t = ((nvec + v - 1) / v + 31) / 32 * 32;
         return static_cast<int>(t < kRmsnormRaggedMinThreads ? kRmsnormRaggedMinThreads : t);
     };
     const int64_t wave1 = 148 * (65536 / (48 * threads_for(1))), wave2 = 148 * (65536 / (64 * threads_for(2)));
-    if (nvec <= 320 && !(T > wave1 && T <= wave2)) return {1, threads_for(1)};
-    if (nvec <= 2 * kRmsnormRaggedMaxThreads) return {2, threads_for(2)};
-    if (binary32 && nvec <= 4 * kRmsnormRaggedMaxThreads && !(vec8_byte && T <= kRmsnormRaggedWideRows))
-        return {4, threads_for(4)};
-    return {0, 0};
+    RaggedShape sh = {0, 0};
+    if (nvec <= 320 && !(T > wave1 && T <= wave2)) sh = {1, threads_for(1)};
+    else if (nvec <= 2 * kRmsnormRaggedMaxThreads) sh = {2, threads_for(2)};
+    else if (binary32 && nvec <= 4 * kRmsnormRaggedMaxThreads) sh = {4, threads_for(4)};
+    if (sh.vpt == 0) return sh;
+    const int regs = sh.vpt == 1 ? (binary32 ? 40 : 48) : sh.vpt == 2 ? (binary32 ? 56 : 64) : 96;
+    if (rmsnorm_keeps_narrow(T, units, binary32, vec, resident_blocks(regs, sh.threads))) return {0, 0};
+    return sh;
 }
 
 template <int DT, int VPT, bool EARLY_W>

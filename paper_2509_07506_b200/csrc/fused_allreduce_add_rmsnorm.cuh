@@ -349,7 +349,7 @@ fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOpera
 // Five shapes: one or two vectors per thread (16 or 32 units), two or four partial loads in flight
 // (four only from four partials on), and two of each with the residual requested last.  What decides
 // between them is how many bytes of loads an SM has in flight, i.e. resident blocks x threads x bytes per
-// thread, with the resident blocks set by the registers (as compiled for sm_100a).  The measurements across H = 2048 ... 16384 fit one rule: take the first shape, in the
+// thread, with the blocks that are resident (resident_blocks, registers as compiled for sm_100a).  The measurements across H = 2048 ... 16384 fit one rule: take the first shape, in the
 // order below, that keeps about 90 KB in flight per SM; if none does, the one with the most.  Examples:
 // H = 4096 takes one vector and four in flight (three 256-thread blocks per SM); H = 8192 with four
 // in flight would leave one 512-thread block per SM, so it takes two vectors in 256-thread blocks
@@ -382,16 +382,6 @@ constexpr WideShape kRaggedShapes[2][kWideShapeCount] = {
     {{1, 4, 64, 512, 64}, {2, 4, 128, 256, 64}, {1, 2, 64, 1024, 64}, {2, 2, 112, 512, 64}, {2, 2, 72, kAllreduceLateThreads, 64, true}},
     {{1, 4, 64, 512, 64}, {2, 4, 120, 256, 64}, {1, 2, 56, 1024, 64}, {2, 2, 96, 512, 64}, {2, 2, 64, kAllreduceLateThreads, 64, true}}};
 constexpr int64_t kWideBytesInFlight = 90 * 1024;
-
-// Blocks that an SM holds at once.  Each of its four partitions has 16384 registers, hands them out warp by
-// warp in pieces of 256, and a block needs a place for each of its warps: 21 warps of 48 registers fit once, not
-// twice, although 2 * 21 * 32 * 48 registers are fewer than 65536 (counting them as two took fp32 [1024, 5152] with
-// 2 partials from 17.2 to 20.5 us).
-inline int resident_blocks(int regs, int threads) {
-    const int warps = (threads + 31) / 32;
-    const int by_regs = 4 * (16384 / ((regs * 32 + 255) / 256 * 256)) / warps, by_threads = 64 / warps;
-    return by_regs < by_threads ? by_regs : by_threads;
-}
 
 // Shape for T rows of `units` 16-bit units with n_parts partials; vpt = 0 where none applies (rows too narrow for
 // 128-thread blocks, ragged ones for 64, or too wide).

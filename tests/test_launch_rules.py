@@ -36,8 +36,36 @@ static void allreduce() {
         for (int T : {1, 150, 4096}) EXPECT(false, allreduce_keeps_narrow(T, units, 4, false, 1));
 }
 
+static bool norm_is_ragged(int64_t T, int64_t units, bool binary32, int vec) {
+    return rmsnorm_ragged_shape(T, units, binary32, vec).vpt > 0;
+}
+
+static void norm() {
+    EXPECT(false, norm_is_ragged(400, 1060, false, 4));
+    EXPECT(false, norm_is_ragged(256, 3164, false, 4));
+    EXPECT(false, norm_is_ragged(400, 4100, false, 4));
+    EXPECT(false, norm_is_ragged(8, 16388, false, 4));
+    EXPECT(false, norm_is_ragged(400, 1058, false, 2));
+    EXPECT(false, norm_is_ragged(1500, 2084, false, 4));
+    EXPECT(false, norm_is_ragged(400, 4100, true, 4));
+    EXPECT(false, norm_is_ragged(128, 5124, true, 4));
+    EXPECT(false, norm_is_ragged(16, 32768, true, 8));
+    EXPECT(false, norm_is_ragged(160, 22016, true, 8));
+    EXPECT(true, norm_is_ragged(8, 4100, false, 4));
+    EXPECT(true, norm_is_ragged(600, 4100, false, 4));
+    EXPECT(true, norm_is_ragged(450, 8196, false, 4));
+    EXPECT(true, norm_is_ragged(16384, 4100, false, 4));
+    EXPECT(true, norm_is_ragged(128, 16388, false, 4));
+    EXPECT(true, norm_is_ragged(1000, 2050, false, 2));
+    EXPECT(true, norm_is_ragged(1024, 32768, true, 8));
+    EXPECT(true, norm_is_ragged(149, 32768, true, 8));
+    for (int units : {1027, 4099, 16383})
+        for (int T : {1, 150, 4096}) EXPECT(true, norm_is_ragged(T, units, false, 1));
+}
+
 int main() {
     allreduce();
+    norm();
     return failures != 0;
 }
 """

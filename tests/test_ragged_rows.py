@@ -74,10 +74,11 @@ int main() {
     for (int units : widths)
         for (bool binary32 : {false, true}) {
             std::set<std::pair<int, int>> shapes;
-            for (int T = 1; T <= 6000; ++T) {
-                const RaggedShape sh = rmsnorm_ragged_shape(T, units, binary32, T % 2 == 0);
-                if (sh.vpt > 0) shapes.insert({sh.vpt, sh.threads});
-            }
+            for (int T = 1; T <= 6000; ++T)
+                for (int vec : {1, 2, 4, 8}) {
+                    const RaggedShape sh = rmsnorm_ragged_shape(T, units, binary32, vec);
+                    if (sh.vpt > 0) shapes.insert({sh.vpt, sh.threads});
+                }
             expect(binary32 || units >= 16400 || !shapes.empty(), "shape", units, 0, 0, 0);
             for (auto [vpt, threads] : shapes)
                 for (long row = 0; row < 16; ++row)
