@@ -226,11 +226,16 @@ cudaError_t launch_merge_strided(uint16_t *v_out, float *lse_out, const uint16_t
         const uint32_t tile = THREADS * UNROLL;
         const uint32_t blocks = (total + tile - 1) / tile;
         const FastDiv per_row = FastDiv::make(static_cast<uint32_t>(nvec)), heads = FastDiv::make(static_cast<uint32_t>(Hh));
-        const cudaError_t err =
-            dense ? launch(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, true>, blocks, THREADS, stream,
-                           v_out, lse_out, v_a, lse_a, v_b, lse_b, total, static_cast<uint32_t>(r0), per_row, heads, st)
-                  : launch(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, false>, blocks, THREADS, stream,
-                           v_out, lse_out, v_a, lse_a, v_b, lse_b, total, static_cast<uint32_t>(r0), per_row, heads, st);
+        auto issue = [&](auto kernel) {
+            return launch(kernel, blocks, THREADS, stream, v_out, lse_out, v_a, lse_a, v_b, lse_b, total,
+                          static_cast<uint32_t>(r0), per_row, heads, st);
+        };
+        cudaError_t err;
+        switch (merge_strided_reads(blocks, (tile + nvec - 1) / nvec, dense)) {
+            case MergeReads::Few: err = issue(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, MergeReads::Few>); break;
+            case MergeReads::Dense: err = issue(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, MergeReads::Dense>); break;
+            default: err = issue(merge_attn_states_lse_strided_kernel<DT, VEC, UNROLL, THREADS, MergeReads::Rows>); break;
+        }
         if (err != cudaSuccess) return err;
     }
   }

@@ -113,13 +113,23 @@ merge_attn_states_lse_kernel(uint16_t *v_out, float *lse_out,
 
 namespace astra {
 
+// How the kernel below reads: FEW asks for nothing ahead of the dependency wait; DENSE takes the three value tensors
+// as dense [T, Hh, D] (the usual case of head-major scores), addresses their vectors flat, and a block asks for its
+// share of each input, one contiguous range, ahead of the wait, as above; ROWS has a thread per row ask for that row.
+// A request costs its block time, most where 32 or 64 threads make one each, and pays once the grid's loads queue
+// for memory.  FEW against ROWS, L2-cold: 1.17 and 1.97 us at fp32 [8, 32, 64], 1.33 and 2.0 at bf16 [64, 32, 64], 2.0 and 2.35
+// at bf16 [64, 32, 128]; but 3.0 and 2.46 at bf16 [1024, 32, 128], 2.87 and 2.55 at fp32 [256, 20, 128].  FEW against DENSE:
+// 1.33 and 1.44 at bf16 [16, 40, 128], 1.12 and 1.22 at fp32 [8, 20, 128]; but 2.0 and 1.88 at bf16 [64, 32, 128].
+enum class MergeReads { Few, Dense, Rows };
+inline MergeReads merge_strided_reads(int64_t blocks, int64_t rows_per_block, bool dense) {
+    if (blocks < (dense || rows_per_block <= 8 ? 56 : rows_per_block <= 16 ? 64 : 240)) return MergeReads::Few;
+    return dense ? MergeReads::Dense : MergeReads::Rows;
+}
+
 // Same computation for arbitrarily strided tensors (head_dim contiguous): row = token * Hh + head is
 // split again into (token, head) to address each tensor by its own strides.  This is the form for
 // head-major scores ([Hh, T]) or values that are slices of a wider buffer.
-// DENSE_VALUES: the three value tensors are dense [T, Hh, D] (the usual case of head-major scores), so their
-// vectors are addressed flat and a block's share of each input is one contiguous range, which it asks for
-// ahead of the dependency wait, as above; otherwise a thread per row asks for that row.
-template <int DT, int VEC, int UNROLL, int THREADS, bool DENSE_VALUES>
+template <int DT, int VEC, int UNROLL, int THREADS, MergeReads READS>
 __global__ void __launch_bounds__(THREADS)
 merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
                                      const uint16_t *v_a, const float *lse_a,
@@ -127,65 +137,81 @@ merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
                                      uint32_t total_vecs, uint32_t row0, FastDiv nvec, FastDiv heads,
                                      MergeStrides st) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
+    constexpr bool FLAT = READS == MergeReads::Dense;
     const uint32_t first = blockIdx.x * (THREADS * UNROLL);
     const uint32_t base = first + threadIdx.x;
-    const uint32_t count = min(static_cast<uint32_t>(THREADS * UNROLL), total_vecs - first);
     const int64_t flat0 = static_cast<int64_t>(row0) * nvec.d;  // the launch's first vector in a dense tensor
-    if constexpr (DENSE_VALUES) {
-        if (threadIdx.x == 0) {
-            prefetch_l2_range(v_a + (flat0 + first) * UV, static_cast<int64_t>(count) * UV * 2);
-            prefetch_l2_range(v_b + (flat0 + first) * UV, static_cast<int64_t>(count) * UV * 2);
-        }
-    } else {
-        const uint32_t lrow = nvec.div(first) + threadIdx.x;
-        if (lrow <= nvec.div(first + count - 1)) {
-            const uint32_t row = row0 + lrow, t = heads.div(row), h = row - t * heads.d;
-            const int64_t bytes = static_cast<int64_t>(nvec.d) * UV * 2;
-            prefetch_l2_range(v_a + (t * st.va_t + h * st.va_h), bytes);
-            prefetch_l2_range(v_b + (t * st.vb_t + h * st.vb_h), bytes);
+    if constexpr (READS != MergeReads::Few) {
+        const uint32_t count = min(static_cast<uint32_t>(THREADS * UNROLL), total_vecs - first);
+        if constexpr (FLAT) {
+            if (threadIdx.x == 0) {
+                prefetch_l2_range(v_a + (flat0 + first) * UV, static_cast<int64_t>(count) * UV * 2);
+                prefetch_l2_range(v_b + (flat0 + first) * UV, static_cast<int64_t>(count) * UV * 2);
+            }
+        } else {
+            const uint32_t lrow = nvec.div(first) + threadIdx.x;
+            if (lrow <= nvec.div(first + count - 1)) {
+                const uint32_t row = row0 + lrow, t = heads.div(row), h = row - t * heads.d;
+                const int64_t bytes = static_cast<int64_t>(nvec.d) * UV * 2;
+                prefetch_l2_range(v_a + (t * st.va_t + h * st.va_h), bytes);
+                prefetch_l2_range(v_b + (t * st.vb_t + h * st.vb_h), bytes);
+            }
         }
     }
     grid_dependency_wait();
     grid_launch_dependents();
     Pack<UV> a[UNROLL], b[UNROLL];
     float sa[UNROLL], sb[UNROLL];
+    struct Place {
+        uint32_t v, t, h;
+        int64_t col;
+    };
+    auto place = [&](int j) {
+        Place p;
+        p.v = base + j * THREADS;
+        const uint32_t lrow = nvec.div(p.v);
+        const uint32_t row = row0 + lrow;  // rows of this launch start at row0
+        p.t = heads.div(row);
+        p.h = row - p.t * heads.d;
+        p.col = static_cast<int64_t>(p.v - lrow * nvec.d) * UV;
+        return p;
+    };
+    auto fetch = [&](int j, const Place &p) {
+        a[j] = load<UV, Ld::Stream>(v_a + (FLAT ? (flat0 + p.v) * UV : p.t * st.va_t + p.h * st.va_h + p.col));
+        b[j] = load<UV, Ld::Stream>(v_b + (FLAT ? (flat0 + p.v) * UV : p.t * st.vb_t + p.h * st.vb_h + p.col));
+        sa[j] = lse_a[p.t * st.sa_t + p.h * st.sa_h];
+        sb[j] = lse_b[p.t * st.sb_t + p.h * st.sb_h];
+    };
+    auto finish = [&](int j, const Place &p) {
+        const MergeWeights mw = merge_weights(sa[j], sb[j]);
+        float fa[VEC], fb[VEC], fo[VEC];
+        widen<DT, VEC>(a[j], fa);
+        widen<DT, VEC>(b[j], fb);
 #pragma unroll
-    for (int j = 0; j < UNROLL; ++j) {
-        const uint32_t v = base + j * THREADS;
-        if (v < total_vecs) {
-            const uint32_t lrow = nvec.div(v);
-            const int64_t col = static_cast<int64_t>(v - lrow * nvec.d) * UV;
-            const uint32_t row = row0 + lrow;  // rows of this launch start at row0
-            const uint32_t t = heads.div(row);
-            const uint32_t h = row - t * heads.d;
-            a[j] = load<UV, Ld::Stream>(v_a + (DENSE_VALUES ? (flat0 + v) * UV : t * st.va_t + h * st.va_h + col));
-            b[j] = load<UV, Ld::Stream>(v_b + (DENSE_VALUES ? (flat0 + v) * UV : t * st.vb_t + h * st.vb_h + col));
-            sa[j] = lse_a[t * st.sa_t + h * st.sa_h];
-            sb[j] = lse_b[t * st.sb_t + h * st.sb_h];
+        for (int i = 0; i < VEC; ++i) {
+            const float ta = mw.use_a ? fa[i] * mw.wa : 0.f;
+            fo[i] = mw.use_b ? fmaf(fb[i], mw.wb, ta) : ta;
         }
-    }
+        store<UV, St::Stream>(v_out + (FLAT ? (flat0 + p.v) * UV : p.t * st.vo_t + p.h * st.vo_h + p.col),
+                              narrow<DT, VEC>(fo));
+        if (lse_out != nullptr && p.col == 0) lse_out[p.t * st.so_t + p.h * st.so_h] = mw.lse;
+    };
+    if constexpr (READS == MergeReads::Few) {
 #pragma unroll
-    for (int j = 0; j < UNROLL; ++j) {
-        const uint32_t v = base + j * THREADS;
-        if (v < total_vecs) {
-            const uint32_t lrow = nvec.div(v);
-            const int64_t col = static_cast<int64_t>(v - lrow * nvec.d) * UV;
-            const uint32_t row = row0 + lrow;
-            const uint32_t t = heads.div(row);
-            const uint32_t h = row - t * heads.d;
-            const MergeWeights mw = merge_weights(sa[j], sb[j]);
-            float fa[VEC], fb[VEC], fo[VEC];
-            widen<DT, VEC>(a[j], fa);
-            widen<DT, VEC>(b[j], fb);
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                const float ta = mw.use_a ? fa[i] * mw.wa : 0.f;
-                fo[i] = mw.use_b ? fmaf(fb[i], mw.wb, ta) : ta;
+        for (int j = 0; j < UNROLL; ++j) {
+            if (base + j * THREADS < total_vecs) {
+                const Place p = place(j);
+                fetch(j, p);
+                finish(j, p);
             }
-            store<UV, St::Stream>(v_out + (DENSE_VALUES ? (flat0 + v) * UV : t * st.vo_t + h * st.vo_h + col),
-                                  narrow<DT, VEC>(fo));
-            if (lse_out != nullptr && col == 0) lse_out[t * st.so_t + h * st.so_h] = mw.lse;
         }
+    } else {
+#pragma unroll
+        for (int j = 0; j < UNROLL; ++j)
+            if (base + j * THREADS < total_vecs) fetch(j, place(j));
+#pragma unroll
+        for (int j = 0; j < UNROLL; ++j)
+            if (base + j * THREADS < total_vecs) finish(j, place(j));
     }
 }
 

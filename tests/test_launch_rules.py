@@ -8,6 +8,7 @@ from paper_2509_07506_b200 import build as astra_build
 PROGRAM = r"""
 #include <cstdio>
 #include "fused_allreduce_add_rmsnorm.cuh"
+#include "merge_attn_states_lse.cuh"
 using namespace astra;
 
 static int failures = 0;
@@ -63,9 +64,23 @@ static void norm() {
         for (int T : {1, 150, 4096}) EXPECT(true, norm_is_ragged(T, units, false, 1));
 }
 
+static void merge() {
+    // (blocks, rows per block, dense values)
+    EXPECT(MergeReads::Few, merge_strided_reads(4, 32, false));     // fp32 [8, 32, 64]
+    EXPECT(MergeReads::Few, merge_strided_reads(64, 32, false));    // bf16 [64, 32, 128]
+    EXPECT(MergeReads::Few, merge_strided_reads(160, 64, false));   // bf16 [256, 40, 64]
+    EXPECT(MergeReads::Few, merge_strided_reads(40, 16, false));    // bf16 [16, 40, 256]
+    EXPECT(MergeReads::Few, merge_strided_reads(20, 32, true));     // bf16 [16, 40, 128]
+    EXPECT(MergeReads::Rows, merge_strided_reads(1024, 32, false)); // bf16 [1024, 32, 128]
+    EXPECT(MergeReads::Rows, merge_strided_reads(160, 8, false));   // fp32 [32, 40, 256]
+    EXPECT(MergeReads::Dense, merge_strided_reads(64, 32, true));   // bf16 [64, 32, 128]
+    EXPECT(MergeReads::Dense, merge_strided_reads(2560, 32, true)); // bf16 [2048, 40, 128]
+}
+
 int main() {
     allreduce();
     norm();
+    merge();
     return failures != 0;
 }
 """
