@@ -72,11 +72,6 @@ cudaError_t launch_silu(uint16_t *out, const uint16_t *gate, const uint16_t *up,
 // Rows that start at any element (see the kernel): one block per piece of about 192 granules of a row, the
 // pieces of a row equally long.  ALIGN = units to which every row start of every operand is aligned.
 constexpr int kSiluRaggedPiece = 192;
-#ifndef ASTRA_SILU_RAGGED_MIN_UNITS
-#define ASTRA_SILU_RAGGED_MIN_UNITS 1024
-#endif
-constexpr int64_t kSiluRaggedMinUnits = ASTRA_SILU_RAGGED_MIN_UNITS, kSiluRaggedMaxUnits = 1ll << 24;
-constexpr int64_t kSiluRaggedMaxTotal = 1ll << 24;  // units of output, for 8-byte vectors of the 16-bit types
 template <int DT, int ALIGN>
 cudaError_t launch_silu_ragged(uint16_t *out, const uint16_t *gate, const uint16_t *up, int64_t T, int64_t D,
                                int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch, cudaStream_t stream) {
@@ -118,14 +113,8 @@ cudaError_t dispatch_silu(uint16_t *out, const uint16_t *gate, const uint16_t *u
             return launch_silu<DT, 16, 1, 256>(out, gate, up, T, D, out_pitch, gate_pitch, up_pitch, stream);
         vec = 8;  // everything that is 32-byte aligned is 16-byte aligned
     }
-    // Narrower accesses than 16 bytes: rows that start anywhere go to the ragged kernel (figures there).
-    // Short rows of 4- and 8-byte vectors keep the flat forms (its blocks would be too small: 11.2 against
-    // 17.7 us at [16384, 514]), and so do long streams of 8-byte vectors of the 16-bit types (30.3 against
-    // 31.4 us at [8192, 4100], 50.4 against 53.5 us at [4000, 14332]; level at [4000, 4100], 6.0 -> 5.0 us at
-    // [1000, 4100], 14.0 -> 13.5 us at [1000, 14332]; fp32, with half the arithmetic per byte, gains at every
-    // size: 29.7 -> 28.4 us at [4000, 4098]).
-    if (vec < 8 && D >= (vec == 1 ? kSiluRaggedMinUnits / 2 : kSiluRaggedMinUnits) && D <= kSiluRaggedMaxUnits &&
-        !(vec == 4 && DT != ASTRA_FP32 && T > kSiluRaggedMaxTotal / D) &&
+    // Narrower accesses than 16 bytes: rows that start anywhere go to the ragged kernel.
+    if (silu_takes_ragged(T, D, DT == ASTRA_FP32, vec) &&
         !overlaps(out, span_bytes(T, D, out_pitch, 2), gate, span_bytes(T, D, gate_pitch, 2)) &&
         !overlaps(out, span_bytes(T, D, out_pitch, 2), up, span_bytes(T, D, up_pitch, 2))) {
         switch (VecPick(8).extent(out_pitch).extent(gate_pitch).extent(up_pitch).pointer(out).pointer(gate).pointer(up).vec) {

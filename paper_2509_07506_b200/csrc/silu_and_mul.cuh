@@ -167,6 +167,24 @@ __host__ __device__ __forceinline__ RaggedGranule ragged_granule(const uint16_t 
     return g;
 }
 
+// Which rows of less than 16-byte alignment (vec units per access of the flat kernel) come here: not short rows of 4-
+// and 8-byte vectors, whose blocks would be too small (11.2 against 17.7 us at [16384, 514]), nor a single row of
+// them that is little longer, both of whose ends are loaded by element (1.07 against 1.14 us at [1, 1028]), nor long streams
+// of 8-byte vectors of the 16-bit types (30.3 against 31.4 us at [8192, 4100], 50.4 against 53.5 us at [4000, 14332]; level at
+// [4000, 4100], 6.0 -> 5.0 us at [1000, 4100], 14.0 -> 13.5 us at [1000, 14332]; fp32, with half the arithmetic per byte, gains
+// at every size: 29.7 -> 28.4 us at [4000, 4098]).
+#ifndef ASTRA_SILU_RAGGED_MIN_UNITS
+#define ASTRA_SILU_RAGGED_MIN_UNITS 1024
+#endif
+constexpr int64_t kSiluRaggedMinUnits = ASTRA_SILU_RAGGED_MIN_UNITS, kSiluRaggedMaxUnits = 1ll << 24;
+constexpr int64_t kSiluRaggedMaxTotal = 1ll << 24;  // units of output, for 8-byte vectors of the 16-bit types
+inline bool silu_takes_ragged(int64_t T, int64_t D, bool binary32, int vec) {
+    if (vec >= 8 || D > kSiluRaggedMaxUnits) return false;
+    if (vec == 1) return D >= kSiluRaggedMinUnits / 2;
+    return D >= kSiluRaggedMinUnits && T > (kSiluRaggedMinUnits * (vec == 4 ? 8 : 5) / 4 - 1) / D &&
+            !(vec == 4 && !binary32 && T > kSiluRaggedMaxTotal / D);
+}
+
 template <int DT, int ALIGN>
 __global__ void __launch_bounds__(kSiluRaggedMaxThreads, 8)
 silu_and_mul_ragged_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gate,

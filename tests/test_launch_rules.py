@@ -9,6 +9,7 @@ PROGRAM = r"""
 #include <cstdio>
 #include "fused_allreduce_add_rmsnorm.cuh"
 #include "merge_attn_states_lse.cuh"
+#include "silu_and_mul.cuh"
 using namespace astra;
 
 static int failures = 0;
@@ -77,10 +78,25 @@ static void merge() {
     EXPECT(MergeReads::Dense, merge_strided_reads(2560, 32, true)); // bf16 [2048, 40, 128]
 }
 
+static void silu() {
+    // (rows, units, binary32, units per access of the flat form)
+    EXPECT(false, silu_takes_ragged(1, 1028, false, 4));
+    EXPECT(false, silu_takes_ragged(1, 1026, false, 2));
+    EXPECT(false, silu_takes_ragged(16384, 516, false, 4));
+    EXPECT(false, silu_takes_ragged(8192, 4100, false, 4));
+    EXPECT(false, silu_takes_ragged(4, 14336, false, 8));
+    EXPECT(true, silu_takes_ragged(1, 1538, false, 2));
+    EXPECT(true, silu_takes_ragged(1, 3076, true, 4));
+    EXPECT(true, silu_takes_ragged(4, 1028, false, 4));
+    EXPECT(true, silu_takes_ragged(1, 515, false, 1));
+    EXPECT(true, silu_takes_ragged(8192, 8196, true, 4));
+}
+
 int main() {
     allreduce();
     norm();
     merge();
+    silu();
     return failures != 0;
 }
 """
