@@ -332,16 +332,15 @@ struct RaggedShape {
 };
 inline RaggedShape rmsnorm_ragged_shape(int64_t T, int64_t units, bool binary32, int vec) {
     const int64_t nvec = units / 16;
+    if (nvec > (binary32 ? 4 : 2) * kRmsnormRaggedMaxThreads) return {0, 0};
     auto threads_for = [&](int v) {
-        const int64_t t = ((nvec + v - 1) / v + 31) / 32 * 32;
-        return static_cast<int>(t < kRmsnormRaggedMinThreads ? kRmsnormRaggedMinThreads : t);
+        const int t = ((static_cast<int>(nvec) + v - 1) / v + 31) / 32 * 32;
+        return t < kRmsnormRaggedMinThreads ? kRmsnormRaggedMinThreads : t;
     };
     const int64_t wave1 = 148 * (65536 / (48 * threads_for(1))), wave2 = 148 * (65536 / (64 * threads_for(2)));
-    RaggedShape sh = {0, 0};
+    RaggedShape sh = {4, threads_for(4)};
     if (nvec <= 320 && !(T > wave1 && T <= wave2)) sh = {1, threads_for(1)};
     else if (nvec <= 2 * kRmsnormRaggedMaxThreads) sh = {2, threads_for(2)};
-    else if (binary32 && nvec <= 4 * kRmsnormRaggedMaxThreads) sh = {4, threads_for(4)};
-    if (sh.vpt == 0) return sh;
     const int regs = sh.vpt == 1 ? (binary32 ? 40 : 48) : sh.vpt == 2 ? (binary32 ? 56 : 64) : 96;
     if (rmsnorm_keeps_narrow(T, units, binary32, vec, resident_blocks(regs, sh.threads))) return {0, 0};
     return sh;

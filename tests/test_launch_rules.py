@@ -92,7 +92,18 @@ static void silu() {
     EXPECT(true, silu_takes_ragged(8192, 8196, true, 4));
 }
 
+static void largest() {  // the widest rows and the most of them that the entry points accept
+    for (int64_t units : {(1ll << 30) - 1, 1ll << 30, 700000003ll})
+        for (int64_t T : {1ll, 1ll << 31, 1ll << 40})
+            for (int vec : {1, 2, 4, 8})
+                for (bool binary32 : {false, true}) {
+                    EXPECT(false, norm_is_ragged(T, units, binary32, vec));
+                    for (bool ragged : {false, true}) EXPECT(0, allreduce_wide_shape(T, units, 4, binary32, ragged).vpt);
+                }
+}
+
 int main() {
+    largest();
     allreduce();
     norm();
     merge();
@@ -106,6 +117,7 @@ def test_rules_at_sizes_that_were_measured(tmp_path):
     src, exe = tmp_path / "rules.cu", tmp_path / "rules"
     src.write_text(PROGRAM)
     subprocess.check_call([astra_build._nvcc(), "-std=c++17", "-O1", "-gencode", "arch=compute_100a,code=sm_100a",
-                           "-I", astra_build.INCLUDE, "-I", astra_build.CSRC, "-o", str(exe), str(src)])
+                           "-Xcompiler", "-fsanitize=undefined,-fno-sanitize-recover=all", "-I", astra_build.INCLUDE, "-I", astra_build.CSRC,
+                           "-o", str(exe), str(src)])
     done = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
-    assert done.returncode == 0, done.stdout
+    assert done.returncode == 0, done.stdout + done.stderr
