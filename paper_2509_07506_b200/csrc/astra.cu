@@ -87,7 +87,8 @@ cudaError_t launch_silu_ragged(uint16_t *out, const uint16_t *gate, const uint16
         const cudaError_t err =
             launch(silu_and_mul_ragged_kernel<DT, ALIGN>, static_cast<unsigned>(rows * pieces), threads, stream,
                    out + t0 * out_pitch, gate + t0 * gate_pitch, up + t0 * up_pitch,
-                   FastDiv::make(static_cast<uint32_t>(pieces)), static_cast<uint32_t>(rows - 1), static_cast<int>(D),
+                   FastDiv::make(static_cast<uint32_t>(pieces)),
+                   silu_ragged_end_rows(static_cast<uint32_t>(rows), gate, up, D, gate_pitch, up_pitch), static_cast<int>(D),
                    out_pitch, gate_pitch, up_pitch);
         if (err != cudaSuccess) return err;
     }

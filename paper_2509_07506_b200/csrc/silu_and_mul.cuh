@@ -144,11 +144,11 @@ template <int DT, int UV> __device__ __forceinline__ Pack<UV> silu_mul_pack(cons
 // the neighbour's granule by shuffles (18.6 and 43.9 us), two granules per thread (16.5 us), 32-byte
 // granules (16.0 and 37.7 us), blocks of 256 and 448 threads instead of about 192 (14.7 and 15.9 us).
 //
-// Accesses stay inside the tensors: a granule of a row other than the launch's first and last may reach
-// up to 14 units into the row before it or 15 into the one after, which exist (the launch code asks for
-// rows of at least 16 units, and that the output shares no address range with the inputs, so that
-// nothing that is written is read); the first and last row load the few granules that would pass their
-// ends element by element, and so are the ends of every output row stored.
+// Accesses stay inside mapped memory: a granule of a row other than the launch's first and last may reach up to 14
+// units into what lies before it or 15 into what lies after, which silu_ragged_end_rows makes sure of (and the
+// launch code that the output shares no address range with the inputs, so that nothing that is written is read);
+// the rows it names load the few granules that would pass their ends element by element, and so are the ends of
+// every output row stored.
 constexpr int kSiluRaggedMaxThreads = 256;
 struct RaggedGranule {
     int at;                // first unit of the output granule, in the row (negative before its start)
@@ -185,10 +185,22 @@ inline bool silu_takes_ragged(int64_t T, int64_t D, bool binary32, int vec) {
             !(vec == 4 && !binary32 && T > kSiluRaggedMaxTotal / D);
 }
 
+// The rows of a launch of `rows` whose granules must not pass their ends are row 0 and those from the returned one on:
+// the last row, or all where the memory between two rows may not exist.  Between two rows less than a page (4096
+// bytes) apart there is no page without a part of one of them; gate and up that fill one another's gaps (the
+// packed form [gate | up], padded or not) leave only the rest.  Pitches in units.
+inline uint32_t silu_ragged_end_rows(uint32_t rows, const uint16_t *gate, const uint16_t *up, int64_t D, int64_t gate_pitch,
+                                     int64_t up_pitch) {
+    const bool packed = gate_pitch == up_pitch && (up == gate + D || gate == up + D);
+    const int64_t taken = packed ? 2 * D : D;
+    const int64_t gap = (gate_pitch > up_pitch ? gate_pitch : up_pitch) - taken;
+    return gap < 2048 ? rows - 1 : 0;
+}
+
 template <int DT, int ALIGN>
 __global__ void __launch_bounds__(kSiluRaggedMaxThreads, 8)
 silu_and_mul_ragged_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gate,
-                           const uint16_t *__restrict__ up, FastDiv pieces, uint32_t last_row, int D,
+                           const uint16_t *__restrict__ up, FastDiv pieces, uint32_t end_rows, int D,
                            int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch) {
     constexpr int UV = 8, UNITS = Storage<DT>::UNITS;
     const uint32_t row = pieces.div(blockIdx.x);
@@ -204,7 +216,7 @@ silu_and_mul_ragged_kernel(uint16_t *__restrict__ out, const uint16_t *__restric
         }
     }
     const RaggedGranule g = ragged_granule(o, a, b, first / UV + static_cast<int>(threadIdx.x), D,
-                                           row == 0 || row == last_row);
+                                           row == 0 || row >= end_rows);
     grid_dependency_wait();
     grid_launch_dependents();
     if (g.at >= D) return;

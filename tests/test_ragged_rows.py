@@ -44,22 +44,33 @@ template <int UNITS> static void norm_row(long row, long weight, int units, int 
     for (int u = 0; u < units; ++u) expect(owner[u] == 1, "covered once", row, weight, units, u);
 }
 
-// All granules of a [rows, D] call with pitched operands; every tensor is [0, span) units from its base.
+// All granules of a [rows, D] call with pitched operands; the only memory is the pages (2048 units) with a part of a row.
 template <int UNITS> static void silu_rows(long o0, long a0, long b0, int rows, int D, long po, long pa, long pb) {
-    const long sa = (rows - 1) * pa + D, sb = (rows - 1) * pb + D;
+    const uint16_t *gate = at_unit(a0), *up = at_unit(b0);
+    const uint32_t end_rows = silu_ragged_end_rows(rows, gate, up, D, pa, pb);
+    std::set<long> pages;
+    for (int r = 0; r < rows; ++r)
+        for (long row : {a0 + r * pa, b0 + r * pb})
+            for (long page = row / 2048; page <= (row + D - 1) / 2048; ++page) pages.insert(page);
+    auto exists = [&](long at, long n) { return pages.count(at / 2048) && pages.count((at + n - 1) / 2048); };
+    const long first = a0 < b0 ? a0 : b0, last = (rows - 1) * (a0 < b0 ? pb : pa) + (a0 < b0 ? b0 : a0) + D;
+    const bool packed = b0 == a0 + D && pa == pb;  // one tensor, otherwise two
     for (int r = 0; r < rows; ++r) {
         std::vector<int> owner(D, 0);
         const uint16_t *o = at_unit(o0 + r * po), *a = at_unit(a0 + r * pa), *b = at_unit(b0 + r * pb);
         for (int n = 0; n < (D + 14) / 8; ++n) {
-            const RaggedGranule g = ragged_granule(o, a, b, n, D, r == 0 || r == rows - 1);
+            const RaggedGranule g = ragged_granule(o, a, b, n, D, r == 0 || static_cast<uint32_t>(r) >= end_rows);
             if (g.at >= D) continue;
             expect((o0 + r * po + g.at) % 8 == 0, "granule", r, D, g.at, 0);
             expect(g.shift_a % UNITS == 0 && g.shift_b % UNITS == 0 && g.at % UNITS == 0, "units", r, D, g.at, 0);
             if (g.whole) {
-                const long la = r * pa + g.at - g.shift_a, lb = r * pb + g.at - g.shift_b;
-                expect((a0 + la) % 8 == 0 && (b0 + lb) % 8 == 0, "aligned loads", r, D, g.at, 0);
-                expect(la >= 0 && la + (g.shift_a ? 16 : 8) <= sa, "gate granules", r, D, g.at, la);
-                expect(lb >= 0 && lb + (g.shift_b ? 16 : 8) <= sb, "up granules", r, D, g.at, lb);
+                const long la = a0 + r * pa + g.at - g.shift_a, lb = b0 + r * pb + g.at - g.shift_b;
+                const int na = g.shift_a ? 16 : 8, nb = g.shift_b ? 16 : 8;
+                expect(la % 8 == 0 && lb % 8 == 0, "aligned loads", r, D, g.at, 0);
+                expect(exists(la, na) && exists(lb, nb), "pages", r, D, g.at, la);
+                if (packed) expect(la >= first && lb >= first && la + na <= last && lb + nb <= last, "tensor", r, D, g.at, la);
+                else expect(la >= a0 && la + na <= a0 + (rows - 1) * pa + D && lb >= b0 && lb + nb <= b0 + (rows - 1) * pb + D,
+                            "tensors", r, D, g.at, la);
             }
             for (int k = 0; k < 8; ++k) if (g.at + k >= 0 && g.at + k < D) ++owner[g.at + k];
         }
@@ -93,6 +104,9 @@ int main() {
                 for (long a = 0; a < 8; ++a) {
                     silu_rows<1>(o, a, a + D, rows, D, D, 2 * D, 2 * D);        // the packed form
                     silu_rows<1>(o, a, (5 * a + 3) % 8, rows, D, D + 3, D, D + 1);
+                    silu_rows<1>(o, a, a + D, rows, D, D, 2 * D + 1000, 2 * D + 1000);
+                    for (long pitch : {2048L, 4096L, 8192L, 8193L})  // rows that begin or end a page, pages without a row
+                        for (long at : {0L, 2048L - D}) silu_rows<1>(o, at + a, at + (5 * a + 3) % 8, rows, D, D, pitch, pitch);
                     if (D % 2 == 0 && o % 2 == 0 && a % 2 == 0) silu_rows<2>(o, a, a + D, rows, D, D, 2 * D, 2 * D);
                 }
     printf("%ld failures\n", failures);
