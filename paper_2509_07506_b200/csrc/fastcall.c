@@ -18,6 +18,7 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include "astra.h"
@@ -174,21 +175,16 @@ static PyObject *fc_launch(PyObject *self, PyObject *const *args, Py_ssize_t nar
     return PyLong_FromLong((long)st);
 }
 
-/* footprint(prepared) -> ((address, bytes, is_written), ...): the memory the call reads and writes */
-static PyObject *fc_footprint(PyObject *self, PyObject *arg) {
-    if (!Py_IS_TYPE(arg, &PreparedType)) {
-        PyErr_SetString(PyExc_TypeError, "footprint(prepared)");
-        return NULL;
-    }
-    const Prepared *p = (const Prepared *)arg;
+/* The memory a call reads and writes: at most 6 + MAX_PARTS ranges, the first *written of them outputs. */
+static int footprint_of(const Prepared *p, const void **at, int64_t *bytes, int *written) {
     const int64_t elem = p->dtype == ASTRA_FP32 ? 4 : 2;
     const int64_t all = p->ext[0] * p->ext[1] * elem, row = p->ext[1] * elem;
-    const void *at[6 + MAX_PARTS] = {p->ptr[0], p->ptr[1], p->ptr[2], p->ptr[3], p->ptr[4], p->ptr[5]};
-    int64_t bytes[6 + MAX_PARTS] = {0};
-    int n, written = 2;  /* the first `written` pointers are outputs */
+    int n;
+    for (int i = 0; i < 6; ++i) at[i] = p->ptr[i];
+    *written = 2;
     switch (p->kind) {
         case KIND_SILU:
-            n = 2, written = 1, bytes[0] = all, bytes[1] = 2 * all;
+            n = 2, *written = 1, bytes[0] = all, bytes[1] = 2 * all;
             break;
         case KIND_MERGE:
             n = 6, bytes[0] = bytes[2] = bytes[4] = all * p->ext[2], bytes[1] = bytes[3] = bytes[5] = p->ext[0] * p->ext[1] * 4;
@@ -198,13 +194,168 @@ static PyObject *fc_footprint(PyObject *self, PyObject *arg) {
             for (int i = 0; i < p->n_parts; ++i) at[n] = p->parts[i], bytes[n++] = all;
             break;
     }
+    for (int i = 0; i < n; ++i)
+        if (at[i] == NULL) bytes[i] = 0;
+    return n;
+}
+
+/* footprint(prepared) -> ((address, bytes, is_written), ...): the memory the call reads and writes */
+static PyObject *fc_footprint(PyObject *self, PyObject *arg) {
+    if (!Py_IS_TYPE(arg, &PreparedType)) {
+        PyErr_SetString(PyExc_TypeError, "footprint(prepared)");
+        return NULL;
+    }
+    const void *at[6 + MAX_PARTS];
+    int64_t bytes[6 + MAX_PARTS];
+    int written;
+    const int n = footprint_of((const Prepared *)arg, at, bytes, &written);
     PyObject *out = PyTuple_New(n);
     for (int i = 0; out != NULL && i < n; ++i) {
-        PyObject *item = Py_BuildValue("(KLi)", (unsigned long long)(uintptr_t)at[i], (long long)(at[i] ? bytes[i] : 0),
-                                       i < written);
+        PyObject *item = Py_BuildValue("(KLi)", (unsigned long long)(uintptr_t)at[i], (long long)bytes[i], i < written);
         if (item == NULL) Py_CLEAR(out);
         else PyTuple_SET_ITEM(out, i, item);
     }
+    return out;
+}
+
+/* ---- which calls of a sequence depend on one another ------------------------------------------------------ */
+
+typedef struct {
+    uint64_t begin, end;
+    int call, written;
+} Range;
+
+static int by_address(const void *a, const void *b) {
+    const Range *p = a, *q = b;
+    if (p->begin != q->begin) return p->begin < q->begin ? -1 : 1;
+    return (p->end > q->end) - (p->end < q->end);
+}
+
+static int root_of(int *parent, int i) {
+    while (parent[i] != i) i = parent[i] = parent[parent[i]];
+    return i;
+}
+
+/* Groups (0, 1, ... in order of first appearance, into group[n_calls]) such that two calls of different groups share
+ * no byte that either of them writes.  One sweep in address order: a range that reaches into the present run of
+ * overlapping written ranges joins the run's call; a read in front of a run waits until the run begins. */
+static int group_calls(Range *r, Py_ssize_t n, int *group, Py_ssize_t n_calls) {
+    int *parent = PyMem_Malloc((size_t)(2 * n_calls + 1) * sizeof(int));
+    Range *reads = PyMem_Malloc((size_t)(n + 1) * sizeof(Range));  /* reads that may reach a later run */
+    if (parent == NULL || reads == NULL) {
+        PyMem_Free(parent);
+        PyMem_Free(reads);
+        return -1;
+    }
+    int *number = parent + n_calls;
+    for (int i = 0; i < n_calls; ++i) parent[i] = i, number[i] = -1;
+    uint64_t run_end = 0;
+    int owner = -1;
+    Py_ssize_t n_reads = 0;
+    for (Py_ssize_t i = 0; i < n; ++i) {
+        const int in_run = owner >= 0 && r[i].begin < run_end;
+        if (in_run) parent[root_of(parent, r[i].call)] = root_of(parent, owner);
+        if (!r[i].written) {
+            reads[n_reads++] = r[i];
+            continue;
+        }
+        if (!in_run) owner = r[i].call, run_end = r[i].end;
+        else if (r[i].end > run_end) run_end = r[i].end;
+        /* the reads that reach into this range are of its group from here on: one stands for all */
+        uint64_t reach = 0;
+        for (Py_ssize_t k = 0; k < n_reads; ++k) {
+            if (reads[k].end <= r[i].begin) continue;  /* ends before this and every later written range */
+            parent[root_of(parent, reads[k].call)] = root_of(parent, r[i].call);
+            if (reads[k].end > reach) reach = reads[k].end;
+        }
+        n_reads = reach > 0;
+        reads[0] = (Range){r[i].begin, reach, r[i].call, 0};
+    }
+    int next = 0;
+    for (int i = 0; i < n_calls; ++i) {
+        const int g = root_of(parent, i);
+        if (number[g] < 0) number[g] = next++;
+        group[i] = number[g];
+    }
+    PyMem_Free(parent);
+    PyMem_Free(reads);
+    return 0;
+}
+
+static PyObject *as_list(const int *v, Py_ssize_t n) {
+    PyObject *out = PyList_New(n);
+    for (Py_ssize_t i = 0; out != NULL && i < n; ++i) {
+        PyObject *item = PyLong_FromLong(v[i]);
+        if (item == NULL) Py_CLEAR(out);
+        else PyList_SET_ITEM(out, i, item);
+    }
+    return out;
+}
+
+/* The ranges of a sequence of calls; a call is a Prepared, or the ((address, bytes, is_written), ...) of one.
+ * Returns the number of calls, or -1 with an exception set; *r is the caller's to free. */
+static Py_ssize_t gather(PyObject *arg, Range **r, Py_ssize_t *n) {
+    PyObject *calls = PySequence_Fast(arg, "a sequence of calls");
+    if (calls == NULL) return -1;
+    const Py_ssize_t n_calls = PySequence_Fast_GET_SIZE(calls);
+    Py_ssize_t room = 0, done = -1;
+    *r = NULL, *n = 0;
+    for (Py_ssize_t c = 0; c < n_calls; ++c) {
+        PyObject *call = PySequence_Fast_GET_ITEM(calls, c), *given = NULL;
+        const void *at[6 + MAX_PARTS];
+        int64_t bytes[6 + MAX_PARTS];
+        int written = 0;
+        Py_ssize_t count;
+        if (Py_IS_TYPE(call, &PreparedType)) {
+            count = footprint_of((const Prepared *)call, at, bytes, &written);
+        } else {
+            if ((given = PySequence_Fast(call, "a prepared call or its footprint")) == NULL) goto out;
+            count = PySequence_Fast_GET_SIZE(given);
+        }
+        if (*n + count > room) {
+            room = 2 * (*n + count) + 4 * (n_calls - c);
+            Range *more = PyMem_Realloc(*r, (size_t)room * sizeof(Range));
+            if (more == NULL) {
+                Py_XDECREF(given);
+                PyErr_NoMemory();
+                goto out;
+            }
+            *r = more;
+        }
+        for (Py_ssize_t i = 0; i < count; ++i) {
+            unsigned long long begin;
+            long long size;
+            int is_written;
+            if (given == NULL) {
+                begin = (unsigned long long)(uintptr_t)at[i], size = bytes[i], is_written = i < written;
+            } else if (!PyArg_ParseTuple(PySequence_Fast_GET_ITEM(given, i), "KLp", &begin, &size, &is_written)) {
+                Py_DECREF(given);
+                goto out;
+            }
+            if (size > 0) (*r)[(*n)++] = (Range){begin, begin + (uint64_t)size, (int)c, is_written};
+        }
+        Py_XDECREF(given);
+    }
+    if (*n > 0) qsort(*r, (size_t)*n, sizeof(Range), by_address);
+    done = n_calls;
+out:
+    Py_DECREF(calls);
+    return done;
+}
+
+/* independent_groups(calls) -> group number of each call */
+static PyObject *fc_independent_groups(PyObject *self, PyObject *arg) {
+    Range *r = NULL;
+    Py_ssize_t n;
+    const Py_ssize_t n_calls = gather(arg, &r, &n);
+    PyObject *out = NULL;
+    if (n_calls >= 0) {
+        int *group = PyMem_Malloc((size_t)(n_calls + 1) * sizeof(int));
+        if (group == NULL || group_calls(r, n, group, n_calls) < 0) PyErr_NoMemory();
+        else out = as_list(group, n_calls);
+        PyMem_Free(group);
+    }
+    PyMem_Free(r);
     return out;
 }
 
@@ -217,6 +368,7 @@ static PyMethodDef methods[] = {
     {"prepare", fc_prepare, METH_VARARGS, "prepare(kind, pointers, extents, eps, dtype, parts) -> Prepared"},
     {"launch", (PyCFunction)(void (*)(void))fc_launch, METH_FASTCALL, "launch(prepared, stream_handle) -> status"},
     {"footprint", fc_footprint, METH_O, "footprint(prepared) -> ((address, bytes, is_written), ...)"},
+    {"independent_groups", fc_independent_groups, METH_O, "independent_groups(calls) -> group number of each call"},
     {"build_id", fc_build_id, METH_NOARGS, "hash of the sources this module was compiled from"},
     {NULL, NULL, 0, NULL},
 };

@@ -9,11 +9,11 @@ torch's graph object is used for capture and replay: device plumbing, no arithme
 """
 from __future__ import annotations
 
-import bisect
 from typing import List, Optional, Sequence
 
 import torch
 
+from . import binding
 from .binding import PreparedCall
 
 # Calls that share no memory one of them writes are captured into parallel branches, two at most.  Each call
@@ -25,49 +25,22 @@ from .binding import PreparedCall
 MAX_BRANCHES = 2
 
 
-def independent_groups(footprints: Sequence[Sequence[tuple]]) -> List[int]:
+def independent_groups(calls: Sequence) -> List[int]:
     """A group number per call (0, 1, ... in order of first appearance) such that two calls of different
-    groups touch no common byte that either of them writes.  ``footprints[i]`` lists the
-    ``(address, bytes, is_written)`` ranges of call i."""
-    parent = list(range(len(footprints)))
-
-    def root(i: int) -> int:
-        while parent[i] != i:
-            parent[i] = parent[parent[i]]
-            i = parent[i]
-        return i
-
-    # maximal runs of overlapping written ranges: everything in one run belongs together
-    starts: List[int] = []
-    ends: List[int] = []
-    owner: List[int] = []
-    for begin, size, call in sorted((a, n, i) for i, fp in enumerate(footprints) for a, n, w in fp if w and n):
-        if ends and begin < ends[-1]:
-            ends[-1] = max(ends[-1], begin + size)
-            parent[root(call)] = root(owner[-1])
-        else:
-            starts.append(begin)
-            ends.append(begin + size)
-            owner.append(call)
-    for call, fp in enumerate(footprints):
-        for begin, size, written in fp:
-            if written or not size:
-                continue
-            k = bisect.bisect_right(ends, begin)          # the first run that ends beyond the range's start
-            while k < len(starts) and starts[k] < begin + size:
-                parent[root(call)] = root(owner[k])
-                k += 1
-    number: dict = {}
-    return [number.setdefault(root(i), len(number)) for i in range(len(footprints))]
+    groups touch no common byte that either of them writes.  ``calls[i]`` is the extension's struct of call i or
+    the ``(address, bytes, is_written)`` ranges of it."""
+    binding.load_library()
+    return binding._fast.independent_groups(calls)
 
 
 def _branches(calls: Sequence[PreparedCall]) -> List[int]:
     """The branch each call is captured into; all zeros (one sequence) where a call is not one of ours."""
     if any(type(c) is not PreparedCall for c in calls):
         return [0] * len(calls)
-    footprints = [c.footprint() for c in calls]
-    groups = independent_groups(footprints)
-    sizes = [groups.count(g) for g in range(max(groups) + 1)]
+    groups = independent_groups([c._ready for c in calls])
+    sizes = [0] * (max(groups) + 1)
+    for g in groups:
+        sizes[g] += 1
     load, branch_of = [0] * min(MAX_BRANCHES, len(sizes)), [0] * len(sizes)
     for g in sorted(range(len(sizes)), key=lambda g: -sizes[g]):
         branch_of[g] = min(range(len(load)), key=load.__getitem__)

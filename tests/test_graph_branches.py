@@ -1,12 +1,15 @@
 """Which captured calls may run at the same time: the grouping against a brute-force conflict test (CPU),
 and replays of mixed dependent and independent calls against the same calls issued in order (GPU)."""
 import random
+import time
 
 import pytest
 import torch
 
 import paper_2509_07506_b200 as astra
 from paper_2509_07506_b200 import binding, graphs
+
+A = 1 << 20
 
 
 def conflict(p, q):
@@ -77,3 +80,24 @@ def test_replays_equal_the_calls_in_order(T):
         torch.cuda.synchronize()
         for p, q in zip(mem_a, mem_b):
             assert torch.equal(p.view(torch.int16), q.view(torch.int16))
+
+
+def fake_calls(ranges):
+    """Prepared norms whose x, residual and weight lie at the given addresses (nothing is launched)."""
+    binding.load_library()
+    ready = [binding._fast.prepare(binding._fast.KIND_RMSNORM, r, (4, 64), 1e-6, 0, ()) for r in ranges]
+    return [binding.PreparedCall("norm", None, None, torch.device("cuda", 0), (), r) for r in ready]
+
+
+def test_grouping_is_not_quadratic():
+    """Calls that share nothing with one another: ten times as many take about ten times as long (counting the calls
+    of each group one group at a time took a hundred times)."""
+    def took(n):
+        calls = fake_calls([(A * (3 * i + 1), A * (3 * i + 2), A * (3 * i + 3)) for i in range(n)])
+        best = 1e9
+        for _ in range(3):
+            start = time.perf_counter()
+            graphs._branches(calls)
+            best = min(best, time.perf_counter() - start)
+        return best
+    assert took(20000) < 40 * took(2000)
