@@ -359,6 +359,39 @@ static PyObject *fc_independent_groups(PyObject *self, PyObject *arg) {
     return out;
 }
 
+/* one_address_each(calls, query) -> whether every range lies in memory that has one address in this process.
+ * `query` is the address of the driver's cuPointerGetAttributes.  Memory of the plain allocators (those whose
+ * memory can be handed to another process as a whole) cannot be mapped a second time here; physical memory that
+ * was mapped by hand, imported memory and host memory can. */
+typedef int (*attributes_fn)(unsigned, int *, void **, unsigned long long);
+
+static PyObject *fc_one_address_each(PyObject *self, PyObject *args) {
+    PyObject *calls, *address;
+    if (!PyArg_ParseTuple(args, "OO", &calls, &address)) return NULL;
+    void *p;
+    if (as_address(address, &p) < 0) return NULL;
+    const attributes_fn query = (attributes_fn)p;
+    Range *r = NULL;
+    Py_ssize_t n;
+    if (gather(calls, &r, &n) < 0) {
+        PyMem_Free(r);
+        return NULL;
+    }
+    /* CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE, _RANGE_START_ADDR, _RANGE_SIZE */
+    int wanted[3] = {10, 11, 12}, sole = query != NULL;
+    uint64_t known = 0;  /* ranges that end at or before it and begin after the allocation's start are known */
+    for (Py_ssize_t i = 0; sole && i < n; ++i) {
+        if (r[i].end <= known) continue;
+        uint64_t plain = 0, start = 0, size = 0;
+        void *out[3] = {&plain, &start, &size};
+        sole = query(3, wanted, out, r[i].begin) == 0 && (plain & 0xff) != 0 && start <= r[i].begin &&
+               r[i].end <= start + size;
+        known = start + size;
+    }
+    PyMem_Free(r);
+    return PyBool_FromLong(sole);
+}
+
 static PyObject *fc_build_id(PyObject *self, PyObject *noargs) {
     return PyUnicode_FromString(astra_fastcall_build_marker + sizeof("astra-build-id:") - 1);
 }
@@ -369,6 +402,8 @@ static PyMethodDef methods[] = {
     {"launch", (PyCFunction)(void (*)(void))fc_launch, METH_FASTCALL, "launch(prepared, stream_handle) -> status"},
     {"footprint", fc_footprint, METH_O, "footprint(prepared) -> ((address, bytes, is_written), ...)"},
     {"independent_groups", fc_independent_groups, METH_O, "independent_groups(calls) -> group number of each call"},
+    {"one_address_each", fc_one_address_each, METH_VARARGS,
+     "one_address_each(calls, query) -> whether all their memory has one address in this process"},
     {"build_id", fc_build_id, METH_NOARGS, "hash of the sources this module was compiled from"},
     {NULL, NULL, 0, NULL},
 };

@@ -9,6 +9,7 @@ torch's graph object is used for capture and replay: device plumbing, no arithme
 """
 from __future__ import annotations
 
+import ctypes
 from typing import List, Optional, Sequence
 
 import torch
@@ -33,11 +34,29 @@ def independent_groups(calls: Sequence) -> List[int]:
     return binding._fast.independent_groups(calls)
 
 
+_driver: Optional[ctypes.CDLL] = None
+
+
+def _pointer_attributes() -> Optional[int]:
+    """Address of the driver's cuPointerGetAttributes, or None."""
+    global _driver
+    if _driver is None:
+        try:
+            _driver = ctypes.CDLL("libcuda.so.1")
+        except OSError:
+            return None
+    return ctypes.cast(_driver.cuPointerGetAttributes, ctypes.c_void_p).value
+
+
 def _branches(calls: Sequence[PreparedCall]) -> List[int]:
-    """The branch each call is captured into; all zeros (one sequence) where a call is not one of ours."""
+    """The branch each call is captured into; all zeros (one sequence) where a call is not one of ours or where
+    addresses do not tell whether two calls share memory."""
     if any(type(c) is not PreparedCall for c in calls):
         return [0] * len(calls)
-    groups = independent_groups([c._ready for c in calls])
+    ready = [c._ready for c in calls]
+    groups = independent_groups(ready)
+    if max(groups) == 0 or not binding._fast.one_address_each(ready, _pointer_attributes()):
+        return [0] * len(calls)
     sizes = [0] * (max(groups) + 1)
     for g in groups:
         sizes[g] += 1

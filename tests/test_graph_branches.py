@@ -1,5 +1,6 @@
 """Which captured calls may run at the same time: the grouping against a brute-force conflict test (CPU),
 and replays of mixed dependent and independent calls against the same calls issued in order (GPU)."""
+import ctypes
 import random
 import time
 
@@ -101,3 +102,84 @@ def test_grouping_is_not_quadratic():
             best = min(best, time.perf_counter() - start)
         return best
     assert took(20000) < 40 * took(2000)
+
+
+def test_memory_with_two_addresses_keeps_the_calls_in_order(monkeypatch):
+    """Only where the driver says of every range that it is the plain allocators' does an address stand for memory;
+    anything else (mapped by hand, imported, host memory) may be mapped twice, and the calls stay in one branch."""
+    allocations = {}  # start -> (size, plain)
+    asked = []
+
+    @ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_uint, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_void_p), ctypes.c_uint64)
+    def query(n, which, out, address):
+        assert [which[i] for i in range(n)] == [10, 11, 12]
+        asked.append(address)
+        for start, (size, plain) in allocations.items():
+            if start <= address < start + size:
+                for i, v in enumerate((plain, start, size)):
+                    ctypes.cast(out[i], ctypes.POINTER(ctypes.c_uint64))[0] = v
+                return 0
+        return 1
+    monkeypatch.setattr(graphs, "_pointer_attributes", lambda: ctypes.cast(query, ctypes.c_void_p).value)
+    calls = fake_calls([(A + 4096 * i, 2 * A + 4096 * i, 3 * A) for i in range(20)])
+    allocations.update({A: (A, 1), 2 * A: (A, 1), 3 * A: (A, 1)})
+    assert max(graphs._branches(calls)) == 1 and len(asked) == 3
+    allocations[2 * A] = (A, 0)                       # mapped by hand
+    assert graphs._branches(calls) == [0] * 20
+    allocations[2 * A] = (4096 * 19 + 100, 1)         # the last range ends beyond the allocation
+    assert graphs._branches(calls) == [0] * 20
+    del allocations[3 * A]                            # the driver does not know the address
+    assert graphs._branches(calls) == [0] * 20
+    monkeypatch.setattr(graphs, "_pointer_attributes", lambda: None)
+    assert graphs._branches(calls) == [0] * 20
+
+
+class At:
+    """A [rows, width] float32 array at an address."""
+
+    def __init__(self, address, shape):
+        self.__cuda_array_interface__ = {"shape": shape, "typestr": "<f4", "data": (address, False), "version": 3, "strides": None}
+
+
+@pytest.mark.gpu
+def test_memory_mapped_twice_is_not_captured_into_two_branches():
+    driver = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(result):
+        assert int(result[0]) == 0, result
+        return result[1] if len(result) == 2 else result[1:]
+    torch.zeros(1, device="cuda")
+    where = driver.CUmemLocation()
+    where.type, where.id = driver.CUmemLocationType.CU_MEM_LOCATION_TYPE_DEVICE, 0
+    prop = driver.CUmemAllocationProp()
+    prop.type, prop.location = driver.CUmemAllocationType.CU_MEM_ALLOCATION_TYPE_PINNED, where
+    size = ok(driver.cuMemGetAllocationGranularity(prop, driver.CUmemAllocationGranularity_flags.CU_MEM_ALLOC_GRANULARITY_MINIMUM))
+    access = driver.CUmemAccessDesc()
+    access.location, access.flags = where, driver.CUmemAccess_flags.CU_MEM_ACCESS_FLAGS_PROT_READWRITE
+    handle = ok(driver.cuMemCreate(size, prop, 0))
+    mapped = []
+    for _ in range(2):
+        at = ok(driver.cuMemAddressReserve(size, 0, 0, 0))
+        ok(driver.cuMemMap(at, size, 0, handle, 0))
+        ok(driver.cuMemSetAccess(at, size, [access], 1))
+        mapped.append(int(at))
+    T, H = 64, 256
+    one, two = (torch.as_tensor(At(p, (T, H)), device="cuda") for p in mapped)
+    r, w, out = torch.zeros(T, H, device="cuda"), torch.ones(H, device="cuda"), torch.empty(T, H // 2, device="cuda")
+    calls = [astra.prepare_fused_add_rmsnorm(one, r, w, 1e-5), astra.prepare_silu_and_mul(out, two)]
+    assert graphs.independent_groups([c.footprint() for c in calls]) == [0, 1]   # by their addresses
+    assert graphs._branches(calls) == [0, 0]
+    graph = astra.CapturedCalls(calls)
+    one.copy_(torch.randn(T, H, device="cuda"))
+    r.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    want = torch.empty_like(out)
+    astra.astra_silu_and_mul(want, one)
+    assert torch.equal(out, want)
+    del graph
+    torch.cuda.synchronize()
+    for p in mapped:
+        ok(driver.cuMemUnmap(p, size))
+        ok(driver.cuMemAddressFree(p, size))
+    ok(driver.cuMemRelease(handle))
