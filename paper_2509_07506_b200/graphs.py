@@ -48,10 +48,10 @@ def _pointer_attributes() -> Optional[int]:
     return ctypes.cast(_driver.cuPointerGetAttributes, ctypes.c_void_p).value
 
 
-def _branches(calls: Sequence[PreparedCall]) -> List[int]:
+def _branches(calls: Sequence[PreparedCall], most: int = MAX_BRANCHES) -> List[int]:
     """The branch each call is captured into; all zeros (one sequence) where a call is not one of ours or where
     addresses do not tell whether two calls share memory."""
-    if any(type(c) is not PreparedCall for c in calls):
+    if most < 2 or any(type(c) is not PreparedCall for c in calls):
         return [0] * len(calls)
     ready = [c._ready for c in calls]
     groups = independent_groups(ready)
@@ -60,7 +60,7 @@ def _branches(calls: Sequence[PreparedCall]) -> List[int]:
     sizes = [0] * (max(groups) + 1)
     for g in groups:
         sizes[g] += 1
-    load, branch_of = [0] * min(MAX_BRANCHES, len(sizes)), [0] * len(sizes)
+    load, branch_of = [0] * min(most, len(sizes)), [0] * len(sizes)
     for g in sorted(range(len(sizes)), key=lambda g: -sizes[g]):
         branch_of[g] = min(range(len(load)), key=load.__getitem__)
         load[branch_of[g]] += sizes[g]
@@ -72,13 +72,15 @@ class CapturedCalls:
     (so that lazy initialisation happens outside the capture), then captures them;
     ``replay()`` re-issues the whole sequence on the current stream with one launch, with the results of
     the calls issued in order: calls that depend on one another through a tensor stay in that order, and
-    calls that share no written memory may run at the same time.  The tensors the
+    calls that share no written memory may run at the same time, in at most ``branches`` sequences (1: all in the
+    order given).  The tensors the
     calls were prepared on are the graph's inputs and outputs.  The eager warm-up run has already
     executed every call once when the constructor returns (in-place calls such as fused_add_rmsnorm
     have then modified their operands), so fill the inputs after constructing, and refill them in
     place between replays."""
 
-    def __init__(self, calls: Sequence[PreparedCall], device: Optional[torch.device] = None):
+    def __init__(self, calls: Sequence[PreparedCall], device: Optional[torch.device] = None,
+                 branches: int = MAX_BRANCHES):
         self.calls = list(calls)
         if not self.calls:
             raise ValueError("at least one prepared call is needed")
@@ -89,13 +91,13 @@ class CapturedCalls:
             for call in self.calls:       # warm-up outside the capture
                 call(side)
             side.synchronize()
-            branches = _branches(self.calls)
-            streams = [side] + [torch.cuda.Stream(self.device) for _ in range(max(branches))]
+            branch_of = _branches(self.calls, branches)
+            streams = [side] + [torch.cuda.Stream(self.device) for _ in range(max(branch_of))]
             self.graph = torch.cuda.CUDAGraph()
             with torch.cuda.graph(self.graph, stream=side):
                 for s in streams[1:]:
                     s.wait_stream(side)
-                for call, branch in zip(self.calls, branches):
+                for call, branch in zip(self.calls, branch_of):
                     call(streams[branch])
                 for s in streams[1:]:
                     side.wait_stream(s)

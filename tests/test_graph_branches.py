@@ -183,3 +183,12 @@ def test_memory_mapped_twice_is_not_captured_into_two_branches():
         ok(driver.cuMemUnmap(p, size))
         ok(driver.cuMemAddressFree(p, size))
     ok(driver.cuMemRelease(handle))
+
+
+def test_one_branch_on_request(monkeypatch):
+    calls = fake_calls([(A * (3 * i + 1), A * (3 * i + 2), A * (3 * i + 3)) for i in range(6)])
+    monkeypatch.setattr(graphs, "_pointer_attributes", lambda: None)
+    monkeypatch.setattr(binding._fast, "one_address_each", lambda calls, query: True)
+    assert sorted(graphs._branches(calls)) == [0, 0, 0, 1, 1, 1]
+    assert graphs._branches(calls, 1) == [0] * 6
+    assert sorted(graphs._branches(calls, 3)) == [0, 0, 1, 1, 2, 2]
