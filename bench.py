@@ -13,7 +13,8 @@ fraction is taken against the measured copy bandwidth of the GPU.
 N > 1 (under torchrun, or started plainly, in which case the N ranks are spawned here): every rank runs its own T = 8192 batch (weak scaling; the operations are
 independent per row, so there is no collective on the data path); time is the max over ranks.
 `--impl reference` times the fp64 CPU oracle on the host cores instead (rank 0 only).
-Exactly one JSON line is printed on stdout by rank 0.
+Exactly one JSON line is printed on stdout by rank 0, a few KB long; the tables of the other timings (shapes,
+strided and fp32 forms, all-reduce form, ablation) go to stderr, one JSON line each.
 """
 from __future__ import annotations
 
@@ -841,6 +842,19 @@ def run_reference(args, rank: int, world: int) -> dict | None:
     }
 
 
+# Parts of the result that are tables of their own
+TABLES = ("shape_sweep", "table4", "strided_variants", "decode_chain", "fp32_variants", "rmsnorm_cost_model",
+          "allreduce_rmsnorm", "ablation")
+
+
+def print_result(res: dict) -> None:
+    """The tables on stderr, then the headline alone on stdout: a reader that keeps the end of the output gets all of it."""
+    for name in TABLES:
+        if name in res:
+            print(json.dumps({name: res.pop(name)}), file=sys.stderr, flush=True)
+    print(json.dumps(res), flush=True)
+
+
 def main() -> int:
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -894,7 +908,7 @@ def main() -> int:
             import torch.distributed as dist
             dist.destroy_process_group()
     if res is not None:
-        print(json.dumps(res), flush=True)
+        print_result(res)
     return 0
 
 
