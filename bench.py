@@ -448,7 +448,7 @@ def _time_graph(call, sets, launches=100):
 
 
 def shape_sweep(astra, dev, peak) -> list:
-    """us/call for configs[0..2] and every point of the fused_add_rmsnorm sweep (configs[3]).
+    """us/call for the three single-operation shapes and every point of the fused_add_rmsnorm sweep.
     `us_hot` repeats one buffer set (it stays in L2 when it fits); `us_cold` cycles through enough
     sets to defeat L2 (n_cold_sets); `*_graph` are the same launches replayed from a CUDA graph (device
     time only).  Shapes that stream more than two L2 sizes carry the roofline fraction of their L2-cold
@@ -482,19 +482,19 @@ def shape_sweep(astra, dev, peak) -> list:
         add("fused_add_rmsnorm", dtype, [T, H], wl.rmsnorm_bytes(T, H), make,
             lambda b: astra.astra_fused_add_rmsnorm(b[0], b[1], b[2], 1e-5))
 
-    rms(wl.BF16, 16, 4096)                                            # configs[0]
-    T, D = 128, wl.CHAIN_D                                            # configs[1]
+    rms(wl.BF16, 16, 4096)
+    T, D = 128, wl.CHAIN_D
     add("silu_and_mul", wl.BF16, [T, 2 * D], wl.silu_bytes(T, D),
         lambda: (torch.empty((T, D), device=dev, dtype=torch.bfloat16),
                  (2 * torch.randn((T, 2 * D), device=dev)).to(torch.bfloat16)),
         lambda b: astra.astra_silu_and_mul(b[0], b[1]))
-    T, Hh, Dh = 512, 32, 128                                          # configs[2]
+    T, Hh, Dh = 512, 32, 128
     add("merge_attn_states_lse", wl.BF16, [T, Hh, Dh], wl.merge_bytes(T, Hh, Dh),
         lambda: (torch.empty((T, Hh, Dh), device=dev, dtype=torch.bfloat16), torch.empty((T, Hh), device=dev),
                  torch.randn((T, Hh, Dh), device=dev).to(torch.bfloat16), torch.rand((T, Hh), device=dev) * 20 - 5,
                  torch.randn((T, Hh, Dh), device=dev).to(torch.bfloat16), torch.rand((T, Hh), device=dev) * 20 - 5),
         lambda b: astra.astra_merge_attn_states_lse(b[0], b[1], b[2], b[3], b[4], b[5]))
-    for dtype in wl.SWEEP_DTYPES:                                     # configs[3]
+    for dtype in wl.SWEEP_DTYPES:
         for T in wl.SWEEP_T:
             for H in wl.SWEEP_H:
                 rms(dtype, T, H)
@@ -801,7 +801,7 @@ def oracle_agreement(astra, cfg, dev, rows: int) -> dict:
 
 
 def chain_workload_name(T: int) -> str:
-    return (f"configs[4]: Llama-3-8B prefill-shaped chain, T={T} per GPU, bf16: "
+    return (f"Llama-3-8B prefill-shaped chain, T={T} per GPU, bf16: "
             f"fused_add_rmsnorm [{T},4096] -> silu_and_mul [{T},2*14336] -> "
             f"merge_attn_states_lse [{T},32,128]")
 
@@ -864,7 +864,7 @@ def main() -> int:
     ap.add_argument("--e2e-steps", type=int, default=10, help="steps of the host-to-host timed region")
     ap.add_argument("--e2e-chunk-rows", type=int, default=2048, help="rows per upload/compute/download chunk")
     ap.add_argument("--cpu-rows", type=int, default=8192, help="rows of the chain the CPU baseline covers")
-    ap.add_argument("--no-sweep", action="store_true", help="skip the per-shape timings of configs[0..3]")
+    ap.add_argument("--no-sweep", action="store_true", help="skip the per-shape timings")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU (oracle) baseline leg")
     ap.add_argument("--no-ablation", action="store_true", help="skip the design-pair ablation timings")
     ap.add_argument("--no-clocks", action="store_true", help="do not sample clocks with nvidia-smi")

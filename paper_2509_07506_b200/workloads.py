@@ -211,7 +211,7 @@ TABLE4 = (
 
 
 def table4_inputs(kernel: str, shape, dtype: int = BF16, seed: int = 5):
-    """Seeded inputs for one Table 4 shape (same value distributions as configs[0..2])."""
+    """Seeded inputs for one Table 4 shape (same value distributions as the single-operation shapes)."""
     if kernel == "merge_attn_states_lse":
         return merge_inputs(shape[0], shape[1], shape[2], dtype, seed=seed)
     if kernel == "fused_add_rmsnorm":
