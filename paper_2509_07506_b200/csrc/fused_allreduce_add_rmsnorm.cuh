@@ -95,8 +95,9 @@ constexpr int kAllreduceDenseBlocks = 5;
 
 //
 // LATE_R requests the residual after the partials instead of with the first of them, which frees its
-// registers while they are summed: two vectors per thread with two partial loads in flight then take 72
-// registers instead of 96 and two blocks of up to 448 threads fit an SM instead of one.  For rows of 10241
+// registers while they are summed, and asks for two resident blocks of up to 448 threads: two vectors per thread
+// with two partial loads in flight are held to 72 registers instead of 96 (the 16-bit forms spill 52 to 60 bytes for it,
+// the ragged fp16 form 4; binary32 needs 59 and 63), and two blocks fit an SM instead of one.  For rows of 10241
 // to 14336 units, where every other shape leaves one block per SM that idles at its barrier, L2-cold, with
 // 2 / 4 / 8 partials: 79.7 -> 67.9, 112.7 -> 92.2, 171.0 -> 145.3 us at [4096, 11008] (65.4 / 91.5 / 143.8 us at
 // 6.9 TB/s) and 93.2 -> 86.1, 133.2 -> 119.4, 203.5 -> 188.2 us at [4096, 14336]; no gain where two blocks fit
@@ -356,7 +357,8 @@ fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOpera
 // (78.8 -> 68.0 us with 4 partials, 117.3 -> 105.6 us with 8); H = 10240 with two in flight takes two
 // vectors in 320-thread blocks (two per SM) rather than one 640-thread block (61.6 against 76.7 us);
 // H = 11008 ... 14336 take the late residual (79.7 -> 67.9 us at [4096, 11008] with 2 partials, more at the
-// kernel; but 2.7 against 3.2 us at [16, 11008], where every SM has one row at most); H = 16384 takes one vector in one 1024-thread block (143.1 against 155.8 us with 4 partials).
+// kernel; but 2.7 against 3.2 us at [16, 11008], where every SM has one row at most); H = 16384 takes one vector in
+// one 1024-thread block (143.1 against 155.8 us with 4 partials).
 // Binary32 rows need fewer registers (5120 elements take one vector in two 640-thread blocks: 25.1 -> 23.1 us at
 // [1024, 5120] with 4 partials).
 // Binary32 rows of more than 16384 units take four vectors per thread, one load in flight, in one block

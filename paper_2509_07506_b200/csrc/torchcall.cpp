@@ -10,10 +10,10 @@
 // mode, another current device), it returns None without having launched anything, and the binding takes
 // its own route, which launches or raises the precise error.  Otherwise it returns the entry point's status;
 // every argument check of the C ABI still runs there.
-// Host time per call, enqueued back to back, Python-level checks -> here (a prepared call: 2.2 us, nearly all
-// of it the launch): rmsnorm 5.1 -> 2.3 us, silu 5.0 -> 2.5, merge 7.4 -> 2.6, all-reduce with 8 partials 11.7 ->
-// 2.9; the strided forms, which went through ctypes, 12.8 -> 2.2, 10.3 -> 2.5, 15.1 -> 2.7, and 26.6 -> 3.4 us
-// with 8 partials and 8 destinations.
+// Host time per call, enqueued back to back, Python-level checks -> here (a prepared call: 2.2 to 2.6 us, nearly all
+// of it the launch): rmsnorm 5.1 -> 2.5 us, silu 5.0 -> 2.8, merge 7.4 -> 2.9, all-reduce with 8 partials 11.7 -> 3.3;
+// the strided forms, which went through ctypes, 12.8 -> 2.5, 10.3 -> 2.6, 15.1 -> 2.8, and 26.6 -> 3.7 us with 8
+// partials and 8 destinations.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 

@@ -19,10 +19,11 @@ from .binding import PreparedCall
 
 # Calls that share no memory one of them writes are captured into parallel branches, two at most.  Each call
 # of a dependent sequence is a chain of latencies (launch, first bytes, reduction, completion) that leaves
-# most of the GPU idle while it waits; a second sequence fills that time.  Measured per decode layer (norm,
-# merge, norm, activation, the norms over one residual) with 1 / 2 / 4 branches: 4.41 / 2.59 / 2.64 us at 1 token
-# of width 4096, 4.98 / 3.07 / 2.97 at 16, 9.69 / 7.16 / 7.08 at 256, 14.8 / 10.3 / 10.8 at 512, and still
-# 27.7 / 23.3 / 23.4 at 1024 and 216 / 209 / 210 at 8192 tokens, where the gain is the filled ends of the grids.
+# most of the GPU idle while it waits; a second sequence fills that time.  Measured on norm, merge, norm, activation
+# repeated 32 times where only the norms share a tensor (one residual), per repetition with 1 / 2 / 4 branches:
+# 4.41 / 2.59 / 2.64 us at 1 token of width 4096, 4.98 / 3.07 / 2.97 at 16, 9.69 / 7.16 / 7.08 at 256, 14.8 / 10.3 / 10.8 at
+# 512, and still 27.7 / 23.3 / 23.4 at 1024 and 216 / 209 / 210 at 8192 tokens, where the gain is the filled ends of the
+# grids.  Calls that are linked through their tensors, as a decoder layer's are, stay one sequence and gain nothing.
 MAX_BRANCHES = 2
 
 
