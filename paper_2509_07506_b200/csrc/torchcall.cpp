@@ -11,8 +11,8 @@
 // its own route, which launches or raises the precise error.  Otherwise it returns the entry point's status;
 // every argument check of the C ABI still runs there.
 // Host time per call, enqueued back to back, Python-level checks -> here (a prepared call: 2.2 to 2.6 us, nearly all
-// of it the launch): rmsnorm 5.1 -> 2.5 us, silu 5.0 -> 2.8, merge 7.4 -> 2.9, all-reduce with 8 partials 11.7 -> 3.3;
-// the strided forms, which went through ctypes, 12.8 -> 2.5, 10.3 -> 2.6, 15.1 -> 2.8, and 26.6 -> 3.7 us with 8
+// of it the launch): rmsnorm 5.5 -> 2.4 us, silu 5.3 -> 2.7, merge 7.9 -> 2.8, all-reduce with 8 partials 11.9 -> 3.3;
+// the strided forms, which went through ctypes, 12.4 -> 2.5, 10.4 -> 2.6, 15.7 -> 2.9, and 26.6 -> 3.9 us with 8
 // partials and 8 destinations.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
