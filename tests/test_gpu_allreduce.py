@@ -17,10 +17,10 @@ pytestmark = pytest.mark.gpu
 BF16, FP16, FP32 = wl.BF16, wl.FP16, wl.FP32
 
 
-def run_allreduce(inp: wl.AllreduceRmsnormInputs, offset=0, prepared=False):
+def run_allreduce(inp: wl.AllreduceRmsnormInputs, offset=0, prepared=False, weight_offset=None):
     T, H = inp.residual.shape
     gparts = [Guarded(p, offset) for p in inp.parts]
-    gr, gw = Guarded(inp.residual, offset), Guarded(inp.weight, offset)
+    gr, gw = Guarded(inp.residual, offset), Guarded(inp.weight, offset if weight_offset is None else weight_offset)
     gy = Guarded(torch.zeros_like(inp.residual), offset)
     if prepared:
         astra.prepare_fused_allreduce_add_rmsnorm(gy.t, gr.t, [g.t for g in gparts], gw.t, inp.eps)()

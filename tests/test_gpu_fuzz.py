@@ -68,3 +68,13 @@ def test_fuzz_fused_allreduce_add_rmsnorm(T, H, dtype, offset, seed):
     while T * H * n_parts > 3 * MAX_ELEMS:
         T = max(1, T // 2)
     run_allreduce(wl.allreduce_rmsnorm_inputs(T, H, n_parts, dtype, seed=seed), offset=offset)
+
+
+@pytest.mark.parametrize("T,H,dtype,offset,seed", cases(6, 60, widths=[1025, 1030, 1038, 2051, 2058, 3075, 4099, 4101, 5126, 6407, 8191, 10243,
+                                                                       11007, 14335, 16383]))
+def test_fuzz_fused_allreduce_add_rmsnorm_with_a_weight_of_its_own(T, H, dtype, offset, seed):
+    rng = random.Random(seed)
+    n_parts, T = rng.choice([2, 3, 4, 8]), rng.choice([T, rng.randrange(1, MAX_ELEMS // H)])
+    while T * H * n_parts > 3 * MAX_ELEMS:
+        T = max(1, T // 2)
+    run_allreduce(wl.allreduce_rmsnorm_inputs(T, H, n_parts, dtype, seed=seed), offset=offset, weight_offset=rng.randrange(16))

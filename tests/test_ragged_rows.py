@@ -12,7 +12,7 @@ PROGRAM = r"""
 #include <set>
 #include <utility>
 #include <vector>
-#include "fused_add_rmsnorm.cuh"
+#include "fused_allreduce_add_rmsnorm.cuh"
 #include "silu_and_mul.cuh"
 using namespace astra;
 
@@ -79,7 +79,7 @@ template <int UNITS> static void silu_rows(long o0, long a0, long b0, int rows, 
 }
 
 int main() {
-    // every shape that the launch rule gives a width at any row count
+    // every shape that the launch rules of the two norms give a width at any row count
     std::set<int> widths = {1055, 1056, 1057, 2051, 4099, 5120, 5135, 5136, 8191, 16383, 16399, 16400, 32767, 32782};
     for (int units = 1024; units <= 1041; ++units) widths.insert(units);
     for (int units : widths)
@@ -88,6 +88,11 @@ int main() {
             for (int T = 1; T <= 6000; ++T)
                 for (int vec : {1, 2, 4, 8}) {
                     const RaggedShape sh = rmsnorm_ragged_shape(T, units, binary32, vec);
+                    if (sh.vpt > 0) shapes.insert({sh.vpt, sh.threads});
+                }
+            for (int T : {1, 100, 129, 148, 150, 296, 300, 500, 4096})
+                for (int n_parts : {1, 2, 4, 8}) {
+                    const AllreduceShape sh = allreduce_wide_shape(T, units, n_parts, binary32, true);
                     if (sh.vpt > 0) shapes.insert({sh.vpt, sh.threads});
                 }
             expect(binary32 || units >= 16400 || !shapes.empty(), "shape", units, 0, 0, 0);
