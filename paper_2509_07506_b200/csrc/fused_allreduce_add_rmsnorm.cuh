@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(LATE_R ? kAllreduceLateThreads : DENSE ? kAllr
                                                                   : allreduce_reg_max_threads(VEC * VPT * Storage<DT>::UNITS, GROUP),
                                   LATE_R ? 2 : DENSE ? kAllreduceDenseBlocks : 1)
 fused_allreduce_add_rmsnorm_reg_kernel(const __grid_constant__ AllreduceOperands op,
-                                       const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
+                                       const uint16_t *__restrict__ weight, int H, float eps, float inv_H, LaunchPad<40>) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
     __shared__ __align__(16) float slots[kMaxWarps];
     const int nvec = H / VEC;
@@ -224,7 +224,7 @@ template <int DT, int VPT, int GROUP, bool LATE_R = false>
 __global__ void __launch_bounds__(LATE_R ? kAllreduceLateThreads : VPT == 4 ? 512 : allreduce_reg_max_threads(16 * VPT, GROUP),
                                   LATE_R ? 2 : GROUP == 4 ? 0 : 1)
 fused_allreduce_add_rmsnorm_ragged_kernel(const __grid_constant__ AllreduceOperands op,
-                                          const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
+                                          const uint16_t *__restrict__ weight, int H, float eps, float inv_H, LaunchPad<40>) {
     constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
     constexpr bool EDGE_LAST = GROUP == 4 || GROUP == 1 || LATE_R, EARLY_W = GROUP > 4;
     __shared__ __align__(16) float slots[kMaxWarps];
@@ -494,7 +494,7 @@ __device__ __forceinline__ void rank_order_sum(const AllreduceOperands &op, int6
 template <int DT, int VEC, int GROUP>
 __global__ void __launch_bounds__(1024)
 fused_allreduce_add_rmsnorm_twopass_kernel(const __grid_constant__ AllreduceOperands op,
-                                           const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
+                                           const uint16_t *__restrict__ weight, int H, float eps, float inv_H, LaunchPad<40>) {
     constexpr int UV = VEC * Storage<DT>::UNITS;
     __shared__ __align__(16) float slots[kMaxWarps];
     const int nvec = H / VEC;

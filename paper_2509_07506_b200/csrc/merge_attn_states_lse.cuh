@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(THREADS)
 merge_attn_states_lse_kernel(uint16_t *v_out, float *lse_out,
                              const uint16_t *v_a, const float *lse_a,
                              const uint16_t *v_b, const float *lse_b,
-                             uint32_t total_vecs, FastDiv nvec) {
+                             uint32_t total_vecs, FastDiv nvec, LaunchPad<24>) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
     const uint32_t base = blockIdx.x * (THREADS * UNROLL) + threadIdx.x;
     // Ahead of the dependency wait the block asks for its (contiguous) share of both value tensors to
@@ -135,7 +135,7 @@ merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
                                      const uint16_t *v_a, const float *lse_a,
                                      const uint16_t *v_b, const float *lse_b,
                                      uint32_t total_vecs, uint32_t row0, FastDiv nvec, FastDiv heads,
-                                     MergeStrides st) {
+                                     MergeStrides st, LaunchPad<40>) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
     constexpr bool FLAT = READS == MergeReads::Dense;
     const uint32_t first = blockIdx.x * (THREADS * UNROLL);

@@ -54,7 +54,7 @@ template <int DT, int VEC, int UNROLL, int THREADS, Ld LDH = Ld::StreamReadOnly,
 __global__ void __launch_bounds__(THREADS)
 silu_and_mul_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gate,
                     const uint16_t *__restrict__ up, uint32_t total_vecs, FastDiv nvec,
-                    int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch) {
+                    int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch, LaunchPad<24>) {
     constexpr int UV = VEC * Storage<DT>::UNITS;  // 16-bit units per vector
     const uint32_t base = blockIdx.x * (THREADS * UNROLL) + threadIdx.x;
     // Ahead of the dependency wait, the block asks for the gate and up bytes of its vectors to be
@@ -201,7 +201,7 @@ template <int DT, int ALIGN>
 __global__ void __launch_bounds__(kSiluRaggedMaxThreads, 8)
 silu_and_mul_ragged_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gate,
                            const uint16_t *__restrict__ up, FastDiv pieces, uint32_t end_rows, int D,
-                           int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch) {
+                           int64_t out_pitch, int64_t gate_pitch, int64_t up_pitch, LaunchPad<16>) {
     constexpr int UV = 8, UNITS = Storage<DT>::UNITS;
     const uint32_t row = pieces.div(blockIdx.x);
     const int first = static_cast<int>((blockIdx.x - row * pieces.d) * blockDim.x) * UV;

@@ -276,6 +276,11 @@ __device__ __forceinline__ void store_edge(uint16_t *row, int at, int width, con
     }
 }
 
+// Bytes that bring a kernel's parameters to a size that is quick to launch (see launch.cuh); never read.
+template <int BYTES> struct LaunchPad {
+    uint32_t w[BYTES / 4];
+};
+
 // ---------------------------------------------------------------------------------------------
 // Programmatic dependent launch.  A kernel launched with the programmatic-stream-serialization
 // attribute may be scheduled while the previous kernel in the stream is still draining.  It must
