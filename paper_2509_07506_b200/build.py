@@ -25,7 +25,7 @@ ABLATION_LIB_PATH = os.path.join(PKG_DIR, "libastra_ablation.so")
 FASTCALL_PATH = os.path.join(PKG_DIR, "_astra_fastcall.so")
 TORCHCALL_PATH = os.path.join(PKG_DIR, "_astra_torchcall.so")
 
-SOURCES = ["astra.cu", "astra_allreduce.cu"]
+SOURCES = ["astra.cu", "astra_allreduce.cu", "astra_runs.cu"]
 ABLATION_SOURCES = ["ablation.cu"]
 FASTCALL_SOURCE = "fastcall.c"
 TORCHCALL_SOURCE = "torchcall.cpp"

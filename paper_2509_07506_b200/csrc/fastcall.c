@@ -22,6 +22,7 @@
 #include <string.h>
 
 #include "astra.h"
+#include "call_runs.h"
 #include "fastcall.h"
 
 #ifndef ASTRA_BUILD_ID
@@ -40,7 +41,10 @@ typedef astra_status_t (*merge_fn)(void *, float *, const void *, const float *,
 typedef astra_status_t (*allreduce_fn)(void *, void *, const void *const *, int32_t, const void *, int64_t,
                                        int64_t, float, astra_dtype_t, void *);
 
+typedef astra_status_t (*run_fn)(int, int32_t, const astra_run_call *, const int64_t *, float, astra_dtype_t, void *);
+
 static void *entry_points[KIND_PREPARED];
+static run_fn issue_run;
 
 typedef struct {
     PyObject_HEAD
@@ -172,6 +176,56 @@ static PyObject *fc_launch(PyObject *self, PyObject *const *args, Py_ssize_t nar
                                     p->eps, dt, stream);
             break;
     }
+    return PyLong_FromLong((long)st);
+}
+
+/* bind_run(address): the library's astra_issue_run */
+static PyObject *fc_bind_run(PyObject *self, PyObject *address) {
+    void *p;
+    if (as_address(address, &p) < 0) return NULL;
+    issue_run = (run_fn)p;
+    Py_RETURN_NONE;
+}
+
+/* Do two calls differ in nothing but their addresses?  (The all-reduce form is never part of a run.) */
+static int alike(const Prepared *p, const Prepared *q) {
+    return p->kind == q->kind && p->kind != KIND_ALLREDUCE_RMSNORM && p->dtype == q->dtype &&
+           memcmp(&p->eps, &q->eps, sizeof p->eps) == 0 && memcmp(p->ext, q->ext, sizeof p->ext) == 0;
+}
+
+/* alike(prepared, prepared) -> whether the two can be in one run */
+static PyObject *fc_alike(PyObject *self, PyObject *const *args, Py_ssize_t nargs) {
+    if (nargs != 2 || !Py_IS_TYPE(args[0], &PreparedType) || !Py_IS_TYPE(args[1], &PreparedType)) {
+        PyErr_SetString(PyExc_TypeError, "alike(prepared, prepared)");
+        return NULL;
+    }
+    return PyBool_FromLong(alike((const Prepared *)args[0], (const Prepared *)args[1]));
+}
+
+/* launch_run(calls, stream_handle) -> status: calls that are alike, in order, in as few launches as their operands allow */
+static PyObject *fc_launch_run(PyObject *self, PyObject *args) {
+    PyObject *calls, *handle;
+    void *stream;
+    if (!PyArg_ParseTuple(args, "O!O", &PyList_Type, &calls, &handle) || as_address(handle, &stream) < 0) return NULL;
+    const Py_ssize_t n = PyList_GET_SIZE(calls);
+    if (n < 1 || n > INT32_MAX || issue_run == NULL) {
+        PyErr_SetString(PyExc_ValueError, issue_run == NULL ? "no entry point bound for runs" : "no calls");
+        return NULL;
+    }
+    astra_run_call *each = PyMem_Malloc((size_t)n * sizeof *each);
+    if (each == NULL) return PyErr_NoMemory();
+    const Prepared *first = (const Prepared *)PyList_GET_ITEM(calls, 0);
+    for (Py_ssize_t i = 0; i < n; ++i) {
+        PyObject *c = PyList_GET_ITEM(calls, i);
+        if (!Py_IS_TYPE(c, &PreparedType) || !alike(first, (const Prepared *)c)) {
+            PyMem_Free(each);
+            PyErr_SetString(PyExc_ValueError, "the calls of a run are alike");
+            return NULL;
+        }
+        memcpy(each[i].ptr, ((const Prepared *)c)->ptr, sizeof each[i].ptr);
+    }
+    const astra_status_t st = issue_run(first->kind, (int32_t)n, each, first->ext, first->eps, (astra_dtype_t)first->dtype, stream);
+    PyMem_Free(each);
     return PyLong_FromLong((long)st);
 }
 
@@ -400,6 +454,9 @@ static PyMethodDef methods[] = {
     {"bind", fc_bind, METH_VARARGS, "bind(kind, address): set the entry point of one kind of call"},
     {"prepare", fc_prepare, METH_VARARGS, "prepare(kind, pointers, extents, eps, dtype, parts) -> Prepared"},
     {"launch", (PyCFunction)(void (*)(void))fc_launch, METH_FASTCALL, "launch(prepared, stream_handle) -> status"},
+    {"bind_run", fc_bind_run, METH_O, "bind_run(address): set the entry point of runs of calls"},
+    {"alike", (PyCFunction)(void (*)(void))fc_alike, METH_FASTCALL, "alike(prepared, prepared) -> whether the two can be in one run"},
+    {"launch_run", fc_launch_run, METH_VARARGS, "launch_run(calls, stream_handle) -> status of the calls, issued in order"},
     {"footprint", fc_footprint, METH_O, "footprint(prepared) -> ((address, bytes, is_written), ...)"},
     {"independent_groups", fc_independent_groups, METH_O, "independent_groups(calls) -> group number of each call"},
     {"one_address_each", fc_one_address_each, METH_VARARGS,

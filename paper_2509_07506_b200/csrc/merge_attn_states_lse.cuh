@@ -48,6 +48,22 @@ __device__ __forceinline__ MergeWeights merge_weights(float sa, float sb) {
     return r;
 }
 
+// The blend of two vectors of UV units.  A zero-weight side is dropped, not multiplied: its payload may be
+// Inf/NaN garbage.
+template <int DT, int UV>
+__device__ __forceinline__ Pack<UV> merge_packs(const MergeWeights &mw, const Pack<UV> &a, const Pack<UV> &b) {
+    constexpr int VEC = UV / Storage<DT>::UNITS;
+    float fa[VEC], fb[VEC], fo[VEC];
+    widen<DT, VEC>(a, fa);
+    widen<DT, VEC>(b, fb);
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+        const float ta = mw.use_a ? fa[i] * mw.wa : 0.f;
+        fo[i] = mw.use_b ? fmaf(fb[i], mw.wb, ta) : ta;
+    }
+    return narrow<DT, VEC>(fo);
+}
+
 // Strides of one [T, Hh, D] value tensor (in 16-bit units) or one [T, Hh] score tensor (in floats);
 // D is contiguous.
 struct MergeStrides {
@@ -94,16 +110,7 @@ merge_attn_states_lse_kernel(uint16_t *v_out, float *lse_out,
         const uint32_t v = base + j * THREADS;
         if (v < total_vecs) {
             const MergeWeights mw = merge_weights(sa[j], sb[j]);
-            float fa[VEC], fb[VEC], fo[VEC];
-            widen<DT, VEC>(a[j], fa);
-            widen<DT, VEC>(b[j], fb);
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                // a zero-weight side is dropped, not multiplied: its payload may be Inf/NaN garbage
-                const float ta = mw.use_a ? fa[i] * mw.wa : 0.f;
-                fo[i] = mw.use_b ? fmaf(fb[i], mw.wb, ta) : ta;
-            }
-            store<UV, STH>(v_out + static_cast<int64_t>(v) * UV, narrow<DT, VEC>(fo));
+            store<UV, STH>(v_out + static_cast<int64_t>(v) * UV, merge_packs<DT, UV>(mw, a[j], b[j]));
             if (lse_out != nullptr && v == row[j] * nvec.d) lse_out[row[j]] = mw.lse;
         }
     }
@@ -184,16 +191,8 @@ merge_attn_states_lse_strided_kernel(uint16_t *v_out, float *lse_out,
     };
     auto finish = [&](int j, const Place &p) {
         const MergeWeights mw = merge_weights(sa[j], sb[j]);
-        float fa[VEC], fb[VEC], fo[VEC];
-        widen<DT, VEC>(a[j], fa);
-        widen<DT, VEC>(b[j], fb);
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-            const float ta = mw.use_a ? fa[i] * mw.wa : 0.f;
-            fo[i] = mw.use_b ? fmaf(fb[i], mw.wb, ta) : ta;
-        }
         store<UV, St::Stream>(v_out + (FLAT ? (flat0 + p.v) * UV : p.t * st.vo_t + p.h * st.vo_h + p.col),
-                              narrow<DT, VEC>(fo));
+                              merge_packs<DT, UV>(mw, a[j], b[j]));
         if (lse_out != nullptr && p.col == 0) lse_out[p.t * st.so_t + p.h * st.so_h] = mw.lse;
     };
     if constexpr (READS == MergeReads::Few) {
