@@ -36,9 +36,11 @@ const char kBuildId[] = "astra-build-id:" ASTRA_BUILD_ID;
 // below it the inputs are requested ahead of the dependency wait.
 constexpr uint32_t kSiluPrefetchMaxBlocks = 1u << 14;
 // Range of grid sizes (in 256-thread blocks of one 32-byte vector per thread) in which the 32-byte
-// form is used: from 640 blocks (measured: slower at 448, faster at 896) to 8192 (faster at 7168,
-// slower at 14336).
-constexpr int64_t kSiluWideMinBlocks = 640;
+// form is used.  Up to 960 blocks the grid is less than one wave of eight blocks per SM, which the next kernel's early
+// blocks then fill unevenly; 16-byte form / 32-byte form, us, with operands in L2: 2.53 / 3.44 at 672 blocks
+// ([192, 14336]), 3.05 / 3.39 at 896, 3.46 / 3.53 at 1050, 4.28 / 4.25 at 1400; L2-cold: 3.16 / 3.54, 4.19 / 3.93, 4.68 / 4.22,
+// 5.87 / 5.24.  The upper end: faster at 7168 blocks, slower at 14336.
+constexpr int64_t kSiluWideMinBlocks = 960;
 constexpr int64_t kSiluWideMaxBlocks = 8192;
 
 template <int DT, int UVEC, int UNROLL, int THREADS>
@@ -103,11 +105,10 @@ cudaError_t dispatch_silu(uint16_t *out, const uint16_t *gate, const uint16_t *u
                   .pointer(out).pointer(gate).pointer(up).vec;
     // One 16-byte vector per thread and 256-thread blocks: the smallest work quantum that still
     // keeps the block scheduler ahead, which gives the shortest drain at the end of the grid.
-    // Between about one and ten waves of blocks, one 32-byte vector per thread (half as many blocks,
-    // each still prefetching its share ahead of the dependency wait) is faster where everything is
-    // 32-byte aligned: 4.21 -> 3.83 us at [256, 14336], 7.19 -> 6.73 us at [512, 14336], 13.2 -> 12.6 us
-    // at [1024, 14336], 25.2 -> 24.8 us at [2048, 14336] (L2-cold, bf16); it is slower below that
-    // (2.56 -> 3.14 us at [128, 14336]) and above it (98.3 -> 99.9 us at [8192, 14336]).
+    // Between one and ten waves of blocks, one 32-byte vector per thread (half as many blocks, each still prefetching its
+    // share ahead of the dependency wait) is faster where everything is 32-byte aligned: see kSiluWideMinBlocks, and
+    // 13.2 -> 12.6 us at [1024, 14336], 25.2 -> 24.8 us at [2048, 14336] (L2-cold, bf16); it is slower below that and above
+    // it (98.3 -> 99.9 us at [8192, 14336]).
     if (vec == 16) {
         const int64_t blocks_wide = (T * (D / 16) + 255) / 256;
         if (blocks_wide >= kSiluWideMinBlocks && blocks_wide <= kSiluWideMaxBlocks)

@@ -6,43 +6,109 @@
 // element (ex2 and rcp, the fast-math forms the paper's optimised kernel also turns to), in
 // binary32, with one rounding at the store.  Instruction count matters even though the kernel is
 // HBM-bound: under a sustained power cap the SM clock (and with it the on-chip fabric) drops as
-// issue activity rises, so the arithmetic is kept to the packed two-wide forms.
+// issue activity rises (1.5 to 1.7 GHz at 1 kW), so the arithmetic is kept to the packed two-wide forms and,
+// for all but very negative gates, to half the instructions of the overflow-free form.  Sustained, L2-cold, against
+// that form for all elements: 101.7 -> 100.2 us at bf16 [8192, 14336], 57.9 -> 55.7 at [4000, 14333], 36.0 -> 34.6 at fp16
+// [8192, 4099], 34.5 -> 33.0 at [8192, 4100], 15.2 -> 14.8 at [1000, 14337], 13.4 -> 13.1 at [1024, 14336].
 #pragma once
 
 #include "vec.cuh"
 
 namespace astra {
 
-// SiLU(a) * b in binary32, in the overflow-free form: with t = e^{-|a|} in [0, 1],
-// sigmoid(a) = 1/(1+t) for a >= 0 and t/(1+t) for a < 0, so the reciprocal's argument stays in
-// [1, 2].  t is formed as h*h with h = e^{-|a|/2} = 2^{-|a| * log2(e)/2}: h stays a normal number
-// down to |a| = 174, and the (non-flushing) product h*h reaches the subnormals, so a * e^{a} * b is
-// still produced where e^{a} alone is below 2^-126; beyond |a| = 174 the true result is below every
-// representable magnitude anyway.
-constexpr float kHalfLog2e = 0.7213475204444817f;
+// SiLU(a) * b in binary32.  From a = -40 up directly, a / (1 + e^{-a}) * b.  Below, in the overflow-free form: with
+// t = e^{-|a|} in [0, 1], sigmoid(a) = t/(1+t).  t is formed as h*h with h = e^{-|a|/2} = 2^{-|a| * log2(e)/2}: h stays
+// a normal number down to |a| = 174, and the (non-flushing) product h*h reaches the subnormals, so a * e^{a} * b
+// is still produced where e^{a} alone is below 2^-126; beyond |a| = 174 the true result is below every representable
+// magnitude anyway.  Against 64 bits, binary32: largest relative error 5.9e-7 for |a| < 10 and 2.0e-6 above -40 (6.6e-7
+// and 2.0e-6 with the overflow-free form).  Which form an element takes depends on nothing but itself, so results
+// do not depend on how a row is cut into vectors.
+constexpr float kLog2e = 1.4426950408889634f, kHalfLog2e = 0.7213475204444817f, kSiluDirect = -40.0f;
 
-__device__ __forceinline__ float silu_mul(float a, float b) {
+__device__ __forceinline__ float silu_mul_far(float a, float b) {
     float h, d;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(fabsf(a) * -kHalfLog2e));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(a * kHalfLog2e));
     const float t = h * h;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(1.0f + t));
-    return a * (d * (a >= 0.f ? 1.0f : t)) * b;
+    return a * (d * t) * b;
 }
 
-// Two elements at a time with the packed binary32 instructions of sm_100 (two multiplies or adds
-// per issue slot); the two special-function ops per element stay scalar.  Same arithmetic, element
-// by element, as silu_mul.
-__device__ __forceinline__ float2 silu_mul2(float2 a, float2 b) {
-    const float2 arg = __fmul2_rn(make_float2(fabsf(a.x), fabsf(a.y)), make_float2(-kHalfLog2e, -kHalfLog2e));
-    float2 h, d;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h.x) : "f"(arg.x));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h.y) : "f"(arg.y));
-    const float2 t = __fmul2_rn(h, h);
-    const float2 den = __fadd2_rn(t, make_float2(1.0f, 1.0f));
+__device__ __forceinline__ float silu_mul(float a, float b) {
+    if (a < kSiluDirect) return silu_mul_far(a, b);
+    float e, d;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a * -kLog2e));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(e + 1.0f));
+    return a * d * b;
+}
+
+// Two elements from -40 up, with the packed binary32 instructions of sm_100 (two multiplies or adds per issue slot); the
+// two special-function ops per element stay scalar.  Same arithmetic, element by element, as silu_mul.
+__device__ __forceinline__ float2 silu_mul2_direct(float2 a, float2 b) {
+    const float2 arg = __fmul2_rn(a, make_float2(-kLog2e, -kLog2e));
+    float2 e, d;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(arg.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(arg.y));
+    const float2 den = __fadd2_rn(e, make_float2(1.0f, 1.0f));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d.x) : "f"(den.x));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d.y) : "f"(den.y));
-    const float2 f = make_float2(a.x >= 0.f ? 1.0f : t.x, a.y >= 0.f ? 1.0f : t.y);
-    return __fmul2_rn(__fmul2_rn(a, __fmul2_rn(d, f)), b);
+    return __fmul2_rn(__fmul2_rn(a, d), b);
+}
+
+// Is any element below -40 (or, of the 16-bit types, a NaN with its sign set)?  The patterns of negative numbers grow
+// with their magnitude, so 16-bit elements are compared as unsigned integers, two per instruction.
+template <int DT, int UV> __device__ __forceinline__ bool any_far(const Pack<UV> &a) {
+    constexpr int WORDS = Pack<UV>::WORDS;
+    if constexpr (DT == ASTRA_FP32) {
+        float least = kSiluDirect;
+#pragma unroll
+        for (int i = 0; i < WORDS; ++i) least = fminf(least, __uint_as_float(a.w[i]));
+        return least < kSiluDirect;
+    } else {
+        constexpr uint32_t limit = DT == ASTRA_FP16 ? 0xd100d100u : 0xc220c220u;  // -40, twice
+        uint32_t most = limit;
+#pragma unroll
+        for (int i = 0; i < WORDS; i += 2)
+            most = i + 1 < WORDS ? __vimax3_u16x2(most, a.w[i], a.w[i + 1]) : __vmaxu2(most, a.w[i]);
+        return most != limit;
+    }
+}
+
+// SiLU(a) * b on whole packs.  A pack with a far element goes word by word, in a loop that moves the words along (it is
+// rarely taken, and unrolled its code cost small calls 0.05 us).
+template <int DT, int UV> __device__ __forceinline__ Pack<UV> silu_mul_pack(const Pack<UV> &a, const Pack<UV> &b) {
+    constexpr int VEC = UV / Storage<DT>::UNITS, WORDS = Pack<UV>::WORDS, PER_WORD = UV == 1 ? 1 : 2 / Storage<DT>::UNITS;
+    if (VEC == 1 || any_far<DT, UV>(a)) {
+        Pack<UV> x = a, y = b, v;
+#pragma unroll 1
+        for (int i = 0; i < WORDS; ++i) {
+            Pack<PER_WORD * Storage<DT>::UNITS> xw, yw;
+            xw.w[0] = x.w[0];
+            yw.w[0] = y.w[0];
+            float fa[PER_WORD], fb[PER_WORD], fo[PER_WORD];
+            widen<DT, PER_WORD>(xw, fa);
+            widen<DT, PER_WORD>(yw, fb);
+#pragma unroll
+            for (int k = 0; k < PER_WORD; ++k) fo[k] = silu_mul(fa[k], fb[k]);
+#pragma unroll
+            for (int k = 0; k + 1 < WORDS; ++k) {
+                x.w[k] = x.w[k + 1];
+                y.w[k] = y.w[k + 1];
+                v.w[k] = v.w[k + 1];
+            }
+            v.w[WORDS - 1] = narrow<DT, PER_WORD>(fo).w[0];
+        }
+        return v;
+    }
+    float fa[VEC], fb[VEC], fo[VEC];
+    widen<DT, VEC>(a, fa);
+    widen<DT, VEC>(b, fb);
+#pragma unroll
+    for (int i = 0; i + 1 < VEC; i += 2) {
+        const float2 o = silu_mul2_direct(make_float2(fa[i], fa[i + 1]), make_float2(fb[i], fb[i + 1]));
+        fo[i] = o.x;
+        fo[i + 1] = o.y;
+    }
+    return narrow<DT, VEC>(fo);
 }
 
 // Flat indexing: vector v of the output covers out[row, col*VEC .. col*VEC+VEC) with
@@ -91,40 +157,12 @@ silu_and_mul_kernel(uint16_t *__restrict__ out, const uint16_t *__restrict__ gat
     for (int j = 0; j < UNROLL; ++j) {
         const uint32_t v = base + j * THREADS;
         if (v < total_vecs) {
-            float fa[VEC], fb[VEC], fo[VEC];
-            widen<DT, VEC>(a[j], fa);
-            widen<DT, VEC>(b[j], fb);
-            if constexpr (VEC == 1) {
-                fo[0] = silu_mul(fa[0], fb[0]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < VEC; i += 2) {
-                    const float2 o = silu_mul2(make_float2(fa[i], fa[i + 1]), make_float2(fb[i], fb[i + 1]));
-                    fo[i] = o.x;
-                    fo[i + 1] = o.y;
-                }
-            }
             const uint32_t row = nvec.div(v);
             const uint32_t col = v - row * nvec.d;
             store<UV, STH>(out + (static_cast<int64_t>(row) * out_pitch + static_cast<int64_t>(col) * UV),
-                            narrow<DT, VEC>(fo));
+                            silu_mul_pack<DT, UV>(a[j], b[j]));
         }
     }
-}
-
-// SiLU(a) * b on whole packs.
-template <int DT, int UV> __device__ __forceinline__ Pack<UV> silu_mul_pack(const Pack<UV> &a, const Pack<UV> &b) {
-    constexpr int VEC = UV / Storage<DT>::UNITS;
-    float fa[VEC], fb[VEC], fo[VEC];
-    widen<DT, VEC>(a, fa);
-    widen<DT, VEC>(b, fb);
-#pragma unroll
-    for (int i = 0; i < VEC; i += 2) {
-        const float2 o = silu_mul2(make_float2(fa[i], fa[i + 1]), make_float2(fb[i], fb[i + 1]));
-        fo[i] = o.x;
-        fo[i + 1] = o.y;
-    }
-    return narrow<DT, VEC>(fo);
 }
 
 // Rows that start at any element: the widths and pitches whose common divisor leaves less than a 16-byte
@@ -136,8 +174,8 @@ template <int DT, int UV> __device__ __forceinline__ Pack<UV> silu_mul_pack(cons
 // an L1 hit) and the 8 units are taken out of them with ASTRA_FOR_SHIFT, uniformly for the block, which
 // covers one piece of one row.
 //
-// What bounds it: HBM, then issue slots (about 165 warp instructions per 32 granules against 113 of the
-// aligned kernel; 73 % of the slots at [8192, 4099]).  Measured L2-cold, fp16, against the narrow flat
+// What bounds it: HBM, then issue slots (two loads, up to eight shifts and the edges' tests more per granule than the
+// aligned kernel).  Measured L2-cold, fp16, against the narrow flat
 // kernels: 28.5 -> 14.1 us at [1000, 14337] (12.5 us at 6.9 TB/s), 64.0 -> 33.7 us at [8192, 4099], 39.9 -> 33.7 us at
 // [8192, 4098], 5.69 -> 4.5 us at [300, 11010]; fp32 16.0 -> 13.1 us at [1000, 7001].  Also tried: flat
 // indexing over all rows' granules (15.3 and 33.8 us: the shifts are then per thread and need selects),
