@@ -186,13 +186,20 @@ cudaError_t launch_merge(uint16_t *v_out, float *lse_out, const uint16_t *v_a, c
   return cudaSuccess;
 }
 
+constexpr int64_t kMergeSmallVecs = 1 << 18;  // 32-byte vectors up to which blocks have 128 threads
 template <int DT>
 cudaError_t dispatch_merge(uint16_t *v_out, float *lse_out, const uint16_t *v_a, const float *lse_a,
                     const uint16_t *v_b, const float *lse_b, int64_t rows, int64_t D,
                     cudaStream_t stream) {
-    // 32-byte accesses measured best here (one per thread, 256-thread blocks)
+    // 32-byte accesses measured best here, one per thread.  Up to about a wave in blocks of 128 threads, whose ends are
+    // shorter and which spread more evenly; then of 256, of which fewer have to be started.  256 / 128 threads, us, operands
+    // in L2: 1.32 / 1.03 at [16, 32, 128], 1.83 / 1.61 at [256, 32, 128], 2.49 / 2.38 at [512, 32, 128], 3.14 / 2.95 at [1024,
+    // 32, 128], 4.16 / 4.22 at [1280, 32, 128]; L2-cold 1.39 / 1.13, 2.24 / 2.22, 2.90 / 2.85, 4.64 / 4.61, 6.18 / 6.16.
     switch (VecPick(16).extent(D).pointer(v_out).pointer(v_a).pointer(v_b).vec) {
-        case 16: return launch_merge<DT, 16, 1, 256>(v_out, lse_out, v_a, lse_a, v_b, lse_b, rows, D, stream);
+        case 16:
+            if (rows <= kMergeSmallVecs / (D / 16))
+                return launch_merge<DT, 16, 1, 128>(v_out, lse_out, v_a, lse_a, v_b, lse_b, rows, D, stream);
+            return launch_merge<DT, 16, 1, 256>(v_out, lse_out, v_a, lse_a, v_b, lse_b, rows, D, stream);
         case 8: return launch_merge<DT, 8, 2, 256>(v_out, lse_out, v_a, lse_a, v_b, lse_b, rows, D, stream);
         case 4: return launch_merge<DT, 4, 4, 256>(v_out, lse_out, v_a, lse_a, v_b, lse_b, rows, D, stream);
         case 2: return launch_merge<DT, 2, 4, 256>(v_out, lse_out, v_a, lse_a, v_b, lse_b, rows, D, stream);
