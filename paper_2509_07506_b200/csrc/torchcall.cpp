@@ -10,10 +10,9 @@
 // mode, another current device), it returns None without having launched anything, and the binding takes
 // its own route, which launches or raises the precise error.  Otherwise it returns the entry point's status;
 // every argument check of the C ABI still runs there.
-// Host time per call, enqueued back to back, Python-level checks -> here (a prepared call: 2.2 to 2.6 us, nearly all
-// of it the launch): rmsnorm 5.5 -> 2.4 us, silu 5.3 -> 2.7, merge 7.9 -> 2.8, all-reduce with 8 partials 11.9 -> 3.3;
-// the strided forms, which went through ctypes, 12.4 -> 2.5, 10.4 -> 2.6, 15.7 -> 2.9, and 26.6 -> 3.9 us with 8
-// partials and 8 destinations.
+// Host time per call, enqueued back to back, Python-level checks -> here (nearly all of it the launch): rmsnorm 5.5 ->
+// 2.3 us, silu 5.3 -> 2.35, merge 7.9 -> 2.4, all-reduce with 8 partials 11.9 -> 2.8; the strided forms 12.4 -> 2.4, 10.4 ->
+// 2.3, 15.7 -> 2.6, and 26.6 -> 3.5 us with 8 partials and 8 destinations.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
