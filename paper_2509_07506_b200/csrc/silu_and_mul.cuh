@@ -9,7 +9,7 @@
 // issue activity rises (1.5 to 1.7 GHz at 1 kW), so the arithmetic is kept to the packed two-wide forms and,
 // for all but very negative gates, to half the instructions of the overflow-free form.  Sustained, L2-cold, against
 // that form for all elements: 101.7 -> 100.2 us at bf16 [8192, 14336], 57.9 -> 55.7 at [4000, 14333], 36.0 -> 34.6 at fp16
-// [8192, 4099], 34.5 -> 33.0 at [8192, 4100], 15.2 -> 14.8 at [1000, 14337], 13.4 -> 13.1 at [1024, 14336].
+// [8192, 4099] (21.8 instead of 25.9 million warp instructions at [4096, 14336]), 34.5 -> 33.0 at [8192, 4100], 15.2 -> 14.8 at [1000, 14337], 13.4 -> 13.1 at [1024, 14336].
 #pragma once
 
 #include "vec.cuh"

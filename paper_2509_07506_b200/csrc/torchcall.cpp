@@ -11,8 +11,8 @@
 // its own route, which launches or raises the precise error.  Otherwise it returns the entry point's status;
 // every argument check of the C ABI still runs there.
 // Host time per call, enqueued back to back, Python-level checks -> here (nearly all of it the launch): rmsnorm 5.5 ->
-// 2.3 us, silu 5.3 -> 2.35, merge 7.9 -> 2.4, all-reduce with 8 partials 11.9 -> 2.8; the strided forms 12.4 -> 2.4, 10.4 ->
-// 2.3, 15.7 -> 2.6, and 26.6 -> 3.5 us with 8 partials and 8 destinations.
+// 2.2 us, silu 5.3 -> 2.0, merge 7.9 -> 2.2, all-reduce with 8 partials 11.9 -> 2.5; the strided forms of norm and merge 12.4 ->
+// 2.2 and 15.7 -> 2.3, and 26.6 -> 3.1 us with 8 partials and 8 destinations.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 

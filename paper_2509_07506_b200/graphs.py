@@ -1,7 +1,7 @@
 """Replaying a fixed sequence of calls from a CUDA graph.
 
 For decode-sized batches every call of this library is bound by launch cost, not by the GPU: a
-call costs 2.0-2.8 us of host time for 1-2 us of device time.  A sequence of prepared
+call costs 2.0-2.5 us of host time for 1-2 us of device time.  A sequence of prepared
 calls on fixed tensors (a layer's add+norm, activation and merge, say) can be captured once into a
 CUDA graph and replayed with a single launch; the kernels keep their programmatic-dependent-launch
 edges inside the graph, so each one's prologue (and its L2 prefetch) overlaps the previous one's tail, and
@@ -21,10 +21,9 @@ from .binding import PreparedCall
 # Calls that share no memory one of them writes are captured into parallel branches, two at most.  Each call
 # of a dependent sequence is a chain of latencies (launch, first bytes, reduction, completion) that leaves
 # most of the GPU idle while it waits; a second sequence fills that time.  Measured on norm, merge, norm, activation
-# repeated 32 times where only the norms share a tensor (one residual), per repetition with 1 / 2 / 4 branches:
-# 4.41 / 2.59 / 2.64 us at 1 token of width 4096, 4.98 / 3.07 / 2.97 at 16, 9.69 / 7.16 / 7.08 at 256, 14.8 / 10.3 / 10.8 at
-# 512, and still 27.7 / 23.3 / 23.4 at 1024 and 216 / 209 / 210 at 8192 tokens, where the gain is the filled ends of the
-# grids.  Calls that are linked through their tensors, as a decoder layer's are, stay one sequence and gain nothing.
+# repeated 32 times where only the norms share a tensor (one residual), per repetition with 1 / 2 / 4 branches, the latter
+# two with like calls in one launch: 4.17 / 0.71 / 0.77 us at 1 token of width 4096, 4.68 / 0.77 / 0.77 at 16, 9.56 / 4.43 /
+# 4.63 at 256, 13.7 / 10.1 / 10.1 at 512, 26.6 / 19.2 / 19.6 at 1024 and 212 / 176 / 176 at 8192 tokens.  Calls that are linked through their tensors, as a decoder layer's are, stay one sequence and gain nothing.
 MAX_BRANCHES = 2
 
 
