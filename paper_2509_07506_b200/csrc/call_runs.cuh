@@ -31,7 +31,8 @@ struct RmsnormRun {
 // `uvec` units.  threads = 0: no form for this size.
 // Spreading a row pays while SMs would be idle: one SM moves a row's 24 KB per call (x, weight, y at H = 4096) at 52
 // GB/s.  64 calls in one launch, from a graph, us, with 1 / 2 / 4 / 8 blocks per row: 43 / 24.6 / 22.6 / 26.6 at
-// [16, 4096], 45 / 24.8 / 28.7 / 32.8 at [64, 4096], 59 / 47 / 28.7 / 34 at [16, 8192]; one by one 92, 107 and 110.
+// [16, 4096], 45 / 24.8 / 28.7 / 32.8 at [64, 4096], 59 / 47 / 28.7 / 34 at [16, 8192]; one
+// by one (beside as many merges and activations) 99, 131 and 120.
 struct NormRunShape {
     int blocks = 0, threads = 0, uvec = 0;
 };
