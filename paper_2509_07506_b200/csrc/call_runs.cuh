@@ -18,6 +18,13 @@ namespace astra {
 
 constexpr int kMaxRun = 64;  // calls of one launch: their addresses are kernel parameters
 
+// Polls of one wait of a cluster exchange before it is given up, and the limit that the waits of the exchanges use (a
+// test lowers the latter to see what is left of a run whose waits end too early).
+constexpr int kWaitPolls = 1 << 16;
+#ifndef ASTRA_RUN_WAIT_POLLS
+#define ASTRA_RUN_WAIT_POLLS kWaitPolls
+#endif
+
 // ---- fused_add_rmsnorm: calls on one residual ----------------------------------------------------------------
 struct RmsnormRun {
     uint16_t *x[kMaxRun];
@@ -85,9 +92,9 @@ __device__ __forceinline__ void init_barrier(uint32_t barrier) {
 __device__ __forceinline__ void expect_bytes(uint32_t barrier, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(barrier), "r"(bytes) : "memory");
 }
-// Waits for the barrier's phase; false if it does not end.
-__device__ __forceinline__ bool wait_counted(uint32_t barrier, uint32_t phase) {
-    for (int i = 0; i < (1 << 16); ++i) {
+// Waits for the barrier's phase; false if it has not ended after so many polls.
+__device__ __forceinline__ bool wait_counted(uint32_t barrier, uint32_t phase, int polls) {
+    for (int i = 0; i < polls; ++i) {
         uint32_t done;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
@@ -102,7 +109,12 @@ __device__ __forceinline__ bool wait_counted(uint32_t barrier, uint32_t phase) {
 // go through the block or cluster in one exchange: every warp stores its K sums where all can read them
 // (in a cluster, into every block's shared memory), and after one wait every warp adds up all warps' sums in the same
 // order.  The next exchange uses the other half of `slots`; nobody can be two exchanges ahead of another.
-// In a cluster the wait is bounded; the normalised rows are NaN should it ever run out.
+//
+// In a cluster the wait is bounded.  A warp whose wait runs out has its share of the present and of all later normalised
+// rows set to NaN, stores nothing more into other blocks and arms no barrier again (one whose phase has not ended
+// must not be); the other warps of the row, which then lack its sums, run out at the next exchange and do the same.
+// Nobody reads sums of two exchanges that way, and the residual, which needs no sums, is as it should be.  Before it
+// leaves, such a warp waits once more, up to the full limit, for the stores that it gave up on.
 // 1.45 -> 0.35 us per call at [16, 4096].  Also tried: one call at a time with the next x and weight loaded ahead (0.74
 // to 0.9 us with 128 to 512 threads: the loads share the few scoreboards, so a wait for one waits for the latest), and
 // a cluster barrier for the exchange (0.41 us: its release waits for the block's stores to global memory).
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(THREADS) fused_add_rmsnorm_run_kernel(const __
         fetch_x(0);
     }
     if constexpr (CLUSTER) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");  // every block's barriers are ready
-    bool arrived = true;
+    int gave_up = -1;  // the exchange whose wait ran out
     float s[K][VEC];
     for (int i0 = 0, exchange = 0; i0 < n; i0 += K, ++exchange) {
         const int half = exchange & 1;
@@ -166,11 +178,13 @@ __global__ void __launch_bounds__(THREADS) fused_add_rmsnorm_run_kernel(const __
         const float partial = warp_sums<K>(acc);
         float *slot = &slots[half][lane / SHARE][rank * nwarps + warp];
         if constexpr (CLUSTER) {
-            const uint32_t barrier = shared_address(&barriers[half]);
-            if (threadIdx.x == 0) expect_bytes(barrier, blocks * nwarps * K * static_cast<uint32_t>(sizeof(float)));
-            for (int p = lane % SHARE; p < blocks; p += SHARE)
-                store_counted(in_block(shared_address(slot), p), partial, in_block(barrier, p));
-            arrived = arrived && wait_counted(barrier, (exchange >> 1) & 1);
+            if (gave_up < 0) {
+                const uint32_t barrier = shared_address(&barriers[half]);
+                if (threadIdx.x == 0) expect_bytes(barrier, blocks * nwarps * K * static_cast<uint32_t>(sizeof(float)));
+                for (int p = lane % SHARE; p < blocks; p += SHARE)
+                    store_counted(in_block(shared_address(slot), p), partial, in_block(barrier, p));
+                if (!__all_sync(0xffffffffu, wait_counted(barrier, (exchange >> 1) & 1, ASTRA_RUN_WAIT_POLLS))) gave_up = exchange;
+            }
         } else {
             if (lane % SHARE == 0) *slot = partial;
             __syncthreads();
@@ -179,7 +193,7 @@ __global__ void __launch_bounds__(THREADS) fused_add_rmsnorm_run_kernel(const __
         for (int w = lane % SHARE; w < blocks * nwarps; w += SHARE) total += slots[half][lane / SHARE][w];
 #pragma unroll
         for (int off = SHARE / 2; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
-        const float rstd = arrived ? rsqrtf(fmaf(total, run.inv_H, run.eps)) : __int_as_float(0x7fc00000);
+        const float rstd = gave_up < 0 ? rsqrtf(fmaf(total, run.inv_H, run.eps)) : __int_as_float(0x7fc00000);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const float rk = __shfl_sync(0xffffffffu, rstd, k * SHARE);
@@ -194,6 +208,7 @@ __global__ void __launch_bounds__(THREADS) fused_add_rmsnorm_run_kernel(const __
     grid_launch_dependents();
     if (mine) store<UV, St::Stream>(run.r + row + at, pr);
     if constexpr (CLUSTER) {  // no block leaves while another may still store into its shared memory
+        if (gave_up >= 0) wait_counted(shared_address(&barriers[gave_up & 1]), (gave_up >> 1) & 1, kWaitPolls);
         asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
         asm volatile("barrier.cluster.wait;" ::: "memory");
     }
