@@ -12,45 +12,45 @@
 // [8192, 4099] (21.8 instead of 25.9 million warp instructions at [4096, 14336]), 34.5 -> 33.0 at [8192, 4100], 15.2 -> 14.8 at [1000, 14337], 13.4 -> 13.1 at [1024, 14336].
 #pragma once
 
+#include <type_traits>
+
 #include "vec.cuh"
 
 namespace astra {
 
-// SiLU(a) * b in binary32.  From a = -40 up directly, a / (1 + e^{-a}) * b.  Below, in the overflow-free form: with
-// t = e^{-|a|} in [0, 1], sigmoid(a) = t/(1+t).  t is formed as h*h with h = e^{-|a|/2} = 2^{-|a| * log2(e)/2}: h stays
-// a normal number down to |a| = 174, and the (non-flushing) product h*h reaches the subnormals, so a * e^{a} * b
-// is still produced where e^{a} alone is below 2^-126; beyond |a| = 174 the true result is below every representable
-// magnitude anyway.  Against 64 bits, binary32: largest relative error 5.9e-7 for |a| < 10 and 2.0e-6 above -40 (6.6e-7
-// and 2.0e-6 with the overflow-free form).  Which form an element takes depends on nothing but itself, so results
-// do not depend on how a row is cut into vectors.
+// SiLU(a) * b in binary32.  From a = -40 up directly, a / (1 + e^{-a}) * b.  Below, where e^{-a} may overflow, sigmoid(a) =
+// e^a (1 + e^a is 1 there), formed as h*h with h = e^{a/2} = 2^{a * log2(e)/2}: h stays a normal number down to a = -174,
+// and the (non-flushing) product h*h reaches the subnormals, so a * e^{a} * b is still produced where e^{a} alone is
+// below 2^-126; beyond a = -174 the true result is below every representable magnitude anyway.  Against 64 bits,
+// binary32: largest relative error 5.9e-7 for |a| < 10 and 2.0e-6 above -40 (6.6e-7 and 2.0e-6 with the overflow-free
+// form).  Which form an element takes depends on nothing but itself, so results do not depend on how a row is cut
+// into vectors.
 constexpr float kLog2e = 1.4426950408889634f, kHalfLog2e = 0.7213475204444817f, kSiluDirect = -40.0f;
 
-__device__ __forceinline__ float silu_mul_far(float a, float b) {
-    float h, d;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(a * kHalfLog2e));
-    const float t = h * h;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(1.0f + t));
-    return a * (d * t) * b;
-}
-
 __device__ __forceinline__ float silu_mul(float a, float b) {
-    if (a < kSiluDirect) return silu_mul_far(a, b);
+    const bool far = a < kSiluDirect;
     float e, d;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a * -kLog2e));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a * (far ? kHalfLog2e : -kLog2e)));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(e + 1.0f));
-    return a * d * b;
+    return a * (far ? e * e : d) * b;
 }
 
-// Two elements from -40 up, with the packed binary32 instructions of sm_100 (two multiplies or adds per issue slot); the
-// two special-function ops per element stay scalar.  Same arithmetic, element by element, as silu_mul.
-__device__ __forceinline__ float2 silu_mul2_direct(float2 a, float2 b) {
-    const float2 arg = __fmul2_rn(a, make_float2(-kLog2e, -kLog2e));
+// Two elements, with the packed binary32 instructions of sm_100 (two multiplies or adds per issue slot); the
+// two special-function ops per element stay scalar.  Same arithmetic, element by element, as silu_mul; without FAR
+// neither may be below -40.
+template <bool FAR> __device__ __forceinline__ float2 silu_mul2(float2 a, float2 b) {
+    const bool far_x = FAR && a.x < kSiluDirect, far_y = FAR && a.y < kSiluDirect;
+    const float2 arg = __fmul2_rn(a, make_float2(far_x ? kHalfLog2e : -kLog2e, far_y ? kHalfLog2e : -kLog2e));
     float2 e, d;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(arg.x));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(arg.y));
     const float2 den = __fadd2_rn(e, make_float2(1.0f, 1.0f));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d.x) : "f"(den.x));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d.y) : "f"(den.y));
+    if constexpr (FAR) {
+        const float2 t = __fmul2_rn(e, e);
+        d = make_float2(far_x ? t.x : d.x, far_y ? t.y : d.y);
+    }
     return __fmul2_rn(__fmul2_rn(a, d), b);
 }
 
@@ -73,42 +73,36 @@ template <int DT, int UV> __device__ __forceinline__ bool any_far(const Pack<UV>
     }
 }
 
-// SiLU(a) * b on whole packs.  A pack with a far element goes word by word, in a loop that moves the words along (it is
-// rarely taken, and unrolled its code cost small calls 0.05 us).
+// SiLU(a) * b on whole packs.  A warp in which any element is below -40 takes the form with the selects as a whole, so that
+// no lane waits for another's branch.  Vector by vector, in a rolled loop, such gates cost up to twice the time; loop /
+// this, us, L2-cold, bf16: 12.85 / 6.78 at [512, 14336] with 1 % of the gates at -60 (6.89 with the overflow-free form
+// throughout), 80.6 / 50.3 at [4096, 14336], 9.42 / 6.74 at [512, 14336] with all, 1.56 / 1.45 at [16, 14336] with one
+// channel, 47.6 / 32.7 at fp16 [8192, 4099] with 1 %; without such gates 6.67 / 6.66 at [512, 14336].  The operands are
+// widened within each branch: ahead of it, 32-byte vectors take 48 registers instead of 32 (6.97 us there).
 template <int DT, int UV> __device__ __forceinline__ Pack<UV> silu_mul_pack(const Pack<UV> &a, const Pack<UV> &b) {
-    constexpr int VEC = UV / Storage<DT>::UNITS, WORDS = Pack<UV>::WORDS, PER_WORD = UV == 1 ? 1 : 2 / Storage<DT>::UNITS;
-    if (VEC == 1 || any_far<DT, UV>(a)) {
-        Pack<UV> x = a, y = b, v;
-#pragma unroll 1
-        for (int i = 0; i < WORDS; ++i) {
-            Pack<PER_WORD * Storage<DT>::UNITS> xw, yw;
-            xw.w[0] = x.w[0];
-            yw.w[0] = y.w[0];
-            float fa[PER_WORD], fb[PER_WORD], fo[PER_WORD];
-            widen<DT, PER_WORD>(xw, fa);
-            widen<DT, PER_WORD>(yw, fb);
+    constexpr int VEC = UV / Storage<DT>::UNITS;
+    if constexpr (VEC == 1) {
+        float fa[VEC], fb[VEC], fo[VEC];
+        widen<DT, VEC>(a, fa);
+        widen<DT, VEC>(b, fb);
+        fo[0] = silu_mul(fa[0], fb[0]);
+        return narrow<DT, VEC>(fo);
+    } else {
+        auto each_pair = [&](auto far) {
+            float fa[VEC], fb[VEC], fo[VEC];
+            widen<DT, VEC>(a, fa);
+            widen<DT, VEC>(b, fb);
 #pragma unroll
-            for (int k = 0; k < PER_WORD; ++k) fo[k] = silu_mul(fa[k], fb[k]);
-#pragma unroll
-            for (int k = 0; k + 1 < WORDS; ++k) {
-                x.w[k] = x.w[k + 1];
-                y.w[k] = y.w[k + 1];
-                v.w[k] = v.w[k + 1];
+            for (int i = 0; i < VEC; i += 2) {
+                const float2 o = silu_mul2<decltype(far)::value>(make_float2(fa[i], fa[i + 1]), make_float2(fb[i], fb[i + 1]));
+                fo[i] = o.x;
+                fo[i + 1] = o.y;
             }
-            v.w[WORDS - 1] = narrow<DT, PER_WORD>(fo).w[0];
-        }
-        return v;
+            return narrow<DT, VEC>(fo);
+        };
+        if (__any_sync(__activemask(), any_far<DT, UV>(a))) return each_pair(std::true_type{});
+        return each_pair(std::false_type{});
     }
-    float fa[VEC], fb[VEC], fo[VEC];
-    widen<DT, VEC>(a, fa);
-    widen<DT, VEC>(b, fb);
-#pragma unroll
-    for (int i = 0; i + 1 < VEC; i += 2) {
-        const float2 o = silu_mul2_direct(make_float2(fa[i], fa[i + 1]), make_float2(fb[i], fb[i + 1]));
-        fo[i] = o.x;
-        fo[i + 1] = o.y;
-    }
-    return narrow<DT, VEC>(fo);
 }
 
 // Flat indexing: vector v of the output covers out[row, col*VEC .. col*VEC+VEC) with
