@@ -42,6 +42,13 @@ constexpr uint32_t kSiluPrefetchMaxBlocks = 1u << 14;
 // 5.87 / 5.24.  The upper end: faster at 7168 blocks, slower at 14336.
 constexpr int64_t kSiluWideMinBlocks = 960;
 constexpr int64_t kSiluWideMaxBlocks = 8192;
+// From so many bytes on, normalised rows (as the residual always) and merged values leave L2 first (St::First): most of
+// them are gone before anybody reads them.  Without / with, us: norm [6144, 4096] (50 MB) 52.6 / 55.1 with a reader and
+// 30.0 / 30.4 alone; [8192, 4096] (67 MB) 81.0 / 80.5 with a reader, 97.4 / 97.4 with a reader and other traffic; ragged
+// [8192, 4100] 41.1 / 40.6 alone, 100.4 / 100.1 with both; [16384, 4100] 79.9 / 78.9, 184.4 / 183.5; merge [5120, 32, 128] (42 MB)
+// 56.9 / 57.5 with a reader, [8192, 32, 128] 95.6 / 95.5; a chain of the three operations at 8192 tokens 174.4 / 172.0 without
+// readers, 289.6 / 291.7 with.
+constexpr int64_t kResultsBeyondL2Bytes = 56ll << 20;
 
 template <int DT, int UVEC, int UNROLL, int THREADS>
 cudaError_t launch_silu(uint16_t *out, const uint16_t *gate, const uint16_t *up, int64_t T, int64_t D,
@@ -171,13 +178,16 @@ cudaError_t launch_merge(uint16_t *v_out, float *lse_out, const uint16_t *v_a, c
     constexpr int VEC = UVEC / Storage<DT>::UNITS;
     const int64_t nvec = D / UVEC;
     const int64_t rows_per_launch = kMaxVecsPerLaunch / nvec;
+    auto kernel = merge_attn_states_lse_kernel<DT, VEC, UNROLL, THREADS>;
+    if constexpr (UVEC == 16 && THREADS == 256)
+        if (rows_total >= kResultsBeyondL2Bytes / (2 * UVEC) / nvec) kernel = merge_attn_states_lse_kernel<DT, VEC, UNROLL, THREADS, Ld::Stream, St::First>;
     for (int64_t r0 = 0; r0 < rows_total; r0 += rows_per_launch) {
         const int64_t rows = (rows_total - r0 < rows_per_launch) ? (rows_total - r0) : rows_per_launch;
         const uint32_t total = static_cast<uint32_t>(rows * nvec);
         const uint32_t tile = THREADS * UNROLL;
         const uint32_t blocks = (total + tile - 1) / tile;
         const cudaError_t err =
-            launch(merge_attn_states_lse_kernel<DT, VEC, UNROLL, THREADS>, blocks, THREADS, stream,
+            launch(kernel, blocks, THREADS, stream,
                    v_out + r0 * D, lse_out ? lse_out + r0 : nullptr, v_a + r0 * D, lse_a + r0, v_b + r0 * D,
                    lse_b + r0, total, FastDiv::make(static_cast<uint32_t>(nvec)));
         if (err != cudaSuccess) return err;
@@ -397,6 +407,8 @@ bool launch_rmsnorm_wide(const RmsnormOperands &op, const uint16_t *w, int64_t T
     const int threads = round_up((nvec + VPT - 1) / VPT, 32);
     if ((T > kWideVectorDecodeRows && T < kWideVectorRows) || threads < 64 || threads > 448) return false;
     const float inv_H = 1.0f / static_cast<float>(H);
+    auto kernel = fused_add_rmsnorm_reg_kernel<DT, VEC, VPT>;
+    if (T * nvec >= kResultsBeyondL2Bytes / (2 * UVEC)) kernel = fused_add_rmsnorm_reg_kernel<DT, VEC, VPT, Ld::Stream, St::First>;
     *err = cudaSuccess;
     for (int64_t t0 = 0; t0 < T && *err == cudaSuccess; t0 += kMaxGridX) {
         const unsigned rows = static_cast<unsigned>(T - t0 < kMaxGridX ? T - t0 : kMaxGridX);
@@ -409,7 +421,7 @@ bool launch_rmsnorm_wide(const RmsnormOperands &op, const uint16_t *w, int64_t T
             *err = launch(fused_add_rmsnorm_reg_kernel<DT, VEC, VPT, Ld::Stream, St::Stream, false, true>, rows, threads,
                           stream, o, w, H, eps, inv_H);
         else
-            *err = launch(fused_add_rmsnorm_reg_kernel<DT, VEC, VPT>, rows, threads, stream, o, w, H, eps, inv_H);
+            *err = launch(kernel, rows, threads, stream, o, w, H, eps, inv_H);
     }
     return true;
 }
@@ -425,6 +437,8 @@ template <int DT, int VPT, bool EARLY_W>
 cudaError_t launch_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, int64_t T, int H, int threads, float eps,
                                   cudaStream_t stream) {
     const float inv_H = 1.0f / static_cast<float>(H);
+    auto kernel = fused_add_rmsnorm_ragged_kernel<DT, VPT, EARLY_W>;
+    if (T >= kResultsBeyondL2Bytes / (2 * Storage<DT>::UNITS) / H) kernel = fused_add_rmsnorm_ragged_kernel<DT, VPT, EARLY_W, St::First>;
     for (int64_t t0 = 0; t0 < T; t0 += kMaxGridX) {
         const unsigned rows = static_cast<unsigned>(T - t0 < kMaxGridX ? T - t0 : kMaxGridX);
         RmsnormOperands o = op;
@@ -432,8 +446,7 @@ cudaError_t launch_rmsnorm_ragged(const RmsnormOperands &op, const uint16_t *w, 
         o.r += t0 * op.r_pitch;
         o.y += t0 * op.y_pitch;
         o.r_out += t0 * op.r_out_pitch;
-        const cudaError_t err = launch(fused_add_rmsnorm_ragged_kernel<DT, VPT, EARLY_W>, rows, threads, stream, o, w, H,
-                                       eps, inv_H);
+        const cudaError_t err = launch(kernel, rows, threads, stream, o, w, H, eps, inv_H);
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;

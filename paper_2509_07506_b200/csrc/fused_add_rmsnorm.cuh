@@ -170,7 +170,7 @@ fused_add_rmsnorm_reg_kernel(RmsnormOperands op, const uint16_t *__restrict__ we
             widen<DT, VEC>(px[i], fx);
             widen<DT, VEC>(pr[i], fr);
             add_and_square(fx, fr, s[i], acc, acc2);  // the one binary32 add per element
-            store<UV, STH>(ror + v * UV, narrow<DT, VEC>(s[i]));
+            store<UV, St::First>(ror + v * UV, narrow<DT, VEC>(s[i]));
         }
     }
 
@@ -346,7 +346,7 @@ inline RaggedShape rmsnorm_ragged_shape(int64_t T, int64_t units, bool binary32,
     return sh;
 }
 
-template <int DT, int VPT, bool EARLY_W>
+template <int DT, int VPT, bool EARLY_W, St STH = St::Stream>
 __global__ void __launch_bounds__(kRmsnormRaggedMaxThreads, VPT <= 2 ? 2 : 1)
 fused_add_rmsnorm_ragged_kernel(RmsnormOperands op, const uint16_t *__restrict__ weight, int H, float eps, float inv_H) {
     constexpr int UV = 16, UNITS = Storage<DT>::UNITS, VEC = UV / UNITS;
@@ -391,7 +391,7 @@ fused_add_rmsnorm_ragged_kernel(RmsnormOperands op, const uint16_t *__restrict__
             widen<DT, VEC>(px[i], fx);
             widen<DT, VEC>(pr[i], fr);
             add_and_square(fx, fr, s[i], acc, acc2);
-            store<UV, St::Stream>(ror + (g.first + v * UV), narrow<DT, VEC>(s[i]));
+            store<UV, St::First>(ror + (g.first + v * UV), narrow<DT, VEC>(s[i]));
         }
     }
     if (g.edge >= 0) {
@@ -399,9 +399,9 @@ fused_add_rmsnorm_ragged_kernel(RmsnormOperands op, const uint16_t *__restrict__
         widen<DT, 1>(ex, fx);
         widen<DT, 1>(er, fr);
         add_and_square(fx, fr, es, acc, acc2);
-        store<UNITS, St::Stream>(ror + g.edge, narrow<DT, 1>(es));
+        store<UNITS, St::First>(ror + g.edge, narrow<DT, 1>(es));
     }
-    auto store_y = [&](int at, const auto &v) { store<std::decay_t<decltype(v)>::UNITS_PER_PACK, St::Stream>(yr + at, v); };
+    auto store_y = [&](int at, const auto &v) { store<std::decay_t<decltype(v)>::UNITS_PER_PACK, STH>(yr + at, v); };
     ASTRA_FOR_SHIFT(g.shift, UNITS,
                     (ragged_finish<SHIFT, DT, VPT, EARLY_W>(g, weight, acc + (acc2.x + acc2.y), eps, inv_H, slots, s, es, ew,
                                                             store_y)))
@@ -469,7 +469,7 @@ fused_add_rmsnorm_cluster_kernel(RmsnormOperands op, const uint16_t *__restrict_
                 s[i][k] = fx[k] + fr[k];
                 acc = fmaf(s[i][k], s[i][k], acc);
             }
-            store<UV, St::Stream>(ror + v * UV, narrow<DT, VEC>(s[i]));
+            store<UV, St::First>(ror + v * UV, narrow<DT, VEC>(s[i]));
         }
     }
 #pragma unroll
@@ -541,7 +541,7 @@ __global__ void fused_add_rmsnorm_twopass_kernel(RmsnormOperands op,
             fs[k] = fx[k] + fr[k];
             fy[k] = fs[k] * rstd * fw[k];
         }
-        store<UV, St::Stream>(ror + v * UV, narrow<DT, VEC>(fs));
+        store<UV, St::First>(ror + v * UV, narrow<DT, VEC>(fs));
         store<UV, St::Stream>(yr + v * UV, narrow<DT, VEC>(fy));
     }
 }

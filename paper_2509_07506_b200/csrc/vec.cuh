@@ -67,7 +67,7 @@ template <> struct Storage<ASTRA_FP32> {
 // N = 1 is the scalar fallback for odd widths or 2-byte-aligned pointers of the 16-bit types.
 // ---------------------------------------------------------------------------------------------
 enum class Ld { Stream, StreamReadOnly, Keep };  // once-touched / once-touched and never written / reused (weights)
-enum class St { Stream, Default };
+enum class St { Stream, First, Default };  // a result / one that is read again only much later / kept like anything else
 
 template <int VEC> struct Pack {
     static_assert(VEC == 2 || VEC == 4 || VEC == 8 || VEC == 16, "unsupported vector width");
@@ -132,37 +132,50 @@ template <int VEC, Ld HINT> __device__ __forceinline__ Pack<VEC> load(const uint
     return v;
 }
 
-// Streamed results are the first to leave L2, which then keeps what is still to be read.  32-byte stores have to ask for it
-// by name: `.cs` does nothing for them.  Measured where a few calls' tensors just fit L2 (three sets of operands in
-// turn, sustained): rmsnorm 10.46 -> 9.56 us at fp16 [1024, 8192], 10.65 -> 9.50 at [2048, 4096], 18.8 -> 17.7 at
-// [1024, 14336], silu 5.12 -> 4.41 at [400, 14336], merge 6.31 -> 6.08 at [1536, 32, 128]; level L2-cold.
+// St::First: the first to leave L2, which then keeps what is read sooner; for the residual of a norm, whose next reader
+// comes a layer's matrix products later.  32-byte stores have to ask for it by name, `.cs` does nothing for them.
+// What the next operation reads (normalised rows and merged values below kResultsBeyondL2Bytes, activations, all
+// destinations of the all-reduce forms) does not get it: the hint then costs more than it gives.  us a call, bf16, with 32-byte stores `.cs` / all of
+// them evict-first / the residual's alone.  A norm whose rows are copied in and read back afterwards, then 96 MB
+// of other traffic: 30.4 / 30.7 / 30.5 at [1024, 4096], 39.5 / 40.1 / 39.6 at [1024, 8192], 53.4 / 54.3 / 53.4 at [4096,
+// 4096], 102.5 / 98.2 / 98.6 at [8192, 4096], 340.3 / 340.7 / 341.4 at [16384, 8192]; without that traffic, so that the
+// residual is soon read as well: 19.0 / 20.2 / 19.7 at [1024, 8192], 34.1 / 34.9 / 33.4 at [4096, 4096], 84.9 / 80.5 / 80.9 at
+// [8192, 4096].  Norms alone on three sets of operands in turn: 10.3 / 9.6 / 8.5 at [1024, 8192], 9.9 / 9.1 / 7.9 at [2048,
+// 4096]; L2-cold 11.2 / 11.2 / 11.0, 11.1 / 11.1 / 10.8, 155.4 / 155.5 / 156.2 at [16384, 8192].  `.cs` / evict-first with
+// a reader: merge 18.8 / 19.2 at [1536, 32, 128], 44.7 / 46.0 at [4096, 32, 128]; all-reduce 32.5 / 32.8 at [1024, 4096] of
+// 4, 38.8 / 41.3 at [394, 2048] of 8 to 8 destinations, 47.9 / 49.7 at [1024, 4096] of 4 to 4; that reader left out,
+// merge 6.53 / 5.92 at [1536, 32, 128] and all-reduce 7.73 / 6.30 at [394, 2048] of 8 to 8.
 template <int VEC, St HINT> __device__ __forceinline__ void store(uint16_t *p, const Pack<VEC> &v) {
     if constexpr (VEC == 1) {
         uint16_t h = static_cast<uint16_t>(v.w[0]);
-        if constexpr (HINT == St::Stream)
+        if constexpr (HINT != St::Default)
             asm volatile("st.global.cs.u16 [%0], %1;" ::"l"(p), "h"(h) : "memory");
         else
             asm volatile("st.global.u16 [%0], %1;" ::"l"(p), "h"(h) : "memory");
     } else if constexpr (VEC == 2) {
-        if constexpr (HINT == St::Stream)
+        if constexpr (HINT != St::Default)
             asm volatile("st.global.cs.u32 [%0], %1;" ::"l"(p), "r"(v.w[0]) : "memory");
         else
             asm volatile("st.global.u32 [%0], %1;" ::"l"(p), "r"(v.w[0]) : "memory");
     } else if constexpr (VEC == 4) {
-        if constexpr (HINT == St::Stream)
+        if constexpr (HINT != St::Default)
             asm volatile("st.global.cs.v2.u32 [%0], {%1,%2};" ::"l"(p), "r"(v.w[0]), "r"(v.w[1]) : "memory");
         else
             asm volatile("st.global.v2.u32 [%0], {%1,%2};" ::"l"(p), "r"(v.w[0]), "r"(v.w[1]) : "memory");
     } else if constexpr (VEC == 8) {
-        if constexpr (HINT == St::Stream)
+        if constexpr (HINT != St::Default)
             asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};"
                          ::"l"(p), "r"(v.w[0]), "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3]) : "memory");
         else
             asm volatile("st.global.v4.u32 [%0], {%1,%2,%3,%4};"
                          ::"l"(p), "r"(v.w[0]), "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3]) : "memory");
     } else {  // 32-byte access (sm_100+)
-        if constexpr (HINT == St::Stream)
+        if constexpr (HINT == St::First)
             asm volatile("st.global.L2::evict_first.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                         ::"l"(p), "r"(v.w[0]), "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3]),
+                           "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7]) : "memory");
+        else if constexpr (HINT == St::Stream)
+            asm volatile("st.global.cs.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                          ::"l"(p), "r"(v.w[0]), "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3]),
                            "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7]) : "memory");
         else
