@@ -108,7 +108,7 @@ bool runnable(const Shape &sh) {
 }
 
 // Is a launch of `count` calls the faster?  The elementwise kernels of a run keep fewer threads resident than those of
-// single calls (94 to 116 registers) and lose where a single call fills the GPU: us a call together / one by one, silu
+// single calls (96 registers silu, 104 to 116 merge) and lose where a single call fills the GPU: us a call together / one by one, silu
 // 2.05 / 3.33 at [256, 14336] but 31 / 26 for two calls at [2048, 14336]; merge 1.92 / 2.50 at [256, 64, 128] but 3.45 / 3.14
 // at [512, 64, 128].  Norms, which keep their residual, gain at every size (24 / 41 us at [8192, 4096], 8 calls).  Two or
 // three calls have too few loads in flight beyond smaller sizes (silu 5.1 / 4.1 at [256, 14336], merge 4.1 / 3.1 at
@@ -191,33 +191,56 @@ astra_status_t issue_together(const Shape &sh, const astra_run_call *c, int n, i
     return launch_status(err);
 }
 
-}  // namespace
+// How many of the n calls, from the first on, share a launch; vec is the width of its accesses.
+int calls_together(const Shape &sh, const astra_run_call *calls, int32_t n, int *vec) {
+    Footprint f[kMaxRun];
+    f[0] = footprint(sh, calls[0]);
+    *vec = f[0].vec;
+    int count = 1;
+    bool more = f[0].usable;
+    while (more && count < kMaxRun && count < n) {
+        f[count] = footprint(sh, calls[count]);
+        more = f[count].usable;
+        for (int k = 0; more && k < count; ++k) more = together(sh, f[k], f[count]);
+        count += more;
+    }
+    return worth(sh, count) ? count : 1;
+}
 
-extern "C" astra_status_t astra_issue_run(int kind, int32_t n, const astra_run_call *calls, const int64_t *ext, float eps,
-                                          astra_dtype_t dtype, void *cuda_stream) {
+// The calls of each launch, in order, to issue(first call, count, vec); stops at what is not ASTRA_OK.
+template <typename ISSUE>
+astra_status_t for_each_launch(int kind, int32_t n, const astra_run_call *calls, const int64_t *ext, float eps, astra_dtype_t dtype,
+                               ISSUE issue) {
     if ((kind != KIND_RMSNORM && kind != KIND_SILU && kind != KIND_MERGE) || n < 0) return ASTRA_ERR_BAD_SHAPE;
     if (n == 0) return ASTRA_OK;
     if (!calls || !ext) return ASTRA_ERR_NULL_POINTER;
     const Shape sh = {kind, {ext[0], ext[1], kind == KIND_MERGE ? ext[2] : 0}, eps, dtype};
     const bool may_run = runnable(sh);
-    Footprint f[kMaxRun];
     for (int32_t i = 0; i < n;) {
-        int count = 1;  // calls [i, i + count) share a launch
-        if (may_run) {
-            f[0] = footprint(sh, calls[i]);
-            bool more = f[0].usable;
-            while (more && count < kMaxRun && i + count < n) {
-                f[count] = footprint(sh, calls[i + count]);
-                more = f[count].usable;
-                for (int k = 0; more && k < count; ++k) more = together(sh, f[k], f[count]);
-                count += more;
-            }
-            if (!worth(sh, count)) count = 1;
-        }
-        const astra_status_t st = count > 1 ? issue_together(sh, calls + i, count, f[0].vec, static_cast<cudaStream_t>(cuda_stream))
-                                            : issue_one(sh, calls[i], cuda_stream);
+        int vec = 0;
+        const int count = may_run ? calls_together(sh, calls + i, n - i, &vec) : 1;
+        const astra_status_t st = issue(sh, calls + i, count, vec);
         if (st != ASTRA_OK) return st;
         i += count;
     }
     return ASTRA_OK;
+}
+
+}  // namespace
+
+extern "C" astra_status_t astra_issue_run(int kind, int32_t n, const astra_run_call *calls, const int64_t *ext, float eps,
+                                          astra_dtype_t dtype, void *cuda_stream) {
+    return for_each_launch(kind, n, calls, ext, eps, dtype, [&](const Shape &sh, const astra_run_call *c, int count, int vec) {
+        return count > 1 ? issue_together(sh, c, count, vec, static_cast<cudaStream_t>(cuda_stream)) : issue_one(sh, *c, cuda_stream);
+    });
+}
+
+extern "C" astra_status_t astra_plan_run(int kind, int32_t n, const astra_run_call *calls, const int64_t *ext, astra_dtype_t dtype,
+                                         int32_t *counts, int32_t *launches) {
+    if (!counts || !launches) return ASTRA_ERR_NULL_POINTER;
+    *launches = 0;
+    return for_each_launch(kind, n, calls, ext, 0.0f, dtype, [&](const Shape &, const astra_run_call *, int count, int) {
+        counts[(*launches)++] = count;
+        return ASTRA_OK;
+    });
 }

@@ -25,6 +25,13 @@ typedef struct {
 astra_status_t astra_issue_run(int kind, int32_t n, const astra_run_call *calls, const int64_t *ext, float eps,
                                astra_dtype_t dtype, void *cuda_stream);
 
+/*
+ * The launches that astra_issue_run would make of these calls: their number, and how many calls each of them takes, in
+ * order (room for n).  Nothing is launched, and no address is followed.
+ */
+astra_status_t astra_plan_run(int kind, int32_t n, const astra_run_call *calls, const int64_t *ext, astra_dtype_t dtype,
+                              int32_t *counts, int32_t *launches);
+
 #ifdef __cplusplus
 }
 #endif
