@@ -37,9 +37,13 @@ const char kBuildId[] = "astra-build-id:" ASTRA_BUILD_ID;
 constexpr uint32_t kSiluPrefetchMaxBlocks = 1u << 14;
 // Range of grid sizes (in 256-thread blocks of one 32-byte vector per thread) in which the 32-byte
 // form is used.  Up to 960 blocks the grid is less than one wave of eight blocks per SM, which the next kernel's early
-// blocks then fill unevenly; 16-byte form / 32-byte form, us, with operands in L2: 2.53 / 3.44 at 672 blocks
-// ([192, 14336]), 3.05 / 3.39 at 896, 3.46 / 3.53 at 1050, 4.28 / 4.25 at 1400; L2-cold: 3.16 / 3.54, 4.19 / 3.93, 4.68 / 4.22,
-// 5.87 / 5.24.  The upper end: faster at 7168 blocks, slower at 14336.
+// blocks then fill unevenly.  16-byte form / 32-byte form, us, bf16, width 14336.  Between a copy that writes the input and one
+// that reads the result 9.97 / 10.19 at 644 blocks, 11.15 / 11.33 at 784, 11.87 / 12.06 at 896, 13.6 / 13.8 at 1120, 20.0 / 19.9
+// at 1792, 30.9 / 30.5 at 2688; between the two matrix products of an MLP 79.3 / 79.6 at 644, 93.1 / 93.3 at 896; three sets
+// of operands in turn 2.54 / 3.46 at 644, 3.77 / 4.41 at 896, 3.7 / 4.2 at 1120, 6.4 / 7.1 at 1792, 11.2 / 10.6 at 2688; a stream
+// of calls whose operands are all cold 3.21 / 3.43 at 644, 4.35 / 4.12 at 896 (fp32 4.12 / 3.85), 5.0 / 4.8 at 1120, 7.45 / 7.15
+// at 1792.  So below the line only such a stream would gain, from about 870 blocks on; the input comes from a matrix product
+// that has just written it.  The upper end: faster at 7168 blocks, slower at 14336.
 constexpr int64_t kSiluWideMinBlocks = 960;
 constexpr int64_t kSiluWideMaxBlocks = 8192;
 // From so many bytes on, normalised rows (as the residual always) and merged values leave L2 first (St::First): most of
@@ -114,8 +118,8 @@ cudaError_t dispatch_silu(uint16_t *out, const uint16_t *gate, const uint16_t *u
     // keeps the block scheduler ahead, which gives the shortest drain at the end of the grid.
     // Between one and ten waves of blocks, one 32-byte vector per thread (half as many blocks, each still prefetching its
     // share ahead of the dependency wait) is faster where everything is 32-byte aligned: see kSiluWideMinBlocks, and
-    // 13.2 -> 12.6 us at [1024, 14336], 25.2 -> 24.8 us at [2048, 14336] (L2-cold, bf16); it is slower below that and above
-    // it (98.3 -> 99.9 us at [8192, 14336]).
+    // 13.2 -> 12.6 us at [1024, 14336], 25.2 -> 24.8 us at [2048, 14336] (L2-cold, bf16); it is slower below that
+    // unless every operand is cold, and above it (98.3 -> 99.9 us at [8192, 14336]).
     if (vec == 16) {
         const int64_t blocks_wide = (T * (D / 16) + 255) / 256;
         if (blocks_wide >= kSiluWideMinBlocks && blocks_wide <= kSiluWideMaxBlocks)
