@@ -39,7 +39,11 @@ struct RmsnormRun {
 // Spreading a row pays while SMs would be idle: one SM moves a row's 24 KB per call (x, weight, y at H = 4096) at 52
 // GB/s.  64 calls in one launch, from a graph, us, with 1 / 2 / 4 / 8 blocks per row: 43 / 24.6 / 22.6 / 26.6 at
 // [16, 4096], 45 / 24.8 / 28.7 / 32.8 at [64, 4096], 59 / 47 / 28.7 / 34 at [16, 8192]; one
-// by one (beside as many merges and activations) 99, 131 and 120.
+// by one 86, 115 and 113.
+// Rows of up to 8192 units (16-bit elements; half as many of binary32); wider ones, and widths that are not whole
+// vectors, have no form and are launched one by one.  Rows of fewer vectors than a cluster has threads leave some of its
+// blocks without any.
+constexpr int64_t kSms = 148;
 struct NormRunShape {
     int blocks = 0, threads = 0, uvec = 0;
 };
@@ -49,8 +53,8 @@ inline NormRunShape norm_run_shape(int64_t T, int64_t units, int vec) {
     };
     auto shape = [&](int uvec, int blocks) { return NormRunShape{blocks, static_cast<int>(threads_for(uvec, blocks)), uvec}; };
     if (vec < 8 || units % vec != 0) return {};
-    if (T <= 37 && threads_for(8, 4) <= 256) return shape(8, 4);
-    if (T <= 74 && threads_for(8, 2) <= 256) return shape(8, 2);
+    if (T <= kSms / 4 && threads_for(8, 4) <= 256) return shape(8, 4);
+    if (T <= kSms / 2 && threads_for(8, 2) <= 256) return shape(8, 2);
     if (threads_for(8, 1) <= 512) return shape(8, 1);
     if (vec == 16 && threads_for(16, 1) <= 512) return shape(16, 1);
     return {};
@@ -115,7 +119,7 @@ __device__ __forceinline__ bool wait_counted(uint32_t barrier, uint32_t phase, i
 // must not be); the other warps of the row, which then lack its sums, run out at the next exchange and do the same.
 // Nobody reads sums of two exchanges that way, and the residual, which needs no sums, is as it should be.  Before it
 // leaves, such a warp waits once more, up to the full limit, for the stores that it gave up on.
-// 1.45 -> 0.35 us per call at [16, 4096].  Also tried: one call at a time with the next x and weight loaded ahead (0.74
+// 1.34 -> 0.35 us per call at [16, 4096].  Also tried: one call at a time with the next x and weight loaded ahead (0.74
 // to 0.9 us with 128 to 512 threads: the loads share the few scoreboards, so a wait for one waits for the latest), and
 // a cluster barrier for the exchange (0.41 us: its release waits for the block's stores to global memory).
 template <int DT, int VEC, int K, int THREADS, bool CLUSTER>

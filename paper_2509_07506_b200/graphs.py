@@ -22,8 +22,9 @@ from .binding import PreparedCall
 # of a dependent sequence is a chain of latencies (launch, first bytes, reduction, completion) that leaves
 # most of the GPU idle while it waits; a second sequence fills that time.  Measured on norm, merge, norm, activation
 # repeated 32 times where only the norms share a tensor (one residual), per repetition with 1 / 2 / 4 branches, the latter
-# two with like calls in one launch: 4.17 / 0.71 / 0.77 us at 1 token of width 4096, 4.68 / 0.77 / 0.77 at 16, 9.56 / 4.43 /
-# 4.63 at 256, 13.7 / 10.1 / 10.1 at 512, 26.6 / 19.2 / 19.6 at 1024 and 212 / 176 / 176 at 8192 tokens.  Calls that are linked through their tensors, as a decoder layer's are, stay one sequence and gain nothing.
+# two with like calls in one launch: 4.70 / 0.71 / 0.77 us at 1 token of width 4096, 4.93 / 0.77 / 0.77 at 16, 6.40 / 1.60 /
+# 1.58 at 64, 9.53 / 4.22 / 4.37 at 256, 13.2 / 9.7 / 9.7 at 512 and 26.2 / 18.0 / 20.5 at 1024 tokens.  Calls that are linked
+# through their tensors, as a decoder layer's are, stay one sequence and gain nothing.
 MAX_BRANCHES = 2
 
 
